@@ -98,7 +98,11 @@ typedef struct {
     int max_sweeps;    /* outer sweep limit; 0 = 40                                        */
     double tol;        /* pair rotates iff |g_ij| >= tol sqrt(g_ii g_jj) (Alg. 1, Alg. 2);
                           0 = 30 u, u the unit roundoff of the type (Sec. 5.4, k = 30)      */
-    int inner_sweeps;  /* inner eigensolver sweeps per Gram block; 0 = 1 (Design-2, Sec. 5) */
+    int inner_sweeps;  /* inner eigensolver sweeps per Gram block (Design-2, Sec. 5).  0 = one,
+                          over all index pairs in a sweep's first round and the pairs between
+                          the two blocks in the others (block widths of at least 16; see
+                          cross_only in csrc/jacobi_common.cuh); >= 1: over all index pairs in
+                          every round                                                       */
     int path;          /* bsvd_path                                                         */
     int flags;         /* bit 0: skip the final orthogonality correction of V;
                           bit 1: two-stage vector update (Design-3 off; multi-kernel path);

@@ -116,7 +116,10 @@ bool resolve(const bsvd_opts* o, bool single, int N, Resolved& r) {
     r.max_sweeps = o->max_sweeps ? o->max_sweeps : kDefaultMaxSweeps;
     r.max_sweeps = std::min(r.max_sweeps, bsvd::kMaxSweeps);
     r.path = o->path;
-    r.inner_sweeps = o->inner_sweeps ? o->inner_sweeps : (r.path == BSVD_PATH_PLAIN ? 30 : 1);
+    // 0 in the kernels: one inner sweep, over the cross pairs only outside an
+    // outer sweep's first round (not on the comparison paths: PLAIN and the
+    // unfused or unmasked multi-kernel variants)
+    r.inner_sweeps = o->inner_sweeps ? o->inner_sweeps : (r.path == BSVD_PATH_PLAIN ? 30 : (o->flags & 6) ? 1 : 0);
     r.tol = o->tol > 0 ? o->tol : 30.0 * (single ? kU32 : kU64);
     r.flags = o->flags;
     r.prec = o->prec;
@@ -276,7 +279,7 @@ bsvd_status plan_mixed(int max_smem, char t, int m, int n, int batch, bool wantU
     // FP32 sweeps: FMA tiles / FP64 rotations, and how the sweep loop runs
     // (no graph, host checks, host-replayed graph), as the caller asked
     mp.r32.flags = r.flags & (128 | 256 | 8 | 16 | 2048 | 4096);
-    mp.r32.inner_sweeps = 1;
+    mp.r32.inner_sweeps = r.inner_sweeps ? 1 : 0;
     mp.r32.prec = BSVD_PREC_NATIVE;
     mp.r64 = r;
     mp.r64.prec = BSVD_PREC_NATIVE;

@@ -46,6 +46,12 @@ __device__ __forceinline__ bool blk_pair(const BlkShape& s, int r, int q, int& b
     return bj < s.l;
 }
 
+// whether round r's pair step of (bi, bj) takes the cross pairs only
+template <class T, int NB>
+__device__ __forceinline__ bool blk_cross(const BlockedArgs& a, const BlkShape& s, int r, int bi, int bj) {
+    return NB >= 16 && cross_only<T>(a.inner_sweeps, s.l, r, bi, bj);
+}
+
 // skip this matrix? (bad input always; converged ones only with masks)
 __device__ __forceinline__ bool blk_skip(const BlockedArgs& a, int b) {
     const int st = a.state[4 * b];
@@ -415,8 +421,8 @@ __global__ void __launch_bounds__(GT) blk_heevj(const BlockedArgs a, int r) {
         G[j + i * LDG] = conj_s(g);
     }
     __syncthreads();
-    const int seen = inner_jacobi<T, NB, GT>(G, J, tb, (Real<T>)a.tol, a.inner_sweeps, tid, 1, NoBackground(),
-                                             nullptr, (a.flags & 256) != 0);
+    const int seen = inner_jacobi<T, NB, GT>(G, J, tb, (Real<T>)a.tol, max(a.inner_sweeps, 1), tid, 1, NoBackground(),
+                                             nullptr, (a.flags & 256) != 0, blk_cross<T, NB>(a, sh, r, bi, bj));
     T* Jg = static_cast<T*>(a.J) + sh.oJ + (long long)q * TWO * TWO;
     for (int e = tid; e < TWO * TWO; e += GT) Jg[(e % TWO) + (e / TWO) * TWO] = J[(e % TWO) + (e / TWO) * LDG];
     if (tid == 0) {

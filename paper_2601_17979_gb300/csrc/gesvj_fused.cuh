@@ -351,10 +351,12 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
                 // S3: inner Jacobi sweeps on G (round-robin over the 2nb indices)
                 int seen;
                 stepped = true;
+                const bool cross = NB >= 16 && cross_only<T>(a.inner_sweeps, a.l, r, bi, bj);
+                const int isw = a.inner_sweeps > 0 ? a.inner_sweeps : 1;
                 if constexpr (kDefer) {
                     int ns = 0;
-                    seen = inner_jacobi<T, NB, GT>(G, J, tb, tol, a.inner_sweeps, gt, g + 1, dv, &ns,
-                                                   (a.flags & kFlagWideAngles) != 0);
+                    seen = inner_jacobi<T, NB, GT>(G, J, tb, tol, isw, gt, g + 1, dv, &ns,
+                                                   (a.flags & kFlagWideAngles) != 0, cross);
                     if (dv.J) {   // the deferred V rows the background warps did not reach
                         for (int wt = ns * inner_background_warps<GT>() + (gt >> 5); wt < dv.tasks(); wt += GT / 32)
                             dv(wt);
@@ -362,8 +364,8 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
                     }
                     group_sync(g, GT);
                 } else {
-                    seen = inner_jacobi<T, NB, GT>(G, J, tb, tol, a.inner_sweeps, gt, g + 1, NoBackground(), nullptr,
-                                                   (a.flags & kFlagWideAngles) != 0);
+                    seen = inner_jacobi<T, NB, GT>(G, J, tb, tol, isw, gt, g + 1, NoBackground(), nullptr,
+                                                   (a.flags & kFlagWideAngles) != 0, cross);
                 }
                 if (seen == 0) break;                       // J = I: pair masked (Design-4)
                 if (gt == 0) swflag[sw] = 1;

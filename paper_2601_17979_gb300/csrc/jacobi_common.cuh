@@ -59,6 +59,17 @@ __device__ __forceinline__ void named_sync(int id, int nthreads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 
+// Named barrier over `nthreads` threads that also ORs their predicates.
+__device__ __forceinline__ bool named_sync_or(int id, int nthreads, bool x) {
+    int any;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.s32 q, %3, 0;\n\tbar.red.or.pred p, %1, %2, q;\n\tselp.s32 %0, 1, 0, p;\n\t}"
+        : "=r"(any)
+        : "r"(id), "r"(nthreads), "r"((int)x)
+        : "memory");
+    return any != 0;
+}
+
 template <class R> __device__ __forceinline__ R warp_max(R v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
@@ -248,6 +259,53 @@ __device__ __forceinline__ void diagonal_block(T* G, int p, int q, Real<T> gpp, 
     G[q + p * LDG] = make_s<T>(0);
 }
 
+// The pair test |g_pq| >= tol sqrt(g_pp) sqrt(g_qq) (Alg. 1), compared in
+// squares while the product stays well inside the normal range; the sign and
+// range tests on the bit patterns (a NaN operand still fails the comparison).
+template <class R>
+__device__ __forceinline__ bool pair_fires(R gpp, R gqq, R apq, R tol) {
+    const R prod = rmul(gpp, gqq);
+    const bool pos = (as_ord(gpp) > 0) & (as_ord(gqq) > 0) & (as_ord(apq) > 0);
+    return pos && (as_ord(prod) > as_ord(kJacobiProdMin<R>)
+                       ? rmul(apq, apq) >= rmul(rmul(tol, tol), prod)
+                       : apq >= rmul(rmul(tol, sqrt_r(gpp)), sqrt_r(gqq)));
+}
+// The same in FP64 on widened single-precision entries (their squares stay
+// inside FP64's range).
+__device__ __forceinline__ bool pair_fires_wide(double gpp, double gqq, double apq, double tol) {
+    return gpp > 0 && gqq > 0 && apq > 0 && apq * apq >= (tol * tol) * (gpp * gqq);
+}
+
+// Whether the test fires for entry (p, q) of G.
+template <class T, int LDG>
+__device__ __forceinline__ bool entry_fires(const T* G, int p, int q, Real<T> tol, bool wide) {
+    if constexpr (!std::is_same<T, typename WideOf<T>::type>::value)
+        if (wide)
+            return pair_fires_wide((double)re(G[p + p * LDG]), (double)re(G[q + q * LDG]),
+                                   abs_rot(to_wide(G[p + q * LDG])), (double)tol);
+    return pair_fires<Real<T>>(re(G[p + p * LDG]), re(G[q + q * LDG]), abs_rot(G[p + q * LDG]), tol);
+}
+
+// Whether a pair step takes all index pairs of its Gram block or only the
+// cross pairs (p in block i, q in block j).  An outer sweep needs each index
+// pair once: the first round's blocks cover the pairs inside every block
+// (with an odd block count l the last block sits out round 0 and catches up
+// in round 1), so the other rounds sweep the nb^2 cross pairs in nb steps
+// instead of all (2nb - 1) nb pairs in 2nb - 1 steps.  A caller that sets
+// inner_sweeps gets full sweeps everywhere.  Single precision keeps full
+// sweeps above 20 blocks: there the many FP32 updates' own roundings set the
+// singular values' last digits, and the shorter sweeps (which leave S closer
+// to the exact values: 4.9e-5 against 6.9e-5 relative on 512 x 512) would
+// move them by more than FP32 results may move between versions (2e-5).
+// Complex128 keeps them up to 4 blocks (75 x 50: 47.9 ms against 50.1).
+// Sweeps on 256 x 256 FP32: 11.3 full, 11.6 with cross pairs, half the steps.
+template <class T>
+__device__ __forceinline__ bool cross_only(int inner_sweeps, int l, int r, int bi, int bj) {
+    constexpr bool kSingle = sizeof(Real<T>) == 4, kC128 = sizeof(T) == 16;
+    return inner_sweeps == 0 && r > 0 && (!kSingle || l <= 20) && (!kC128 || l > 4) &&
+           !((l & 1) && r == 1 && (bi == l - 1 || bj == l - 1));
+}
+
 // The rotation of inner_rotation with the pair test and Eq. (sin-cos)
 // evaluated in FP64 on the single-precision Gram entries (exactly widened),
 // c, t and e s rounded once to the working precision at the end.
@@ -260,9 +318,8 @@ __device__ __forceinline__ int inner_rotation_wide(T* G, Real<T> tol, int p, int
     constexpr int LDG = 2 * NB + 1;
     const RW gpp = (RW)re(G[p + p * LDG]), gqq = (RW)re(G[q + q * LDG]);
     const TW gpq = to_wide(G[p + q * LDG]);
-    const RW apq = abs_rot(gpq), tw = (RW)tol;
-    // squares of widened single-precision values stay inside FP64's range
-    const bool fire = gpp > 0 && gqq > 0 && apq > 0 && apq * apq >= (tw * tw) * (gpp * gqq);
+    const RW apq = abs_rot(gpq);
+    const bool fire = pair_fires_wide(gpp, gqq, apq, (RW)tol);
     RW c = 1, t = 0;
     TW es = make_s<TW>(0);
     if (fire) {
@@ -294,14 +351,7 @@ __device__ __forceinline__ int inner_rotation(T* G, Real<T> tol, int p, int q, i
     const R gpp = re(G[p + p * LDG]), gqq = re(G[q + q * LDG]);
     const T gpq = G[p + q * LDG];
     const R apq = abs_rot(gpq);
-    // |g_pq| >= tol sqrt(g_pp) sqrt(g_qq), compared in squares while the
-    // product stays well inside the normal range; the sign and range tests
-    // on the bit patterns (a NaN operand still fails the comparison)
-    const R prod = rmul(gpp, gqq);
-    const bool pos = (as_ord(gpp) > 0) & (as_ord(gqq) > 0) & (as_ord(apq) > 0);
-    const bool fire = pos && (as_ord(prod) > as_ord(kJacobiProdMin<R>)
-                                  ? rmul(apq, apq) >= rmul(rmul(tol, tol), prod)
-                                  : apq >= rmul(rmul(tol, sqrt_r(gpp)), sqrt_r(gqq)));
+    const bool fire = pair_fires<R>(gpp, gqq, apq, tol);
     R c = 1, t = 0;
     T es = make_s<T>(0);
     if (fire) {
@@ -332,6 +382,15 @@ __device__ __forceinline__ int inner_rotation(T* G, Real<T> tol, int p, int q, i
 // gt) sharing named barrier `bar`; the caller must have finished writing G and
 // synchronised.  Returns the number of rotations fired (0: G was diagonal to
 // tol); uniform over the group.
+//
+// `cross`: only the pairs (p in the first block, q in the second), in NB steps
+// of NB disjoint rotations, slot s of step k taking (s, NB + (s + k) % NB);
+// one sweep.
+//
+// All entries are tested at once before the first step: a block in which no
+// pair fires would run its steps without changing G, so it returns at once
+// (a converged block, and the last sweep of every matrix, cost one test
+// instead of 2NB - 1 steps of two barriers).
 // Work the caller hands the J-update warps: called once per step by each of
 // them, with a running per-warp task index (step * background warps + warp).
 struct NoBackground {
@@ -342,9 +401,11 @@ __host__ __device__ constexpr int inner_background_warps() { return GT > 32 ? GT
 
 template <class T, int NB, int GT, class Bg = NoBackground>
 __device__ int inner_jacobi(T* G, T* J, const InnerTables<T, NB>& tb, Real<T> tol, int sweeps,
-                            int gt, int bar, const Bg& bg = Bg(), int* nsteps = nullptr, bool wide = false) {
+                            int gt, int bar, const Bg& bg = Bg(), int* nsteps = nullptr, bool wide = false,
+                            bool cross = false) {
     using R = Real<T>;
-    constexpr int TWO = 2 * NB, LDG = TWO + 1, STEPS = TWO - 1;
+    constexpr int TWO = 2 * NB, LDG = TWO + 1;
+    const int STEPS = cross ? NB : TWO - 1;
     // The off-diagonal 2x2 blocks of G by slot pair (two rotations each);
     // the diagonal ones (the closed form) are applied by the lane of warp 0
     // that forms their rotation, right after forming it.
@@ -368,9 +429,13 @@ __device__ int inner_jacobi(T* G, T* J, const InnerTables<T, NB>& tb, Real<T> to
             bq1[u] = -1; bq2[u] = -1;
         }
     }
-    for (int e = gt; e < TWO * TWO; e += GT)
-        J[(e % TWO) + (e / TWO) * LDG] = make_s<T>((e % TWO) == (e / TWO) ? 1 : 0);
-    named_sync(bar, GT);
+    bool any = false;
+    for (int e = gt; e < TWO * TWO; e += GT) {
+        const int i = e % TWO, j = e / TWO;
+        J[i + j * LDG] = make_s<T>(i == j ? 1 : 0);
+        if (i < j && (!cross || (i < NB && j >= NB))) any |= entry_fires<T, LDG>(G, i, j, tol, wide);
+    }
+    if (!named_sync_or(bar, GT, any)) return 0;
     // warp 0 forms the rotations, lane `slot` those of one slot, following
     // its pair through the steps (the next step's pair is found during the
     // block transforms, where warp 0 is not the last to finish); one ballot
@@ -379,7 +444,8 @@ __device__ int inner_jacobi(T* G, T* J, const InnerTables<T, NB>& tb, Real<T> to
     RRSlot rs(TWO, gt < NB ? gt : 0);
     int np = 0, nq = 0, fired_sweep = 0;
     if (gt < 32) {
-        rs.pair(np, nq);
+        if (cross) { np = gt; nq = NB + gt; }
+        else rs.pair(np, nq);
         const int f = gt < NB ? inner_rotation<T, NB>(G, tol, np, nq, gt, tb.step(0), wide) : 0;
         fired_sweep = __popc(__ballot_sync(0xffffffffu, f));
     }
@@ -443,8 +509,12 @@ __device__ int inner_jacobi(T* G, T* J, const InnerTables<T, NB>& tb, Real<T> to
                 }
             }
             if (gt < 32) {
-                rs.next();                    // step st + 1, or step 0 of the next sweep (2NB - 1 = 0 mod the ring)
-                rs.pair(np, nq);
+                if (cross) {
+                    nq = nq == TWO - 1 ? NB : nq + 1;
+                } else {
+                    rs.next();                // step st + 1, or step 0 of the next sweep (2NB - 1 = 0 mod the ring)
+                    rs.pair(np, nq);
+                }
             }
             named_sync(bar, GT);
             // warp 0: the rotations of the next step (this sweep, or the first
