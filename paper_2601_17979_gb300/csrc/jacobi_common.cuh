@@ -228,6 +228,7 @@ __device__ __forceinline__ double phase_times(double g, double, double s) {
     return __longlong_as_double(__double_as_longlong(s) ^ (__double_as_longlong(g) & (long long)0x8000000000000000ull));
 }
 __device__ __forceinline__ float2 phase_times(float2 g, float a, float s) {
+    if (a < 1e-37f) return make_float2(g.x / a * s, g.y / a * s);   // 1 / a would overflow
     const float k = s * (1.0f / a);
     return make_float2(g.x * k, g.y * k);
 }
