@@ -46,10 +46,11 @@ __device__ __forceinline__ bool blk_pair(const BlkShape& s, int r, int q, int& b
     return bj < s.l;
 }
 
-// whether round r's pair step of (bi, bj) takes the cross pairs only
+// whether round r's pair step of (bi, bj) takes the cross pairs only (not from
+// a given V, close to convergence: full sweeps save an outer one there)
 template <class T, int NB>
 __device__ __forceinline__ bool blk_cross(const BlockedArgs& a, const BlkShape& s, int r, int bi, int bj) {
-    return NB >= 16 && cross_only<T>(a.inner_sweeps, s.l, r, bi, bj);
+    return NB >= 16 && !a.V0 && cross_only<T>(a.inner_sweeps, s.l, r, bi, bj);
 }
 
 // skip this matrix? (bad input always; converged ones only with masks)

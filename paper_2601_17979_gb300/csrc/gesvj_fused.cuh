@@ -22,6 +22,7 @@
 
 #include "fused_f32.cuh"
 #include "jacobi_common.cuh"
+#include "precondition.cuh"
 #include "tc_f32.cuh"
 
 namespace bsvd {
@@ -133,6 +134,38 @@ struct DeferredV {
     }
 };
 
+// Scratch of the preconditioner in a group's bytes (real FP32: also the two
+// column buffers of apply_q).
+template <class T>
+__device__ __forceinline__ long long pre_bytes(int M, int N) {
+    if constexpr (std::is_same<T, float>::value) return max(PreF32::bytes(M, N), 4LL * kQPanel * PreF32::f32_buf(M));
+    else                                         return PreScratch<T>::bytes(N);
+}
+
+// Whether the sweeps start from the preconditioned matrix (precondition.cuh):
+// a rule on the shape; a flat spectrum may still decline.  Measured against
+// the sweeps without it (ms, batches of 500 to 5,000):
+//   nb = 16: FP64 128 x 64, kappa 1e6, 4,000: 317 -> 99; FP32 128 x 64, kappa
+//   1e3, 3,000: 12.0 -> 7.1; complex64 64 x 64, kappa 1e3, 2,000: 18.0 -> 12.0;
+//   nb = 8 (below 48 columns, the AUTO rule's width): FP64 20 x 20 5.55 -> 5.24,
+//   complex128 40 x 40 17.8 -> 15.8, complex64 97 x 45 13.5 -> 12.5; but FP32
+//   32 x 32 2.3 -> 2.4 and complex64 32 x 32 4.2 -> 4.6;
+//   one pair of blocks (at most 2 nb columns): complex128 24 x 16 1.48 -> 1.76,
+//   FP32 100 x 16 0.85 -> 1.1, worth it only for the rows QR takes off tall
+//   FP64 (1000 x 16, 1,000: 13.1 -> 11.0).
+// Single precision up to 160 columns (on chip about 128): beyond, on global
+// slots, it would move FP32 results as noted at cross_only.  A caller that sets
+// inner_sweeps gets the sweeps of the plain method from the start, and a start
+// from a given V (the mixed-precision polish) comes preconditioned already.
+template <class T, int NB>
+__device__ __forceinline__ bool preconditioned(const FusedArgs& a) {
+    constexpr bool kSingle = sizeof(Real<T>) == 4, kReal32 = std::is_same<T, float>::value;
+    if (a.inner_sweeps != 0 || a.V0 || NB < 8 || pre_bytes<T>(a.M, a.N) > a.groupBytes) return false;
+    if (a.l == 2 && (kSingle || a.M < 8 * a.N)) return false;
+    if (kSingle && a.N > 160) return false;
+    return NB == 16 || (!kReal32 && a.N < 48 && (!kSingle || a.N > 32));
+}
+
 // Real FP32 keeps two CTAs per SM (its shared memory allows them).
 template <class T>
 constexpr int fused_min_blocks() { return std::is_same<T, float>::value ? 2 : 1; }
@@ -149,7 +182,8 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
     constexpr int TWO = 2 * NB, LDG = TWO + 1, NT = NG * GT, NW = NT / 32;
 
     const int tid = threadIdx.x, g = tid / GT, gt = tid % GT, lane = tid & 31, warp = tid >> 5;
-    const int M = a.M, N = a.N, ldw = a.ldw, ldvs = a.ldvs;
+    const int M0 = a.M, N = a.N, ldw = a.ldw, ldvs = a.ldvs;
+    int M = M0;                                        // rows the sweeps work on: N once preconditioned
     const bool needVs = a.trans ? a.wantU : a.wantV;   // V is part of the output
     const bool wantWout = a.trans ? a.wantV : a.wantU; // W / sigma is part of the output
 
@@ -243,6 +277,21 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
             *p = scalb_s(*p, -ex);
         }
     __syncthreads();
+
+    // ---- W P = Q [L; 0] (P Z)^H: sweep L with V from P Z, Q kept in the output --
+    T* const Y = a.trans ? Vout : Uout;                        // W / sigma; M0 x N
+    T* const Z = a.trans ? Uout : Vout;                        // V; N x N
+    const long long ldy = a.trans ? ldv : ldu, ldz = a.trans ? ldu : ldv;
+    bool pre = false;
+    if (preconditioned<T, NB>(a)) {
+        if constexpr (std::is_same<T, float>::value)
+            pre = precondition_f32<NT>(W, ldw, M0, N, needVs ? Vs : nullptr, ldvs, wantWout ? Y : nullptr, ldy,
+                                       PreF32(smem + a.offG, M0, N));
+        else
+            pre = precondition<T, NT>(W, ldw, M0, N, needVs ? Vs : nullptr, ldvs, nullptr, 0, wantWout ? Y : nullptr, ldy,
+                                      PreScratch<T>(smem + a.offG, N));
+        if (pre) M = N;
+    }
 
     // ---- sweeps -----------------------------------------------------------------
     const R tol = (R)a.tol;
@@ -351,7 +400,7 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
                 // S3: inner Jacobi sweeps on G (round-robin over the 2nb indices)
                 int seen;
                 stepped = true;
-                const bool cross = NB >= 16 && cross_only<T>(a.inner_sweeps, a.l, r, bi, bj);
+                const bool cross = (NB >= 16 || pre) && !a.V0 && cross_only<T>(a.inner_sweeps, a.l, r, bi, bj);
                 const int isw = a.inner_sweeps > 0 ? a.inner_sweeps : 1;
                 if constexpr (kDefer) {
                     int ns = 0;
@@ -384,7 +433,7 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
                     } else {
                         for (int e = gt; e < TWO * TWO; e += GT) Jt[(e / TWO) + (e % TWO) * TWO] = J[(e % TWO) + (e / TWO) * LDG];
                         group_sync(g, GT);
-                        update_f32_tiled<NB, GT, 2>(W, ldw, ldw, Vs, ldvs, needVs ? ldvs : 0, bi * NB, bj * NB, Jt, gt, g + 1);
+                        update_f32_tiled<NB, GT, 2>(W, ldw, pre ? (M + 3) & ~3 : ldw, Vs, ldvs, needVs ? ldvs : 0, bi * NB, bj * NB, Jt, gt, g + 1);
                     }
                 } else if constexpr (std::is_same<T, float2>::value) {
                     // complex64: 4 rows x 2nb/8 columns per lane (columns
@@ -498,15 +547,26 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
     }
 
     // ---- finalise (Alg. 2): sigma, sort, U = W Sigma^-1, V correction --------
-    {
-        T* Y = a.trans ? Vout : Uout;
-        T* Z = a.trans ? Uout : Vout;
-        const long long ldy = a.trans ? ldv : ldu, ldz = a.trans ? ldu : ldv;
-        const FinalScratch<T> fs{sig, rank, red, iscr, bcast};
+    const FinalScratch<T> fs{sig, rank, red, iscr, bcast};
+    const bool correct = !(a.flags & kFlagNoVCorrection);
+    if (!pre) {
         // W's space is free once Y is written: it holds the completion vector and V^H V - I
-        finalize_outputs<T, NT>(W, ldw, Vs, ldvs, M, N, ex, W, W, a.lde,
-                                !(a.flags & kFlagNoVCorrection), Sout, Y, ldy, wantWout, Z, ldz,
+        finalize_outputs<T, NT>(W, ldw, Vs, ldvs, M, N, ex, W, W, a.lde, correct, Sout, Y, ldy, wantWout, Z, ldz,
                                 needVs, fs);
+    } else {
+        finalize_sigma<T, NT>(W, ldw, N, N, ex, Sout, fs);
+        if (wantWout) {
+            T* const buf = reinterpret_cast<T*>(smem + a.offG);
+            normalize_columns<T, NT>(W, ldw, N, buf, fs);
+            if constexpr (std::is_same<T, float>::value) apply_q_f32<NT>(W, ldw, M0, N, Y, ldy, buf);
+            else apply_q<T, NT>(W, ldw, M0, N, Y, ldy, 2LL * M0 * (int)sizeof(T) <= a.groupBytes ? buf : nullptr);
+            for (int e = tid; e < M0 * N; e += NT) {
+                const int i = e % M0, k = e / M0;
+                Y[i + (long long)rank[k] * ldy] = W[i + k * ldw];
+            }
+            __syncthreads();
+        }
+        if (needVs) finalize_z<T, NT>(Vs, ldvs, N, W, a.lde, correct, Z, ldz, rank);
     }
     if (tid == 0) {
         a.info[mid] = converged ? 0 : sw;

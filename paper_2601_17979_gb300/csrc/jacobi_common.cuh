@@ -88,6 +88,15 @@ __device__ __forceinline__ float2 shfl_xor_s(float2 v, int o) {
 __device__ __forceinline__ double2 shfl_xor_s(double2 v, int o) {
     return make_double2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
 }
+template <class T> __device__ __forceinline__ T shfl_s(T v, int src);
+template <> __device__ __forceinline__ float shfl_s(float v, int src) { return __shfl_sync(0xffffffffu, v, src); }
+template <> __device__ __forceinline__ double shfl_s(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
+template <> __device__ __forceinline__ float2 shfl_s(float2 v, int src) {
+    return make_float2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
+}
+template <> __device__ __forceinline__ double2 shfl_s(double2 v, int src) {
+    return make_double2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
+}
 __device__ __forceinline__ float warp_sum_s(float v) { return warp_sum(v); }
 __device__ __forceinline__ double warp_sum_s(double v) { return warp_sum(v); }
 __device__ __forceinline__ float2 warp_sum_s(float2 v) { return make_float2(warp_sum(v.x), warp_sum(v.y)); }
@@ -284,7 +293,17 @@ __device__ __forceinline__ bool entry_fires(const T* G, int p, int q, Real<T> to
         if (wide)
             return pair_fires_wide((double)re(G[p + p * LDG]), (double)re(G[q + q * LDG]),
                                    abs_rot(to_wide(G[p + q * LDG])), (double)tol);
-    return pair_fires<Real<T>>(re(G[p + p * LDG]), re(G[q + q * LDG]), abs_rot(G[p + q * LDG]), tol);
+    using R = Real<T>;
+    if constexpr (Traits<T>::kComplex) {
+        // without |g_pq|'s square root: well below the bound the pair does not
+        // fire; near it, or where squares leave the safe range, the full test
+        const T g = G[p + q * LDG];
+        const R prod = rmul(re(G[p + p * LDG]), re(G[q + q * LDG])), g2 = fma_s(g.x, g.x, rmul(g.y, g.y));
+        if (as_ord(prod) > as_ord(kJacobiProdMin<R>) && as_ord(g2) > as_ord(kJacobiProdMin<R>) &&
+            rmul(g2, R(1.001)) < rmul(rmul(tol, tol), prod))
+            return false;
+    }
+    return pair_fires<R>(re(G[p + p * LDG]), re(G[q + q * LDG]), abs_rot(G[p + q * LDG]), tol);
 }
 
 // Whether a pair step takes all index pairs of its Gram block or only the
@@ -592,21 +611,11 @@ struct FinalScratch {
     Real<T>* sig; int* rank; Real<T>* red; int* iscr; T* bcast;
 };
 
-// The end of Alg. 2 for one matrix, by a whole CTA of NT threads.
-//   sigma_k = ||w_k||_2 (exact power-of-two scaled sum of squares), a stable
-//   descending sort (rank of each column), Sout[rank] = sigma * 2^ex;
-//   Y[:, rank_k] = w_k / sigma_k (U, or V for a transposed problem) when
-//   wantY, with zero columns completed to an orthonormal basis;
-//   Z[:, rank_k] = v_k - (V (V^H V - I))_k / 2 (one Newton-Schulz step
-//   towards the nearest orthonormal V) when wantZ; `correct` = false copies V.
-// W (M x N, ldw) and V (N x N, ldvs) may live in shared or global memory.
-// x (M elements) and E (N x N, lde) are scratch and may alias W: W is not
-// read after Y is complete.
+// sigma_k = ||w_k||_2 (exact power-of-two scaled sum of squares) into sig, the
+// rank of each column in a stable descending sort, Sout[rank] = sigma * 2^ex.
 template <class T, int NT>
-__device__ void finalize_outputs(const T* W, int ldw, const T* V, int ldvs, int M, int N, int ex,
-                                 T* x, T* E, int lde, bool correct, Real<T>* Sout, T* Y,
-                                 long long ldy, bool wantY, T* Z, long long ldz, bool wantZ,
-                                 const FinalScratch<T>& fs) {
+__device__ __forceinline__ void finalize_sigma(const T* W, int ldw, int M, int N, int ex, Real<T>* Sout,
+                                               const FinalScratch<T>& fs) {
     using R = Real<T>;
     constexpr int NW = NT / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -634,6 +643,61 @@ __device__ void finalize_outputs(const T* W, int ldw, const T* V, int ldvs, int 
         Sout[rk] = scalb_r(sk, ex);
     }
     __syncthreads();
+}
+
+// Z[:, rank_k] = v_k - (V (V^H V - I))_k / 2 (correct = false: v_k); E is N x N scratch.
+template <class T, int NT>
+__device__ __forceinline__ void finalize_z(const T* V, int ldvs, int N, T* E, int lde, bool correct, T* Z,
+                                           long long ldz, const int* rank) {
+    using R = Real<T>;
+    const int tid = threadIdx.x;
+    {
+        if (correct) {
+            for (int e = tid; e < N * (N + 1) / 2; e += NT) {
+                int ca, cb;
+                tri_index(e, ca, cb);
+                T acc = make_s<T>(0);
+                for (int i = 0; i < N; ++i)
+                    acc = cfma(V[i + (long long)ca * ldvs], V[i + (long long)cb * ldvs], acc);
+                if (ca == cb) acc = make_s<T>(re(acc) - R(1));
+                E[ca + (long long)cb * lde] = acc;
+                E[cb + (long long)ca * lde] = conj_s(acc);
+            }
+            __syncthreads();
+        }
+        for (int e = tid; e < N * N; e += NT) {
+            const int i = e % N, k = e / N;
+            T z = V[i + (long long)k * ldvs];
+            if (correct) {
+                T acc = make_s<T>(0);
+                for (int j = 0; j < N; ++j) acc = fma_s(V[i + (long long)j * ldvs], E[j + (long long)k * lde], acc);
+                z = sub(z, scale(acc, R(0.5)));
+            }
+            Z[i + (long long)rank[k] * ldz] = z;
+        }
+    }
+}
+
+// The end of Alg. 2 for one matrix, by a whole CTA of NT threads.
+//   sigma_k = ||w_k||_2 (exact power-of-two scaled sum of squares), a stable
+//   descending sort (rank of each column), Sout[rank] = sigma * 2^ex;
+//   Y[:, rank_k] = w_k / sigma_k (U, or V for a transposed problem) when
+//   wantY, with zero columns completed to an orthonormal basis;
+//   Z[:, rank_k] = v_k - (V (V^H V - I))_k / 2 (one Newton-Schulz step
+//   towards the nearest orthonormal V) when wantZ; `correct` = false copies V.
+// W (M x N, ldw) and V (N x N, ldvs) may live in shared or global memory.
+// x (M elements) and E (N x N, lde) are scratch and may alias W: W is not
+// read after Y is complete.
+template <class T, int NT>
+__device__ void finalize_outputs(const T* W, int ldw, const T* V, int ldvs, int M, int N, int ex,
+                                 T* x, T* E, int lde, bool correct, Real<T>* Sout, T* Y,
+                                 long long ldy, bool wantY, T* Z, long long ldz, bool wantZ,
+                                 const FinalScratch<T>& fs) {
+    using R = Real<T>;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const R* sig = fs.sig;
+    const int* rank = fs.rank;
+    finalize_sigma<T, NT>(W, ldw, M, N, ex, Sout, fs);
     if (wantY) {
         for (int e = tid; e < M * N; e += NT) {
             const int i = e % M, k = e / M;
@@ -688,31 +752,7 @@ __device__ void finalize_outputs(const T* W, int ldw, const T* V, int ldvs, int 
         }
     }
     __syncthreads();
-    if (wantZ) {
-        if (correct) {
-            for (int e = tid; e < N * (N + 1) / 2; e += NT) {
-                int ca, cb;
-                tri_index(e, ca, cb);
-                T acc = make_s<T>(0);
-                for (int i = 0; i < N; ++i)
-                    acc = cfma(V[i + (long long)ca * ldvs], V[i + (long long)cb * ldvs], acc);
-                if (ca == cb) acc = make_s<T>(re(acc) - R(1));
-                E[ca + (long long)cb * lde] = acc;
-                E[cb + (long long)ca * lde] = conj_s(acc);
-            }
-            __syncthreads();
-        }
-        for (int e = tid; e < N * N; e += NT) {
-            const int i = e % N, k = e / N;
-            T z = V[i + (long long)k * ldvs];
-            if (correct) {
-                T acc = make_s<T>(0);
-                for (int j = 0; j < N; ++j) acc = fma_s(V[i + (long long)j * ldvs], E[j + (long long)k * lde], acc);
-                z = sub(z, scale(acc, R(0.5)));
-            }
-            Z[i + (long long)rank[k] * ldz] = z;
-        }
-    }
+    if (wantZ) finalize_z<T, NT>(V, ldvs, N, E, lde, correct, Z, ldz, rank);
 }
 
 }  // namespace bsvd

@@ -2,9 +2,10 @@
 //
 // FP64 results from mostly-FP32 work: the FP32 solver runs on an FP32 copy
 // of A until its own convergence test passes, giving V32; this file's
-// kernels then restore an orthonormal V in FP64 (two Newton-Schulz steps
-// V <- V - V (V^H V - I) / 2 from the widened V32) and form A_hat = A V in
-// FP64; FP64 polish sweeps on A_hat, starting from that V, win the accuracy
+// kernels then restore an orthonormal V in FP64 (Newton-Schulz steps
+// V <- V - V (V^H V - I) / 2 from the widened V32, up to 127 columns with a
+// preconditioning and a first-order diagonalisation step between them) and
+// form A_hat = A V in FP64; FP64 polish sweeps on A_hat, starting from that V, win the accuracy
 // back (the FP64 test decides convergence).  On a GB300, whose FP64 rate is
 // about 1/64 of its FP32 rate, the polish needs a few FP64 sweeps instead of
 // the full count.
@@ -14,6 +15,7 @@
 
 #include "internal.h"
 #include "jacobi_common.cuh"
+#include "precondition.cuh"
 
 namespace bsvd {
 
@@ -66,12 +68,88 @@ __global__ void __launch_bounds__(kMxThreads) mx_convert(const MixedArgs a) {
     }
 }
 
-// V (N x N) = two Newton-Schulz steps from widen(V32); A_hat (M x N, ld M) =
-// A' V in FP64, A' = A or A^H.  One CTA per matrix on L2-resident buffers.
+// V <- V - V (V^H V - I) / 2 (N x N, ld N), from Vin to Vout; E is scratch.
+// Synchronised on return.
+template <class T64, int NT>
+__device__ __forceinline__ void mx_newton_schulz(const T64* Vin, T64* Vout, T64* E, int N) {
+    using R = Real<T64>;
+    const int tid = threadIdx.x;
+    for (int e = tid; e < N * (N + 1) / 2; e += NT) {
+        int ca, cb;
+        tri_index(e, ca, cb);
+        T64 acc = make_s<T64>(0);
+        for (int i = 0; i < N; ++i) acc = cfma(Vin[i + (long long)ca * N], Vin[i + (long long)cb * N], acc);
+        if (ca == cb) acc = make_s<T64>(re(acc) - R(1));
+        E[ca + (long long)cb * N] = acc;
+        E[cb + (long long)ca * N] = conj_s(acc);
+    }
+    __syncthreads();
+    for (int e = tid; e < N * N; e += NT) {
+        const int i = e % N, k = e / N;
+        T64 acc = make_s<T64>(0);
+        for (int j = 0; j < N; ++j) acc = fma_s(Vin[i + (long long)j * N], E[j + (long long)k * N], acc);
+        Vout[i + (long long)k * N] = sub(Vin[i + (long long)k * N], scale(acc, R(0.5)));
+    }
+    __syncthreads();
+}
+
+// First-order diagonalisation of L^H L (L: N x N, leading dimension ldl) from
+// the V that belongs to it: Vout = V (I + Omega), Omega antihermitian with
+// omega_ij = g_ij / (g_jj - g_ii), where that is below 1e-2 (closer pairs are
+// left to the sweeps).  One product instead of a sweep's dependent rotations:
+// off-diagonals of 1e-7 become 1e-14.  d: N reals in shared memory.  V (I +
+// Omega) is orthonormal to |Omega|^2; the caller restores it.
+template <class T64, int NT>
+__device__ __forceinline__ void mx_refine(const T64* L, int ldl, const T64* V, T64* Vout, T64* E, Real<T64>* d, int N) {
+    using R = Real<T64>;
+    const int tid = threadIdx.x;
+    for (int e = tid; e < N * (N + 1) / 2; e += NT) {
+        int ca, cb;
+        tri_index(e, ca, cb);
+        T64 acc = make_s<T64>(0);
+        for (int i = cb; i < N; ++i)                       // L is lower triangular
+            acc = cfma(L[i + (long long)ca * ldl], L[i + (long long)cb * ldl], acc);
+        E[ca + (long long)cb * N] = acc;
+        if (ca == cb) d[ca] = re(acc);
+    }
+    __syncthreads();
+    for (int e = tid; e < N * (N + 1) / 2; e += NT) {
+        int ca, cb;
+        tri_index(e, ca, cb);
+        T64 w = make_s<T64>(0);
+        if (ca < cb) {
+            const T64 g = E[ca + (long long)cb * N];
+            const R den = d[cb] - d[ca];
+            if (abs_rot(g) < R(1e-2) * abs_s(den)) w = divr(g, den);
+        }
+        E[ca + (long long)cb * N] = w;
+        E[cb + (long long)ca * N] = scale(conj_s(w), R(-1));
+    }
+    __syncthreads();
+    for (int e = tid; e < N * N; e += NT) {
+        const int i = e % N, k = e / N;
+        T64 acc = V[i + (long long)k * N];
+        for (int j = 0; j < N; ++j) acc = fma_s(V[i + (long long)j * N], E[j + (long long)k * N], acc);
+        Vout[i + (long long)k * N] = acc;
+    }
+    __syncthreads();
+}
+
+// V (N x N) orthonormal in FP64 from V32, close to the right singular vectors
+// of A' = A or A^H; A_hat (M x N, ld M) = A' V.  One CTA per matrix on
+// L2-resident buffers:
+//   V = widen(V32), one Newton-Schulz step; A_hat = A' V (off-diagonal to
+//   1e-7, FP32's accuracy, but O(1) relative to short columns of a graded
+//   matrix); A_hat P = Q L Z^H, V <- V P Z (precondition.cuh: contracts those
+//   by the squared ratio of the singular values); the first-order step on
+//   L^H L; two Newton-Schulz steps; A_hat = A' V.
+// The FP64 sweeps that follow need 2 sweeps instead of 4 on 128 x 64 with
+// kappa = 1e6, 3.5 instead of 8 on the clustered 96 x 96 set.
 template <class T64, class T32>
 __global__ void __launch_bounds__(kMxThreads) mx_restore(const MixedArgs a) {
     using R = Real<T64>;
     constexpr int NT = kMxThreads;
+    extern __shared__ __align__(16) unsigned char smem[];
     const int b = blockIdx.x, tid = threadIdx.x;
     const int M = a.M, N = a.N;
     const long long nn = (long long)N * N;
@@ -79,40 +157,34 @@ __global__ void __launch_bounds__(kMxThreads) mx_restore(const MixedArgs a) {
     T64* Va = static_cast<T64*>(a.V64) + b * nn;
     T64* Vb = static_cast<T64*>(a.Vtmp) + b * nn;
     T64* E = static_cast<T64*>(a.E) + b * nn;
-    for (int e = tid; e < N * N; e += NT) Va[e] = widen_s(V32[e]);
-    __syncthreads();
-    for (int it = 0; it < 2; ++it) {
-        for (int e = tid; e < N * (N + 1) / 2; e += NT) {
-            int ca, cb;
-            tri_index(e, ca, cb);
-            T64 acc = make_s<T64>(0);
-            for (int i = 0; i < N; ++i) acc = cfma(Va[i + (long long)ca * N], Va[i + (long long)cb * N], acc);
-            if (ca == cb) acc = make_s<T64>(re(acc) - R(1));
-            E[ca + (long long)cb * N] = acc;
-            E[cb + (long long)ca * N] = conj_s(acc);
-        }
-        __syncthreads();
-        for (int e = tid; e < N * N; e += NT) {
-            const int i = e % N, k = e / N;
-            T64 acc = make_s<T64>(0);
-            for (int j = 0; j < N; ++j) acc = fma_s(Va[i + (long long)j * N], E[j + (long long)k * N], acc);
-            Vb[i + (long long)k * N] = sub(Va[i + (long long)k * N], scale(acc, R(0.5)));
-        }
-        __syncthreads();
-        T64* t = Va; Va = Vb; Vb = t;     // two steps: the result is back in the V64 buffer
-    }
+    T64* Ah = static_cast<T64*>(a.Ahat) + (long long)b * M * N;
     const T64* A = mixed_a<T64>(a, b);
     const int lda = a.Ap ? a.ldap[a.index[b]] : a.lda;
-    T64* Ah = static_cast<T64*>(a.Ahat) + (long long)b * M * N;
-    for (int e = tid; e < M * N; e += NT) {
-        const int i = e % M, k = e / M;
-        T64 acc = make_s<T64>(0);
-        for (int j = 0; j < N; ++j) {
-            const T64 aij = a.trans ? conj_s(A[j + (long long)i * lda]) : A[i + (long long)j * lda];
-            acc = fma_s(aij, Va[j + (long long)k * N], acc);
+    auto product = [&](const T64* V) {                     // A_hat = A' V
+        for (int e = tid; e < M * N; e += NT) {
+            const int i = e % M, k = e / M;
+            T64 acc = make_s<T64>(0);
+            for (int j = 0; j < N; ++j) {
+                const T64 aij = a.trans ? conj_s(A[j + (long long)i * lda]) : A[i + (long long)j * lda];
+                acc = fma_s(aij, V[j + (long long)k * N], acc);
+            }
+            Ah[i + (long long)k * M] = acc;
         }
-        Ah[i + (long long)k * M] = acc;
-    }
+        __syncthreads();
+    };
+    for (int e = tid; e < N * N; e += NT) Vb[e] = widen_s(V32[e]);
+    __syncthreads();
+    mx_newton_schulz<T64, NT>(Vb, Va, E, N);
+    product(Va);
+    const PreScratch<T64> sc(smem, N);
+    // A_hat carries A's scale: without it where squares could leave FP64's range (or A is not finite)
+    int wide = 0;
+    for (int e = tid; e < M * N; e += NT) wide |= !(maxabs(Ah[e]) < R(1e100));
+    if (!__syncthreads_or(wide) && precondition<T64, NT>(Ah, M, M, N, Vb, N, Va, N, nullptr, 0, sc))
+        mx_refine<T64, NT>(Ah, M, Vb, Va, E, sc.nrm2, N);
+    mx_newton_schulz<T64, NT>(Va, Vb, E, N);
+    mx_newton_schulz<T64, NT>(Vb, Va, E, N);
+    product(Va);
 }
 
 // ---- the restoration tiled over the whole GPU (N >= kMxTiledN) ---------------
@@ -290,7 +362,7 @@ cudaError_t mixed_prepare(const MixedArgs& a, int batch, cudaStream_t st) {
 template <class T64, class T32>
 cudaError_t mixed_restore(const MixedArgs& a, int batch, cudaStream_t st) {
     if (a.N >= kMxTiledN) return mixed_restore_tiled<T64, T32>(a, batch, st);
-    mx_restore<T64, T32><<<batch, kMxThreads, 0, st>>>(a);
+    mx_restore<T64, T32><<<batch, kMxThreads, (size_t)PreScratch<T64>::bytes(a.N), st>>>(a);
     return cudaGetLastError();
 }
 

@@ -24,12 +24,12 @@
 
 namespace bsvd {
 
-// Global -> shared copies of 4 or 8 bytes that do not wait for the data, so
+// Global -> shared copies of 4, 8 or 16 bytes that do not wait for the data, so
 // that the next staged panel chunk loads while the tensor cores work on the
 // current one; a source size of 0 writes zeros.
 template <int BYTES>
 __device__ __forceinline__ void cp_async(void* dst, const void* src, int src_bytes) {
-    static_assert(BYTES == 4 || BYTES == 8, "4- or 8-byte copies");
+    static_assert(BYTES == 4 || BYTES == 8 || BYTES == 16, "4-, 8- or 16-byte copies");
     const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
     asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;\n" ::"r"(d), "l"(src), "n"(BYTES), "r"(src_bytes)
                  : "memory");
