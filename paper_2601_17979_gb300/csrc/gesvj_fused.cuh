@@ -145,14 +145,14 @@ __device__ __forceinline__ long long pre_bytes(int M, int N) {
 // Whether the sweeps start from the preconditioned matrix (precondition.cuh):
 // a rule on the shape; a flat spectrum may still decline.  Measured against
 // the sweeps without it (ms, batches of 500 to 5,000):
-//   nb = 16: FP64 128 x 64, kappa 1e6, 4,000: 317 -> 99; FP32 128 x 64, kappa
+//   nb = 16: FP64 128 x 64, kappa 1e6, 4,000: 317 -> 92; FP32 128 x 64, kappa
 //   1e3, 3,000: 12.0 -> 7.1; complex64 64 x 64, kappa 1e3, 2,000: 18.0 -> 12.0;
 //   nb = 8 (below 48 columns, the AUTO rule's width): FP64 20 x 20 5.55 -> 5.24,
 //   complex128 40 x 40 17.8 -> 15.8, complex64 97 x 45 13.5 -> 12.5; but FP32
 //   32 x 32 2.3 -> 2.4 and complex64 32 x 32 4.2 -> 4.6;
 //   one pair of blocks (at most 2 nb columns): complex128 24 x 16 1.48 -> 1.76,
 //   FP32 100 x 16 0.85 -> 1.1, worth it only for the rows QR takes off tall
-//   FP64 (1000 x 16, 1,000: 13.1 -> 11.0).
+//   FP64 (1000 x 16, 1,000: 13.1 -> 7.9).
 // Single precision up to 160 columns (on chip about 128): beyond, on global
 // slots, it would move FP32 results as noted at cross_only.  A caller that sets
 // inner_sweeps gets the sweeps of the plain method from the start, and a start

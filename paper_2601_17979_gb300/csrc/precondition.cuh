@@ -25,7 +25,7 @@
 //
 // What bounds it: N dependent steps per factorisation, in FP64 the FP64 pipe
 // (66 % busy), in FP32 latency and shared-memory bandwidth.  128 x 64, one CTA:
-// FP64 1.63 M cycles and 0.85 M for Q's application (17 sweeps take 23 M, the
+// FP64 1.48 M cycles and 0.74 M for Q's application (17 sweeps take 23 M, the
 // 6.3 left 5 M); FP32 0.21 M and 0.075 M on the float4 form below (0.45 M and
 // 0.20 M on the scalar one), 11 sweeps about 1.5 M.  Measured and not kept:
 // panels of eight vectors factorised by one warp in registers (FP32 0.35 M;
@@ -105,9 +105,10 @@ __device__ __forceinline__ void reflection(T x0, Real<T> ss, T& ph, Real<T>& tau
     tau = rmul(st, st);
 }
 
-// Elements in flight per pass of the two loops below: what the products of a
-// reflection wait for is shared-memory latency, not arithmetic.
-template <class T> constexpr int kPreBatch = sizeof(T) <= 8 ? 8 : 4;
+// Elements per pass of the two loops below.  Single precision waits for
+// shared-memory latency: eight loads of each operand in flight, the last pass
+// padded with zeros.  FP64 waits for its arithmetic pipe: two, none wasted.
+template <class T> constexpr int kPreBatch = sizeof(Real<T>) == 4 ? 8 : 2;
 
 // sum over i < n of conj(v[i sv]) y[i sy] (ConjV) or v[i sv] conj(y[i sy])
 template <class T, bool ConjV>
@@ -115,7 +116,16 @@ __device__ __forceinline__ T strided_dot(const T* v, int sv, const T* y, int sy,
     constexpr int B = kPreBatch<T>;
     T a = make_s<T>(0), b = make_s<T>(0);
     auto mac = [](T x, T z, T acc) { return ConjV ? cfma(x, z, acc) : fma_s(x, conj_s(z), acc); };
-    for (int i = 0; i < n; i += B) {
+    int i = 0;
+    if constexpr (sizeof(Real<T>) == 8) {
+#pragma unroll 2
+        for (; i + 1 < n; i += 2) {
+            a = mac(v[i * sv], y[i * sy], a);
+            b = mac(v[(i + 1) * sv], y[(i + 1) * sy], b);
+        }
+        if (i < n) a = mac(v[i * sv], y[i * sy], a);
+    } else
+    for (; i < n; i += B) {
         T vv[B], yy[B];
 #pragma unroll
         for (int u = 0; u < B; ++u) {
@@ -135,6 +145,10 @@ __device__ __forceinline__ T strided_dot(const T* v, int sv, const T* y, int sy,
 template <class T>
 __device__ __forceinline__ void strided_axpy(const T* v, int sv, T* y, int sy, int n, T f) {
     constexpr int B = kPreBatch<T>;
+    if constexpr (sizeof(Real<T>) == 8) {
+#pragma unroll 4
+        for (int i = 0; i < n; ++i) y[i * sy] = nfma(v[i * sv], f, y[i * sy]);
+    } else
     for (int i = 0; i < n; i += B) {
         T vv[B], yy[B];
 #pragma unroll
