@@ -197,6 +197,9 @@ __device__ __forceinline__ double abs_rot(double2 z) {
 // the FP64 pipe does not share.
 __device__ __forceinline__ int as_ord(float x) { return __float_as_int(x); }
 __device__ __forceinline__ long long as_ord(double x) { return __double_as_longlong(x); }
+// biased binary exponent (0: zero or denormal)
+__device__ __forceinline__ int binary_exponent(float x) { return (__float_as_int(x) >> 23) & 0xff; }
+__device__ __forceinline__ int binary_exponent(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 template <class R> struct RotRange;
 template <> struct RotRange<float> { static constexpr float lo = 1e-18f, hi = 1e18f; };
 template <> struct RotRange<double> { static constexpr double lo = 1e-150, hi = 1e150; };
@@ -389,6 +392,22 @@ __device__ __forceinline__ int inner_rotation(T* G, Real<T> tol, int p, int q, i
     return fire;
 }
 
+// Whether G's columns span more than a factor of 2^20 in norm (2^40 on the
+// diagonal).  Such a block is far from converged, and full sweeps take fewer
+// outer sweeps there (48 columns graded over 2^150: 29 against 38).  The same
+// answer in every warp.
+template <class T, int TWO, int LDG>
+__device__ __forceinline__ bool graded_block(const T* G) {
+    const int lane = threadIdx.x & 31;
+    int lo = 1 << 20, hi = 0;
+    for (int i = lane; i < TWO; i += 32) {
+        const int e = binary_exponent(re(G[i + i * LDG]));
+        if (e > 0) lo = min(lo, e);                        // zero columns do not count
+        hi = max(hi, e);
+    }
+    return (int)__reduce_max_sync(0xffffffffu, hi) - (int)__reduce_min_sync(0xffffffffu, lo) > 40;
+}
+
 // Up to `sweeps` sweeps of Alg. 1 on the Hermitian G (2NB x 2NB, leading
 // dimension 2NB+1, in shared memory), accumulating the rotations into J
 // (set to I here).  One sweep is 2NB-1 parallel steps of the round-robin
@@ -425,6 +444,7 @@ __device__ int inner_jacobi(T* G, T* J, const InnerTables<T, NB>& tb, Real<T> to
                             bool cross = false) {
     using R = Real<T>;
     constexpr int TWO = 2 * NB, LDG = TWO + 1;
+    if (cross) cross = !graded_block<T, TWO, LDG>(G);
     const int STEPS = cross ? NB : TWO - 1;
     // The off-diagonal 2x2 blocks of G by slot pair (two rotations each);
     // the diagonal ones (the closed form) are applied by the lane of warp 0

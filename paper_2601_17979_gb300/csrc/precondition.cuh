@@ -210,6 +210,33 @@ __device__ __forceinline__ void reflect_columns(T* X, int ldx, int k, int M, int
 template <int NT>
 __device__ __forceinline__ bool eight_lanes(int N) { return NT <= 128 && 8 * N <= NT; }
 
+// Whether the rows' largest entries span more than a factor of 2^10 (zero rows
+// apart).  The factorisations are accurate relative to each column, not to each
+// row: from a matrix with rows of very different sizes they would take the
+// relative accuracy of its smallest singular values, which the plain start
+// keeps.  red: 2 NT / 32 ints.  Synchronised.
+template <class T, int NT>
+__device__ __forceinline__ bool graded_rows(const T* W, int ldw, int M, int N, int* red) {
+    constexpr int NW = NT / 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int lo = 1 << 20, hi = 0;
+    for (int r = tid; r < M; r += NT) {
+        int e = 0;
+        for (int j = 0; j < N; ++j) e = max(e, binary_exponent(maxabs(W[r + (long long)j * ldw])));
+        if (e > 0) {
+            lo = min(lo, e);
+            hi = max(hi, e);
+        }
+    }
+    lo = (int)__reduce_min_sync(0xffffffffu, (unsigned)lo);
+    hi = (int)__reduce_max_sync(0xffffffffu, (unsigned)hi);
+    if (lane == 0) { red[2 * warp] = lo; red[2 * warp + 1] = hi; }
+    __syncthreads();
+    for (int w = 0; w < NW; ++w) { lo = min(lo, red[2 * w]); hi = max(hi, red[2 * w + 1]); }
+    __syncthreads();
+    return hi - lo > 10;
+}
+
 // Whether the spectrum is so flat that the sweeps gain little from the
 // preconditioner: the participation ratio (sum sigma^2)^2 / (N sum sigma^4)
 // above 0.35 (iid normal entries: 0.5 square, 0.67 at 2:1; geometric spectra:
@@ -294,7 +321,8 @@ __device__ __forceinline__ void sort_columns(T* W, int ldw, int M, int N, const 
 // to refl (M x N, scaled so that tau = 1; null: dropped).  Called by all NT
 // threads after W is complete and synchronised; returns synchronised.
 // Returns false, with nothing changed, when a column is too short to square
-// safely (or zero), and in single precision when the spectrum is flat.
+// safely (or zero), when the rows are graded, and in single precision when the
+// spectrum is flat.
 //
 // Double precision picks each column by its remaining norm (QR with column
 // pivoting: 128 x 64 with kappa = 1e6 then takes 6.3 sweeps, 7.1 without).
@@ -372,6 +400,7 @@ __device__ __forceinline__ bool precondition(T* W, int ldw, int M, int N, T* V, 
     bool small = false;
     for (int j = lane; j < N; j += 32) small |= !(sc.nrm2[j] > kPreNormMin<R>);
     if (__any_sync(0xffffffffu, small)) { __syncthreads(); return false; }   // uniform: every warp reads all norms
+    if (graded_rows<T, NT>(W, ldw, M, N, reinterpret_cast<int*>(sc.v0))) return false;
     if constexpr (sizeof(R) == 4)
         if (M <= 2 * N && flat_spectrum<T, NT>(W, ldw, M, N, sc.nrm2, sc.v0, sc.tau)) return false;
     if constexpr (sizeof(R) == 4)
@@ -673,6 +702,7 @@ __device__ __forceinline__ bool precondition_f32(float* W, int ldw, int M, int N
     bool small = false;
     for (int j = lane; j < N; j += 32) small |= !(sc.nrm2[j] > kPreNormMin<float>);
     if (__any_sync(0xffffffffu, small)) { __syncthreads(); return false; }   // uniform: every warp reads all norms
+    if (graded_rows<float, NT>(W, ldw, M, N, sc.tmp)) return false;
     if (flat_spectrum<float, NT>(W, ldw, M, N, sc.nrm2, sc.v, sc.tau)) return false;
     sort_columns<float, NT>(W, ldw, M, N, sc.nrm2, sc.perm, sc.tmp, sc.tmp + N);
 

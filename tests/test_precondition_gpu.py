@@ -109,6 +109,22 @@ def test_small_singular_values_of_scaled_columns(dtype):
         assert rel.max() <= 50 * n * u * cond[k], (k, rel.max())
 
 
+@pytest.mark.parametrize("dtype", [np.float32, np.float64, np.complex64, np.complex128])
+def test_small_singular_values_of_scaled_rows(dtype):
+    """Rows of very different sizes: the plain start is kept, and with it the
+    small singular values' relative accuracy."""
+    rng = np.random.default_rng(10)
+    m, n = 70, 48
+    B = rng.standard_normal((m, n)) + (1j * rng.standard_normal((m, n)) if np.issubdtype(dtype, np.complexfloating) else 0)
+    B[::3] *= 2.0 ** -40                                     # 46 rows of size 1: two singular values near 2^-40
+    mats = [B.astype(dtype)]
+    ref = oracle.gesvj(mats)["S"][0]
+    assert ref[-3] > 1e-3 and ref[-2] < 1e-10
+    S = run(mats, nb=16)[0][0]
+    cond = np.linalg.cond(B[np.arange(m) % 3 != 0])
+    assert np.abs(S - ref)[-2:].max() <= 50 * n * checks.unit_roundoff(dtype) * cond * ref[-2]
+
+
 @pytest.mark.parametrize("m,n", [(128, 64), (96, 96), (64, 100), (33, 20), (9, 3)])
 @pytest.mark.parametrize("dtype", [np.float64, np.complex128])
 def test_mixed_restoration(m, n, dtype):
