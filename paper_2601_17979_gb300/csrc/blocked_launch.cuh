@@ -124,13 +124,15 @@ cudaError_t blk_run_nb(BlockedArgs a, void* work, cudaStream_t st, bool two_stag
     a.J = base;  base += (size_t)nJ;
     a.T = base;
 
+    constexpr bool kSplit = std::is_same<T, double>::value && NB == 16;   // tc_f64.cuh
     const int heevj_smem = 2 * TWO * LDG * (int)sizeof(T) + InnerTables<T, NB>::bytes();
     const int fin_smem = (kBlkThreads / 32) * (int)sizeof(R) + 16 + 2 * (int)sizeof(T) +
                          a.N * ((int)sizeof(R) + 4) + 16;
     // J, column stride up to 2nb + 1; real FP32 J's split-TF32 fragments
     const int upd_smem = std::max(TWO * (TWO + 1) * (int)sizeof(T),
                                   std::is_same<T, float>::value    ? j_fragment_bytes<NB>()
-                                  : std::is_same<T, float2>::value ? jc_fragment_bytes<NB>() : 0);
+                                  : std::is_same<T, float2>::value ? jc_fragment_bytes<NB>()
+                                  : kSplit                         ? kJDigitBytes + 2 * TWO * (int)sizeof(int) : 0);
     if ((e = allow_dynamic_smem<blk_heevj<T, NB, GT>>()) != cudaSuccess ||
         (e = allow_dynamic_smem<blk_finalize<T>>()) != cudaSuccess ||
         (e = allow_dynamic_smem<blk_update_fused<T, NB>>()) != cudaSuccess ||
@@ -156,7 +158,8 @@ cudaError_t blk_run_nb(BlockedArgs a, void* work, cudaStream_t st, bool two_stag
     }
     const long long pairs = (long long)a.count * (a.L / 2);
     const int zrows = (a.M + a.N + kUpdRows - 1) / kUpdRows;
-    const int zcap = (int)std::max(1LL, (16LL * sms + pairs - 1) / pairs);
+    // (FP64 digits: two CTAs per SM do, each prepares J's digits for its share)
+    const int zcap = (int)std::max(1LL, ((kSplit && !two_stage ? 2LL : 16LL) * sms + pairs - 1) / pairs);
     const dim3 gupd(a.count, a.L / 2, two_stage ? zrows : std::min(zrows, zcap));
     // one sweep: every round's stages, then the end-of-sweep bookkeeping
     auto sweep = [&](cudaStream_t s) -> cudaError_t {
@@ -176,6 +179,10 @@ cudaError_t blk_run_nb(BlockedArgs a, void* work, cudaStream_t st, bool two_stag
                 // complex64: the tensor cores (flags bit 7: the FMA pipes)
                 if (a.flags & 128) blk_gram<T, NB><<<gpair, kBlkThreads, 0, s>>>(a, r);
                 else blk_gram_c64_tc<NB><<<gpair, kBlkThreads, 0, s>>>(a, r);
+            }
+            else if constexpr (kSplit) {
+                if (two_stage) blk_gram<T, NB><<<gpair, kBlkThreads, 0, s>>>(a, r);
+                else blk_gram_f64_tc<<<gpair, kPairGramThreads, 0, s>>>(a, r);
             }
             else
                 blk_gram<T, NB><<<gpair, kBlkThreads, 0, s>>>(a, r);

@@ -21,10 +21,11 @@
 #include "jacobi_common.cuh"
 #include "tc_c64.cuh"
 #include "tc_f32.cuh"
+#include "tc_f64.cuh"
 
 namespace bsvd {
 
-enum : int { kBlkThreads = 256, kUpdRows = 128, kGramChunk = 64 };
+enum : int { kBlkThreads = 256, kUpdRows = 128, kGramChunk = 64, kPairGramThreads = 128 };
 
 __device__ __forceinline__ int blk_mid(const BlockedArgs& a, int b) { return a.index ? a.index[b] : b; }
 
@@ -397,6 +398,26 @@ __global__ void __launch_bounds__(kBlkThreads) blk_gram(const BlockedArgs a, int
     }
 }
 
+// ---- S2, real FP64, nb = 16: exact digit products on the tensor cores ------------
+// (tc_f64.cuh).  The FP64 pipe bounds blk_gram (95 % busy, 206 us a round for
+// 64 matrices of 256 x 256); here it only adds a few partial sums.
+static __global__ void __launch_bounds__(kPairGramThreads) blk_gram_f64_tc(const BlockedArgs a, int r) {
+    constexpr int NB = 16, TWO = 2 * NB;
+    __shared__ int ec[TWO];
+    __shared__ double Gs[TWO * (TWO + 1)];
+    const int b = blockIdx.x, q = blockIdx.y, tid = threadIdx.x;
+    if (blk_skip(a, b)) return;
+    const BlkShape sh = blk_shape(a, b);
+    int bi, bj;
+    if (!blk_pair(sh, r, q, bi, bj)) return;
+    const double* W = static_cast<const double*>(a.W) + sh.oW;
+    column_exponents_f64<kPairGramThreads>(W, sh.M, sh.M, bi * NB, bj * NB, ec, tid);
+    __syncthreads();
+    gram_f64_split<kPairGramThreads, TWO + 1>(W, sh.M, sh.M, bi * NB, bj * NB, ec, Gs, tid, 1);
+    double* G = static_cast<double*>(a.G) + sh.oG + (long long)q * TWO * TWO;
+    for (int e = tid; e < TWO * TWO; e += kPairGramThreads) G[e] = Gs[e % TWO + (e / TWO) * (TWO + 1)];
+}
+
 // ---- S3: the Hermitian eigensolver on each Gram block --------------------------
 // grid (count, L/2), GT threads.  J to global; flags the pair and the matrix.
 template <class T, int NB, int GT>
@@ -457,7 +478,7 @@ __global__ void __launch_bounds__(kUpdRows) blk_update_fused(const BlockedArgs a
     int bi, bj;
     if (!blk_pair(sh, r, q, bi, bj)) return;
     const int rows = sh.M + sh.N;
-    if (blockIdx.z * kUpdRows >= rows) return;
+    if (!(std::is_same<T, double>::value && NB == 16) && blockIdx.z * kUpdRows >= rows) return;
     const T* Jg = static_cast<const T*>(a.J) + sh.oJ + (long long)q * TWO * TWO;
     if constexpr (std::is_same<T, float>::value && (NB == 8 || NB == 16))
       if (!(a.flags & 128)) {
@@ -494,6 +515,21 @@ __global__ void __launch_bounds__(kUpdRows) blk_update_fused(const BlockedArgs a
             }
         return;
       }
+    if constexpr (std::is_same<T, double>::value && NB == 16) {
+        // real FP64: exact digit products on the tensor cores (tc_f64.cuh);
+        // a CTA's four warps take the 16-row tiles of its share of W, then of V.
+        // On the FP64 pipe this update ran at 93 % of it: 480 us a round for
+        // 64 matrices of 256 x 256.
+        uint2* Jd = reinterpret_cast<uint2*>(smem_js);
+        int* ek = reinterpret_cast<int*>(smem_js + kJDigitBytes);
+        const double* Gg = static_cast<const double*>(a.G) + sh.oG + (long long)q * TWO * TWO;
+        // exponents of the columns' norms (of 2^-511 where the square underflows)
+        if (tid < TWO) ek[tid] = (max(exp_f64(Gg[tid + tid * TWO]), 1) + 1023) / 2;
+        __syncthreads();
+        update_f64_split<kUpdRows>(static_cast<double*>(a.W) + sh.oW, sh.M, sh.M, static_cast<double*>(a.Vw) + sh.oV, sh.N,
+                                   sh.N, bi * NB, bj * NB, Jg, TWO, ek, Jd, ek + TWO, tid, 1, blockIdx.z, gridDim.z);
+        return;
+    }
     if constexpr (std::is_same<T, float2>::value && NB <= 16) {
         // complex64: 4 rows x 2nb/4 columns per thread.  The four lanes of a
         // quad share 4 rows (rs, rs + 32, ...) and take columns cg, cg + 4,

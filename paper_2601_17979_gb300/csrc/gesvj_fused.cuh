@@ -24,6 +24,7 @@
 #include "jacobi_common.cuh"
 #include "precondition.cuh"
 #include "tc_f32.cuh"
+#include "tc_f64.cuh"
 
 namespace bsvd {
 
@@ -94,15 +95,23 @@ __host__ __device__ inline long long fused_slot_elems(const FusedArgs& a) {
     return w + (long long)a.ldvs * a.Np;
 }
 
+// Real FP64 with nb = 16 forms the Gram block and the update as exact digit
+// products on the tensor cores (tc_f64.cuh).
+template <class T, int NB>
+__host__ __device__ constexpr bool fused_split() { return std::is_same<T, double>::value && NB == 16; }
+
 // FP32 adds J as split-TF32 fragments for the tensor-core update (nb >= 8:
 // 8 (2nb)^2 bytes) or J^T for the FFMA-tiled update (nb = 4), 16-byte
-// aligned; the other types a second J (the previous pair's, for the
-// deferred V update).
+// aligned; FP64 with nb = 16 J's digits, in the place of G once the inner sweep
+// is done, and two sets of column exponents; the others a second J (the
+// previous pair's, for the deferred V update).
 template <class T, int NB>
 __host__ __device__ constexpr int fused_group_bytes() {
-    return ((2 * (2 * NB) * (2 * NB + 1) * (int)sizeof(T) + InnerTables<T, NB>::bytes() + 15) & ~15) +
+    constexpr int mat = (2 * NB) * (2 * NB + 1) * (int)sizeof(T);
+    if (fused_split<T, NB>()) return ((mat + InnerTables<T, NB>::bytes() + 15) & ~15) + kJDigitBytes + 256;
+    return ((2 * mat + InnerTables<T, NB>::bytes() + 15) & ~15) +
            (std::is_same<T, float>::value ? (NB >= 8 ? 8 * (2 * NB) * (2 * NB) : (2 * NB) * (2 * NB) * 4)
-                                          : (((2 * NB) * (2 * NB + 1) * (int)sizeof(T) + 15) & ~15));
+                                          : ((mat + 15) & ~15));
 }
 
 // The V update of a block pair, [V_i V_j] <- [V_i V_j] J, run by whole warps
@@ -188,12 +197,16 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
     const bool wantWout = a.trans ? a.wantV : a.wantU; // W / sigma is part of the output
 
     unsigned char* gb = smem + a.offG + g * a.groupBytes;
-    T* G = reinterpret_cast<T*>(gb);
-    T* const J0 = G + TWO * LDG;
+    // G, J and the rotation tables; then, 16-byte aligned, J^T or J's fragments
+    // for FP32, or the second J buffer of the other types.  FP64 with nb = 16: J,
+    // the tables, then G, whose place J's digits take, and the exponents.
+    constexpr bool kSplit = fused_split<T, NB>();
+    constexpr int kMats = kSplit ? 1 : 2;
+    T* const J0 = reinterpret_cast<T*>(gb) + (kSplit ? 0 : TWO * LDG);
     const InnerTables<T, NB> tb(J0 + TWO * LDG);
-    // after the tables, 16-byte aligned: J^T for the FP32 tiled update, or
-    // the second J buffer of the other types
-    unsigned char* const gb_tail = gb + ((2 * TWO * LDG * (int)sizeof(T) + InnerTables<T, NB>::bytes() + 15) & ~15);
+    unsigned char* const gb_tail = gb + ((kMats * TWO * LDG * (int)sizeof(T) + InnerTables<T, NB>::bytes() + 15) & ~15);
+    T* const G = reinterpret_cast<T*>(kSplit ? gb_tail : gb);
+    int* const ek = reinterpret_cast<int*>(gb_tail + kJDigitBytes);   // [32] column exponents, then [32] J's (kSplit)
     float* Jt = reinterpret_cast<float*>(gb_tail);
     T* const J1 = reinterpret_cast<T*>(gb_tail);
     T* J = J0;
@@ -297,12 +310,12 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
     const R tol = (R)a.tol;
     int sw = 0;
     bool converged = false;
-    // FP64 and complex on chip: a pair's V update is deferred to the group's
+    // Complex and narrow FP64 on chip: a pair's V update is deferred to the group's
     // next pair step and run by the J-update warps during its inner sweep
     // (same arithmetic; the V blocks are read by nothing else in between).
     // Not with V in global memory: a warp reads one row of V, which in
     // global memory would touch a separate cache line per element.
-    constexpr bool kDefer = OnChip && !std::is_same<T, float>::value;
+    constexpr bool kDefer = OnChip && !std::is_same<T, float>::value && !kSplit;
     DeferredV<T, NB> dv{Vs, ldvs, N, nullptr, 0, 0};
     while (sw < a.max_sweeps) {
         for (int r = 0; r < a.L - 1; ++r) {
@@ -323,6 +336,10 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
                 if constexpr (std::is_same<T, float>::value) {
                     if (NB >= 8 && !(a.flags & kFlagF32Ffma)) gram_f32_mma<NB < 8 ? 8 : NB, GT>(W, ldw, M, bi * NB, bj * NB, G, gt);
                     else gram_f32_tiled<NB, GT>(W, ldw, M, bi * NB, bj * NB, G, gt);
+                } else if constexpr (kSplit) {
+                    column_exponents_f64<GT>(W, ldw, M, bi * NB, bj * NB, ek, gt);
+                    group_sync(g, GT);
+                    gram_f64_split<GT, LDG>(W, ldw, M, bi * NB, bj * NB, ek, G, gt, g + 1);
                 } else if constexpr (!OnChip) {
                     // W in global memory: 2 x 2 tiles of upper entries per lane
                     // pair, four independent sums (half the loads per FMA of
@@ -435,6 +452,9 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
                         group_sync(g, GT);
                         update_f32_tiled<NB, GT, 2>(W, ldw, pre ? (M + 3) & ~3 : ldw, Vs, ldvs, needVs ? ldvs : 0, bi * NB, bj * NB, Jt, gt, g + 1);
                     }
+                } else if constexpr (kSplit) {
+                    update_f64_split<GT>(W, ldw, M, Vs, ldvs, needVs ? N : 0, bi * NB, bj * NB, J, LDG, ek,
+                                         reinterpret_cast<uint2*>(gb_tail), ek + 32, gt, g + 1);
                 } else if constexpr (std::is_same<T, float2>::value) {
                     // complex64: 4 rows x 2nb/8 columns per lane (columns
                     // cg, cg + 8, ...: conflict-free J reads with its padded

@@ -1,0 +1,336 @@
+// tc_f64.cuh -- FP64 products on the tensor cores, exact in fixed point.
+//
+// A GB300 SM retires about 1.6 FP64 multiply-adds a clock and 0.47 FP16
+// 16 x 8 x 16 tile products (2,048 multiply-adds each), so the Gram block and
+// the rotation update of real FP64 split every operand into digits that the
+// FP16 units multiply exactly (the scheme of Ozaki, Ogita, Oishi and Rump,
+// "Error-free transformations of matrix multiplication by using fast routines
+// of matrix multiplication and its applications", Numer. Algorithms 59, 2012):
+//   x = 2^(E - 52) sum_i d_i 512^(5 - i),  d_i in [-256, 256], i = 0 .. 5,
+// E the largest exponent of the row (or column) the product sums over; an
+// entry keeps 53 bits below that exponent, rounded to nearest.  A product of
+// two digits is below 2^16 and a sum of 32 times the up to six digit products
+// of equal weight i + j below 2^24: exact in the FP32 accumulator.  Weights
+// up to 6 are kept (26 digit products); what is dropped is below 2^-58 of the
+// row's and column's largest product, the digits' own rounding 2^-53 -- the
+// error of one FP64 rounding at that size, where 32 chained multiply-adds
+// round 32 times.  Accumulators are converted and combined as integers and
+// rounded once to FP64; no FP64 instruction is used at all.
+//
+// Fragments (PTX ISA, mma.sync.m16n8k16 .f16), g = lane / 4, t = lane % 4:
+//   A (16 x 16)  a0 (g, 2t..2t+1)  a1 (g+8, 2t..)  a2 (g, 2t+8..)  a3 (g+8, 2t+8..)
+//   B (16 x 8)   b0 (2t..2t+1, g)  b1 (2t+8.., g)
+//   C (16 x 8)   c0 c1 (g, 2t..2t+1)  c2 c3 (g+8, 2t..)
+#pragma once
+
+#include <cuda_fp16.h>
+
+#include <cstdint>
+
+#include "jacobi_common.cuh"
+
+namespace bsvd {
+
+constexpr int kDigits = 6, kWeights = 7;       // weights i + j = 0 .. 6
+constexpr int kNoExp = -4000;                  // exponent of a zero
+
+// Biased exponent of x (denormals count as zero).
+__device__ __forceinline__ int exp_f64(double x) {
+    const int e = (__double2hiint(x) >> 20) & 0x7ff;
+    return e ? e : kNoExp;
+}
+
+// x as a 54-bit integer relative to exponent E = exp(x) + sh (sh >= 0), rounded
+// to nearest even (an entry one binary order below E drops one bit, a tie half
+// of the time: rounding those one way moves every column a quarter of a unit
+// per update), plus 256 in every digit: digit i is bits 9 (5 - i) .. of the
+// result less 256 (the leading one takes ten bits).
+__device__ __forceinline__ unsigned long long fixed_f64(double x, int sh) {
+    const long long b = __double_as_longlong(x);
+    long long m = (b & 0xfffffffffffffll) | 0x10000000000000ll;
+    if (((b >> 52) & 0x7ff) == 0) m = 0;
+    if (b < 0) m = -m;
+    const int s = min(sh, 60);
+    const long long v = s > 0 ? (m + (1ll << (s - 1)) - 1 + ((m >> s) & 1)) >> s : m;
+    // sum of 256 * 512^i, i < 6
+    return (unsigned long long)v + 0x20100804020100ull;
+}
+
+// digit i of two fixed-point values as an FP16 pair (x0 in the low half)
+template <int I>
+__device__ __forceinline__ uint32_t digit_pair(unsigned long long x0, unsigned long long x1) {
+    constexpr int S = 9 * (5 - I);
+    const uint32_t u0 = I == 0 ? (uint32_t)(x0 >> S) : (uint32_t)(x0 >> S) & 511u;
+    const uint32_t u1 = I == 0 ? (uint32_t)(x1 >> S) : (uint32_t)(x1 >> S) & 511u;
+    // 0x6400 + u is 1024 + u in FP16; less 1280
+    const uint32_t h = (u0 | (u1 << 16)) + 0x64006400u;
+    const __half2 r = __hsub2(*reinterpret_cast<const __half2*>(&h), __half2half2(__ushort_as_half(0x6500)));
+    return *reinterpret_cast<const uint32_t*>(&r);
+}
+
+__device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// The weights' sums as one integer in units of 512^4 / 2^21 (weight 2's unit
+// is 512^8): sum_o acc_o 512^(10 - o) = T 2^51, T below 2^62.
+__device__ __forceinline__ long long combine_weights(const float (&c)[kWeights]) {
+    const int i0 = __float2int_rn(c[0]), i1 = __float2int_rn(c[1]), i2 = __float2int_rn(c[2]), i3 = __float2int_rn(c[3]),
+              i4 = __float2int_rn(c[4]), i5 = __float2int_rn(c[5]), i6 = __float2int_rn(c[6]);
+    const long long hi = (long long)i0 * 262144 + ((long long)i1 * 512 + i2);
+    const long long lo = ((long long)i3 * 512 + i4) * 262144 + ((long long)i5 * 512 + i6);
+    return (hi << 21) + ((lo + (1 << 14)) >> 15);
+}
+
+// T 2^s to FP64, rounded to nearest; zero below the normal range.
+__device__ __forceinline__ double fixed_to_f64(long long T, int s) {
+    const unsigned long long a = T < 0 ? (unsigned long long)-T : (unsigned long long)T;
+    if (a == 0) return 0.0;
+    const int lz = __clzll((long long)a);
+    const int e = 1023 + 63 - lz + s;
+    if (e < 1) return 0.0;
+    const unsigned long long m = a << lz;                  // leading one at bit 63
+    // the leading one adds itself to the exponent field; a rounding carry too
+    const unsigned long long r = ((unsigned long long)(e - 1) << 52) + (m >> 11) + ((m >> 10) & 1);
+    return __longlong_as_double((long long)(r | ((unsigned long long)T & 0x8000000000000000ull)));
+}
+
+// Largest biased exponent of each of the 32 columns of a panel (columns [cbi,
+// cbi + 16) and [cbj, cbj + 16) of W, M rows) into ec.  GT threads (a multiple of
+// 32); the caller synchronises.
+template <int GT>
+__device__ __forceinline__ void column_exponents_f64(const double* W, long long ldw, int M, int cbi, int cbj, int* ec,
+                                                     int gt) {
+    constexpr int P = GT / 32;                             // threads a column
+    const int c = gt / P, q = gt % P;
+    const double* x = W + (c < 16 ? cbi + c : cbj + c - 16) * ldw;
+    int e = kNoExp;
+    for (int r = q; r < M; r += P) e = max(e, exp_f64(x[r]));
+#pragma unroll
+    for (int o = 1; o < P; o <<= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+    if (q == 0) ec[c] = e;
+}
+
+// S2: G = P^T P (32 x 32, column stride LDG) for the panel P of column_exponents.
+// Four warps take 16 rows in turn (always four: the bits do not depend on the
+// group's size); each forms the six 16 x 8 tiles that meet the
+// upper triangle from one set of digits (a column's digits serve as A and as B
+// fragment), converts them to FP64 and sums its own; the warps' sums are added
+// in warp order.  Upper entries are written and mirrored.  GT threads, named
+// barrier `bar`; synchronised on return.
+template <int GT, int LDG>
+__device__ __forceinline__ void gram_f64_split(const double* W, long long ldw, int M, int cbi, int cbj, const int* ec,
+                                               double* G, int gt, int bar) {
+    const int warp = gt >> 5, lane = gt & 31, g = lane >> 2, t = lane & 3;
+    double sum[6][4];
+#pragma unroll
+    for (int u = 0; u < 6; ++u)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) sum[u][i] = 0.0;
+    constexpr int NWS = 4;
+    static_assert(GT >= 32 * NWS, "four warps");
+    for (int k0 = warp < NWS ? 16 * warp : M; k0 < M; k0 += 16 * NWS) {
+        uint32_t D[kDigits][2][4];
+#pragma unroll
+        for (int bm = 0; bm < 2; ++bm)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int c = 8 * h + g;
+                const double* x = W + ((bm ? cbj : cbi) + c) * ldw;
+                const int E = ec[16 * bm + c];
+                unsigned long long v[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int r = k0 + 2 * t + (i & 1) + 8 * (i >> 1);
+                    const double y = r < M ? x[r] : 0.0;
+                    v[i] = fixed_f64(y, E - exp_f64(y));
+                }
+                D[0][bm][h] = digit_pair<0>(v[0], v[1]); D[0][bm][2 + h] = digit_pair<0>(v[2], v[3]);
+                D[1][bm][h] = digit_pair<1>(v[0], v[1]); D[1][bm][2 + h] = digit_pair<1>(v[2], v[3]);
+                D[2][bm][h] = digit_pair<2>(v[0], v[1]); D[2][bm][2 + h] = digit_pair<2>(v[2], v[3]);
+                D[3][bm][h] = digit_pair<3>(v[0], v[1]); D[3][bm][2 + h] = digit_pair<3>(v[2], v[3]);
+                D[4][bm][h] = digit_pair<4>(v[0], v[1]); D[4][bm][2 + h] = digit_pair<4>(v[2], v[3]);
+                D[5][bm][h] = digit_pair<5>(v[0], v[1]); D[5][bm][2 + h] = digit_pair<5>(v[2], v[3]);
+            }
+#pragma unroll
+        for (int u = 0; u < 6; ++u) {
+            const int bm = u < 4 ? 0 : 1, nt = u < 4 ? u : u - 2, bn = nt >> 1, h = nt & 1;
+            float acc[kWeights][4];
+#pragma unroll
+            for (int o = 0; o < kWeights; ++o)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) acc[o][i] = 0.f;
+#pragma unroll
+            for (int j = 0; j < kDigits; ++j)
+#pragma unroll
+                for (int i = 0; i < kDigits; ++i)
+                    if (i + j < kWeights) mma_f16(acc[i + j], D[i][bm], D[j][bn][h], D[j][bn][2 + h]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                float c[kWeights];
+#pragma unroll
+                for (int o = 0; o < kWeights; ++o) c[o] = acc[o][i];
+                const int rr = 16 * bm + g + 8 * (i >> 1), cc = 8 * nt + 2 * t + (i & 1);
+                sum[u][i] += fixed_to_f64(combine_weights(c), ec[rr] + ec[cc] - 2150 + 51);
+            }
+        }
+    }
+    for (int w = 0; w < NWS; ++w) {
+        if (warp == w) {
+#pragma unroll
+            for (int u = 0; u < 6; ++u)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int bm = u < 4 ? 0 : 1, nt = u < 4 ? u : u - 2;
+                    const int rr = 16 * bm + g + 8 * (i >> 1), cc = 8 * nt + 2 * t + (i & 1);
+                    if (rr > cc) continue;                 // lower entries: the mirror of an upper one
+                    const double x = w ? G[rr + cc * LDG] + sum[u][i] : sum[u][i];
+                    G[rr + cc * LDG] = x;
+                    G[cc + rr * LDG] = x;
+                }
+        }
+        named_sync(bar, GT);
+    }
+}
+
+// J (32 x 32, column stride ldj) for the update of columns scaled by 2^-ek[k]
+// (ek null: unscaled): B fragments of the digits of J_kc 2^(ek[k] - fc[c]), fc[c]
+// the largest exponent of column c.  Jd[((d * 2 + ks) * 4 + nt) * 32 + lane]:
+// 12 KB.  GT threads; the caller synchronises.
+constexpr int kJDigitBytes = kDigits * 2 * 4 * 32 * 8;
+template <int GT>
+__device__ __forceinline__ void j_digits_f64(const double* J, int ldj, const int* ek, uint2* Jd, int* fc, int gt) {
+    const int warp = gt >> 5, lane = gt & 31, g = lane >> 2, t = lane & 3;
+    for (int nt = warp; nt < 4; nt += GT / 32) {
+        const int c = 8 * nt + g;
+        double x[8];
+        int e[8], f = kNoExp;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int k = 16 * (i >> 2) + 2 * t + (i & 1) + 8 * ((i >> 1) & 1);
+            x[i] = J[k + c * ldj];
+            e[i] = exp_f64(x[i]) + (ek ? ek[k] : 0);
+            f = max(f, e[i]);
+        }
+        f = max(f, __shfl_xor_sync(0xffffffffu, f, 1));
+        f = max(f, __shfl_xor_sync(0xffffffffu, f, 2));
+        if (t == 0) fc[c] = f;
+        unsigned long long v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = fixed_f64(x[i], f - e[i]);
+#pragma unroll
+        for (int ks = 0; ks < 2; ++ks) {
+            uint2* o = Jd + (ks * 4 + nt) * 32 + lane;
+            o[0 * 256] = make_uint2(digit_pair<0>(v[4 * ks], v[4 * ks + 1]), digit_pair<0>(v[4 * ks + 2], v[4 * ks + 3]));
+            o[1 * 256] = make_uint2(digit_pair<1>(v[4 * ks], v[4 * ks + 1]), digit_pair<1>(v[4 * ks + 2], v[4 * ks + 3]));
+            o[2 * 256] = make_uint2(digit_pair<2>(v[4 * ks], v[4 * ks + 1]), digit_pair<2>(v[4 * ks + 2], v[4 * ks + 3]));
+            o[3 * 256] = make_uint2(digit_pair<3>(v[4 * ks], v[4 * ks + 1]), digit_pair<3>(v[4 * ks + 2], v[4 * ks + 3]));
+            o[4 * 256] = make_uint2(digit_pair<4>(v[4 * ks], v[4 * ks + 1]), digit_pair<4>(v[4 * ks + 2], v[4 * ks + 3]));
+            o[5 * 256] = make_uint2(digit_pair<5>(v[4 * ks], v[4 * ks + 1]), digit_pair<5>(v[4 * ks + 2], v[4 * ks + 3]));
+        }
+    }
+}
+
+// Rows [r0, r0 + 16) of a column-major X (rows valid below `rows`), columns
+// [cbi, cbi + 16) and [cbj, cbj + 16), times J in place, with the fragments of
+// j_digits_f64 for the same ek.  One warp; it reads all its inputs before it
+// writes any output, and no other warp touches these rows.
+__device__ __forceinline__ void update_rows_f64(double* X, long long ld, int rows, int r0, int cbi, int cbj, const int* ek,
+                                                const uint2* Jd, const int* fc, int lane) {
+    const int g = lane >> 2, t = lane & 3, ra = r0 + g, rb = r0 + g + 8;
+    auto col = [&](int c) { return (long long)(c < 16 ? cbi + c : cbj + c - 16) * ld; };
+    uint32_t A[kDigits][2][4];
+    int Ea = kNoExp, Eb = kNoExp;
+    {
+        double x[2][8];                                    // [row][entry]
+        int e[2][8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int k = 16 * (i >> 2) + 2 * t + (i & 1) + 8 * ((i >> 1) & 1);
+            const long long o = col(k);
+            x[0][i] = ra < rows ? X[ra + o] : 0.0;
+            x[1][i] = rb < rows ? X[rb + o] : 0.0;
+            const int sc = ek ? ek[k] : 0;
+            e[0][i] = exp_f64(x[0][i]);
+            e[1][i] = exp_f64(x[1][i]);
+            if (e[0][i] != kNoExp) e[0][i] -= sc;          // a zero does not count, whatever its column's scale
+            if (e[1][i] != kNoExp) e[1][i] -= sc;
+            Ea = max(Ea, e[0][i]);
+            Eb = max(Eb, e[1][i]);
+        }
+        Ea = max(Ea, __shfl_xor_sync(0xffffffffu, Ea, 1));
+        Eb = max(Eb, __shfl_xor_sync(0xffffffffu, Eb, 1));
+        Ea = max(Ea, __shfl_xor_sync(0xffffffffu, Ea, 2));
+        Eb = max(Eb, __shfl_xor_sync(0xffffffffu, Eb, 2));
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {                      // entry pairs (2p, 2p + 1): k-step p / 2, half p % 2
+            const unsigned long long a0 = fixed_f64(x[0][2 * p], Ea - e[0][2 * p]), a1 = fixed_f64(x[0][2 * p + 1], Ea - e[0][2 * p + 1]);
+            const unsigned long long b0 = fixed_f64(x[1][2 * p], Eb - e[1][2 * p]), b1 = fixed_f64(x[1][2 * p + 1], Eb - e[1][2 * p + 1]);
+            const int ks = p >> 1, h = 2 * (p & 1);
+            A[0][ks][h] = digit_pair<0>(a0, a1); A[0][ks][h + 1] = digit_pair<0>(b0, b1);
+            A[1][ks][h] = digit_pair<1>(a0, a1); A[1][ks][h + 1] = digit_pair<1>(b0, b1);
+            A[2][ks][h] = digit_pair<2>(a0, a1); A[2][ks][h + 1] = digit_pair<2>(b0, b1);
+            A[3][ks][h] = digit_pair<3>(a0, a1); A[3][ks][h + 1] = digit_pair<3>(b0, b1);
+            A[4][ks][h] = digit_pair<4>(a0, a1); A[4][ks][h + 1] = digit_pair<4>(b0, b1);
+            A[5][ks][h] = digit_pair<5>(a0, a1); A[5][ks][h + 1] = digit_pair<5>(b0, b1);
+        }
+    }
+    __syncwarp();
+    for (int nt = 0; nt < 4; ++nt) {
+        float acc[kWeights][4];
+#pragma unroll
+        for (int o = 0; o < kWeights; ++o)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[o][i] = 0.f;
+#pragma unroll
+        for (int j = 0; j < kDigits; ++j) {
+            const uint2 b0 = Jd[(j * 8 + nt) * 32 + lane], b1 = Jd[(j * 8 + 4 + nt) * 32 + lane];
+#pragma unroll
+            for (int i = 0; i < kDigits; ++i) {
+                if (i + j >= kWeights) continue;
+                mma_f16(acc[i + j], A[i][0], b0.x, b0.y);
+                mma_f16(acc[i + j], A[i][1], b1.x, b1.y);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float c[kWeights];
+#pragma unroll
+            for (int o = 0; o < kWeights; ++o) c[o] = acc[o][i];
+            const int cc = 8 * nt + 2 * t + (i & 1), r = i < 2 ? ra : rb;
+            // x = int 2^(E - 1075), J = int 2^(f - 1075), the integers' product T 2^51
+            const double y = fixed_to_f64(combine_weights(c), (i < 2 ? Ea : Eb) + fc[cc] - 2150 + 51);
+            if (r < rows) X[r + col(cc)] = y;
+        }
+    }
+}
+
+// S4/S5: [W_i W_j] <- [W_i W_j] J for rowsW rows of W (its columns scaled by
+// their exponents ek) and [V_i V_j] <- [V_i V_j] J for rowsV rows of V (0: V not
+// kept; unscaled), 16-row tiles tile0, tile0 + step .. dealt to the group's
+// warps.  Jd: kJDigitBytes, fc: 32 ints, both in shared memory.
+template <int GT>
+__device__ __forceinline__ void update_f64_split(double* W, long long ldw, int rowsW, double* V, long long ldv, int rowsV,
+                                                 int cbi, int cbj, const double* J, int ldj, const int* ek, uint2* Jd,
+                                                 int* fc, int gt, int bar, int block = 0, int blocks = 1) {
+    constexpr int NWG = GT / 32;
+    const int warp = gt >> 5, lane = gt & 31, tw = (rowsW + 15) / 16, tv = (rowsV + 15) / 16, step = NWG * blocks;
+    if (block * NWG < tw) {
+        j_digits_f64<GT>(J, ldj, ek, Jd, fc, gt);
+        named_sync(bar, GT);
+        for (int t = block * NWG + warp; t < tw; t += step)
+            update_rows_f64(W, ldw, rowsW, 16 * t, cbi, cbj, ek, Jd, fc, lane);
+    }
+    if (block * NWG < tv) {
+        named_sync(bar, GT);
+        j_digits_f64<GT>(J, ldj, nullptr, Jd, fc, gt);
+        named_sync(bar, GT);
+        for (int t = block * NWG + warp; t < tv; t += step)
+            update_rows_f64(V, ldv, rowsV, 16 * t, cbi, cbj, nullptr, Jd, fc, lane);
+    }
+}
+
+}  // namespace bsvd
