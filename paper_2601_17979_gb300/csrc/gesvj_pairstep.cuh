@@ -93,14 +93,7 @@ __global__ void __launch_bounds__(kPairThreads, pair_min_blocks<T>()) blk_pairst
                 for (int i = 0; i < 4; ++i) re[h][j][i] = im[h][j][i] = 0.f;
         // chunk k0 of the pair's columns into buffer `buf` (rows past M as zeros)
         auto stage = [&](int buf, int k0) {
-            const int kc = min(KC, M - k0);
-            T* Pb = P + buf * (L::kChunk / (int)sizeof(T));
-            for (int e = tid; e < KC * TWO; e += NT) {
-                const int kk = e % KC, c = e / KC;
-                const int col = c < NB ? bi * NB + c : bj * NB + (c - NB);
-                cp_async<(int)sizeof(T)>(Pb + kk + c * KP, Wm + k0 + (kk < kc ? kk : 0) + (long long)col * M,
-                                         kk < kc ? (int)sizeof(T) : 0);
-            }
+            stage_panel<T, NB, KC, KP, NT>(P + buf * (L::kChunk / (int)sizeof(T)), Wm, M, k0, bi, bj, tid);
             cp_async_commit();
         };
         stage(0, 0);
@@ -174,15 +167,14 @@ __global__ void __launch_bounds__(kPairThreads, pair_min_blocks<T>()) blk_pairst
     if constexpr (kCplx) jc_fragments<NB, NT, LDG>(J, Jf, tid);
     else                 j_fragments<NB, NT, LDG>(J, Jf, tid);
     __syncthreads();
-    const int tw = (sh.M + 15) / 16, tt = tw + (sh.N + 15) / 16;
-    for (int tile = warp; tile < tt; tile += NW) {
-        if constexpr (kCplx) {
+    if constexpr (kCplx) {
+        const int tw = (sh.M + 15) / 16, tt = tw + (sh.N + 15) / 16;
+        for (int tile = warp; tile < tt; tile += NW) {
             if (tile < tw) update_rows_c64_mma<NB>(Wm, sh.M, sh.M, 16 * tile, bi * NB, bj * NB, Jf, lane);
             else           update_rows_c64_mma<NB>(Vm, sh.N, sh.N, 16 * (tile - tw), bi * NB, bj * NB, Jf, lane);
-        } else {
-            if (tile < tw) update_rows_mma<NB>(Wm, sh.M, sh.M, 16 * tile, bi * NB, bj * NB, Jf, lane);
-            else           update_rows_mma<NB>(Vm, sh.N, sh.N, 16 * (tile - tw), bi * NB, bj * NB, Jf, lane);
         }
+    } else {
+        update_f32_rows<NB>(Wm, sh.M, sh.M, Vm, sh.N, sh.N, bi * NB, bj * NB, Jf, warp, NW, lane);
     }
 }
 
