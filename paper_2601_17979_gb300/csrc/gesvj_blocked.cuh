@@ -25,7 +25,7 @@
 
 namespace bsvd {
 
-enum : int { kBlkThreads = 256, kUpdRows = 128, kGramChunk = 64, kPairGramThreads = 128 };
+enum : int { kBlkThreads = 256, kUpdRows = 128, kGramChunk = 64 };
 
 __device__ __forceinline__ int blk_mid(const BlockedArgs& a, int b) { return a.index ? a.index[b] : b; }
 
@@ -398,11 +398,12 @@ __global__ void __launch_bounds__(kBlkThreads) blk_gram(const BlockedArgs a, int
     }
 }
 
-// ---- S2, real FP64, nb = 16: exact digit products on the tensor cores ------------
+// ---- S2, real FP64, nb = 8, 16: exact digit products on the tensor cores ------------
 // (tc_f64.cuh).  The FP64 pipe bounds blk_gram (95 % busy, 206 us a round for
 // 64 matrices of 256 x 256); here it only adds a few partial sums.
-static __global__ void __launch_bounds__(kPairGramThreads) blk_gram_f64_tc(const BlockedArgs a, int r) {
-    constexpr int NB = 16, TWO = 2 * NB;
+template <int NB>
+__global__ void __launch_bounds__(8 * NB) blk_gram_f64_tc(const BlockedArgs a, int r) {
+    constexpr int TWO = 2 * NB, NT = 8 * NB;
     __shared__ int ec[TWO];
     __shared__ double Gs[TWO * (TWO + 1)];
     const int b = blockIdx.x, q = blockIdx.y, tid = threadIdx.x;
@@ -411,11 +412,11 @@ static __global__ void __launch_bounds__(kPairGramThreads) blk_gram_f64_tc(const
     int bi, bj;
     if (!blk_pair(sh, r, q, bi, bj)) return;
     const double* W = static_cast<const double*>(a.W) + sh.oW;
-    column_exponents_f64<kPairGramThreads>(W, sh.M, sh.M, bi * NB, bj * NB, ec, tid);
+    column_exponents_f64<NB, NT>(W, sh.M, sh.M, bi * NB, bj * NB, ec, tid);
     __syncthreads();
-    gram_f64_split<kPairGramThreads, TWO + 1>(W, sh.M, sh.M, bi * NB, bj * NB, ec, Gs, tid, 1);
+    gram_f64_split<NB, NT, TWO + 1>(W, sh.M, sh.M, bi * NB, bj * NB, ec, Gs, tid, 1);
     double* G = static_cast<double*>(a.G) + sh.oG + (long long)q * TWO * TWO;
-    for (int e = tid; e < TWO * TWO; e += kPairGramThreads) G[e] = Gs[e % TWO + (e / TWO) * (TWO + 1)];
+    for (int e = tid; e < TWO * TWO; e += NT) G[e] = Gs[e % TWO + (e / TWO) * (TWO + 1)];
 }
 
 // ---- S3: the Hermitian eigensolver on each Gram block --------------------------
@@ -478,7 +479,8 @@ __global__ void __launch_bounds__(kUpdRows) blk_update_fused(const BlockedArgs a
     int bi, bj;
     if (!blk_pair(sh, r, q, bi, bj)) return;
     const int rows = sh.M + sh.N;
-    if (!(std::is_same<T, double>::value && NB == 16) && blockIdx.z * kUpdRows >= rows) return;
+    constexpr bool kSplit = std::is_same<T, double>::value && (NB == 8 || NB == 16);
+    if (!kSplit && blockIdx.z * kUpdRows >= rows) return;
     const T* Jg = static_cast<const T*>(a.J) + sh.oJ + (long long)q * TWO * TWO;
     if constexpr (std::is_same<T, float>::value && (NB == 8 || NB == 16))
       if (!(a.flags & 128)) {
@@ -515,18 +517,17 @@ __global__ void __launch_bounds__(kUpdRows) blk_update_fused(const BlockedArgs a
             }
         return;
       }
-    if constexpr (std::is_same<T, double>::value && NB == 16) {
+    if constexpr (kSplit) {
         // real FP64: exact digit products on the tensor cores (tc_f64.cuh);
         // a CTA's four warps take the 16-row tiles of its share of W, then of V.
         // On the FP64 pipe this update ran at 93 % of it: 480 us a round for
         // 64 matrices of 256 x 256.
         uint2* Jd = reinterpret_cast<uint2*>(smem_js);
-        int* ek = reinterpret_cast<int*>(smem_js + kJDigitBytes);
+        int* ek = reinterpret_cast<int*>(smem_js + j_digit_bytes<NB>());
         const double* Gg = static_cast<const double*>(a.G) + sh.oG + (long long)q * TWO * TWO;
-        // exponents of the columns' norms (of 2^-511 where the square underflows)
-        if (tid < TWO) ek[tid] = (max(exp_f64(Gg[tid + tid * TWO]), 1) + 1023) / 2;
+        if (tid < TWO) ek[tid] = norm_exponent_f64(Gg[tid + tid * TWO]);
         __syncthreads();
-        update_f64_split<kUpdRows>(static_cast<double*>(a.W) + sh.oW, sh.M, sh.M, static_cast<double*>(a.Vw) + sh.oV, sh.N,
+        update_f64_split<NB, kUpdRows>(static_cast<double*>(a.W) + sh.oW, sh.M, sh.M, static_cast<double*>(a.Vw) + sh.oV, sh.N,
                                    sh.N, bi * NB, bj * NB, Jg, TWO, ek, Jd, ek + TWO, tid, 1, blockIdx.z, gridDim.z);
         return;
     }

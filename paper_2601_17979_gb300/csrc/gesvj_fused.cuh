@@ -95,20 +95,20 @@ __host__ __device__ inline long long fused_slot_elems(const FusedArgs& a) {
     return w + (long long)a.ldvs * a.Np;
 }
 
-// Real FP64 with nb = 16 forms the Gram block and the update as exact digit
+// Real FP64 with nb = 8 or 16 forms the Gram block and the update as exact digit
 // products on the tensor cores (tc_f64.cuh).
 template <class T, int NB>
-__host__ __device__ constexpr bool fused_split() { return std::is_same<T, double>::value && NB == 16; }
+__host__ __device__ constexpr bool fused_split() { return std::is_same<T, double>::value && NB >= 8; }
 
 // FP32 adds J as split-TF32 fragments for the tensor-core update (nb >= 8:
 // 8 (2nb)^2 bytes) or J^T for the FFMA-tiled update (nb = 4), 16-byte
-// aligned; FP64 with nb = 16 J's digits, in the place of G once the inner sweep
+// aligned; FP64 with nb >= 8 J's digits, in the place of G once the inner sweep
 // is done, and two sets of column exponents; the others a second J (the
 // previous pair's, for the deferred V update).
 template <class T, int NB>
 __host__ __device__ constexpr int fused_group_bytes() {
     constexpr int mat = (2 * NB) * (2 * NB + 1) * (int)sizeof(T);
-    if (fused_split<T, NB>()) return ((mat + InnerTables<T, NB>::bytes() + 15) & ~15) + kJDigitBytes + 256;
+    if (fused_split<T, NB>()) return ((mat + InnerTables<T, NB>::bytes() + 15) & ~15) + j_digit_bytes<NB>() + 16 * NB;
     return ((2 * mat + InnerTables<T, NB>::bytes() + 15) & ~15) +
            (std::is_same<T, float>::value ? (NB >= 8 ? 8 * (2 * NB) * (2 * NB) : (2 * NB) * (2 * NB) * 4)
                                           : ((mat + 15) & ~15));
@@ -198,7 +198,7 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
 
     unsigned char* gb = smem + a.offG + g * a.groupBytes;
     // G, J and the rotation tables; then, 16-byte aligned, J^T or J's fragments
-    // for FP32, or the second J buffer of the other types.  FP64 with nb = 16: J,
+    // for FP32, or the second J buffer of the other types.  FP64 with nb >= 8: J,
     // the tables, then G, whose place J's digits take, and the exponents.
     constexpr bool kSplit = fused_split<T, NB>();
     constexpr int kMats = kSplit ? 1 : 2;
@@ -206,7 +206,7 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
     const InnerTables<T, NB> tb(J0 + TWO * LDG);
     unsigned char* const gb_tail = gb + ((kMats * TWO * LDG * (int)sizeof(T) + InnerTables<T, NB>::bytes() + 15) & ~15);
     T* const G = reinterpret_cast<T*>(kSplit ? gb_tail : gb);
-    int* const ek = reinterpret_cast<int*>(gb_tail + kJDigitBytes);   // [32] column exponents, then [32] J's (kSplit)
+    int* const ek = reinterpret_cast<int*>(gb_tail + j_digit_bytes<NB>());   // [2nb] column exponents, [2nb] J's (kSplit)
     float* Jt = reinterpret_cast<float*>(gb_tail);
     T* const J1 = reinterpret_cast<T*>(gb_tail);
     T* J = J0;
@@ -337,9 +337,10 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
                     if (NB >= 8 && !(a.flags & kFlagF32Ffma)) gram_f32_mma<NB < 8 ? 8 : NB, GT>(W, ldw, M, bi * NB, bj * NB, G, gt);
                     else gram_f32_tiled<NB, GT>(W, ldw, M, bi * NB, bj * NB, G, gt);
                 } else if constexpr (kSplit) {
-                    column_exponents_f64<GT>(W, ldw, M, bi * NB, bj * NB, ek, gt);
+                    column_exponents_f64<NB, GT>(W, ldw, M, bi * NB, bj * NB, ek, gt);
                     group_sync(g, GT);
-                    gram_f64_split<GT, LDG>(W, ldw, M, bi * NB, bj * NB, ek, G, gt, g + 1);
+                    gram_f64_split<NB, GT, LDG>(W, ldw, M, bi * NB, bj * NB, ek, G, gt, g + 1);
+                    if (gt < TWO) ek[gt] = norm_exponent_f64(G[gt + gt * LDG]);   // for the update
                 } else if constexpr (!OnChip) {
                     // W in global memory: 2 x 2 tiles of upper entries per lane
                     // pair, four independent sums (half the loads per FMA of
@@ -453,8 +454,8 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
                         update_f32_tiled<NB, GT, 2>(W, ldw, pre ? (M + 3) & ~3 : ldw, Vs, ldvs, needVs ? ldvs : 0, bi * NB, bj * NB, Jt, gt, g + 1);
                     }
                 } else if constexpr (kSplit) {
-                    update_f64_split<GT>(W, ldw, M, Vs, ldvs, needVs ? N : 0, bi * NB, bj * NB, J, LDG, ek,
-                                         reinterpret_cast<uint2*>(gb_tail), ek + 32, gt, g + 1);
+                    update_f64_split<NB, GT>(W, ldw, M, Vs, ldvs, needVs ? N : 0, bi * NB, bj * NB, J, LDG, ek,
+                                         reinterpret_cast<uint2*>(gb_tail), ek + TWO, gt, g + 1);
                 } else if constexpr (std::is_same<T, float2>::value) {
                     // complex64: 4 rows x 2nb/8 columns per lane (columns
                     // cg, cg + 8, ...: conflict-free J reads with its padded

@@ -98,15 +98,16 @@ __device__ __forceinline__ double fixed_to_f64(long long T, int s) {
     return __longlong_as_double((long long)(r | ((unsigned long long)T & 0x8000000000000000ull)));
 }
 
-// Largest biased exponent of each of the 32 columns of a panel (columns [cbi,
-// cbi + 16) and [cbj, cbj + 16) of W, M rows) into ec.  GT threads (a multiple of
-// 32); the caller synchronises.
-template <int GT>
+// Largest biased exponent of each of the 2 NB columns of a panel (columns [cbi,
+// cbi + NB) and [cbj, cbj + NB) of W, M rows) into ec.  GT threads (a multiple of
+// 2 NB); the caller synchronises.
+template <int NB, int GT>
 __device__ __forceinline__ void column_exponents_f64(const double* W, long long ldw, int M, int cbi, int cbj, int* ec,
                                                      int gt) {
-    constexpr int P = GT / 32;                             // threads a column
+    constexpr int P = GT / (2 * NB);                       // threads a column
+    static_assert(P >= 1 && P <= 32 && (P & (P - 1)) == 0, "threads a column");
     const int c = gt / P, q = gt % P;
-    const double* x = W + (c < 16 ? cbi + c : cbj + c - 16) * ldw;
+    const double* x = W + (c < NB ? cbi + c : cbj + c - NB) * ldw;
     int e = kNoExp;
     for (int r = q; r < M; r += P) e = max(e, exp_f64(x[r]));
 #pragma unroll
@@ -114,33 +115,35 @@ __device__ __forceinline__ void column_exponents_f64(const double* W, long long 
     if (q == 0) ec[c] = e;
 }
 
-// S2: G = P^T P (32 x 32, column stride LDG) for the panel P of column_exponents.
-// Four warps take 16 rows in turn (always four: the bits do not depend on the
-// group's size); each forms the six 16 x 8 tiles that meet the
-// upper triangle from one set of digits (a column's digits serve as A and as B
+// S2: G = P^T P (2 NB x 2 NB, column stride LDG) for the panel P of
+// column_exponents.  Four warps (NB = 8: two) take 16 rows in turn, whatever the
+// group's size, so that the bits do not depend on it; each forms the 16 x 8
+// tiles that meet the upper triangle from one set of digits (a column's digits serve as A and as B
 // fragment), converts them to FP64 and sums its own; the warps' sums are added
 // in warp order.  Upper entries are written and mirrored.  GT threads, named
 // barrier `bar`; synchronised on return.
-template <int GT, int LDG>
+template <int NB, int GT, int LDG>
 __device__ __forceinline__ void gram_f64_split(const double* W, long long ldw, int M, int cbi, int cbj, const int* ec,
                                                double* G, int gt, int bar) {
+    constexpr int NBM = 2 * NB / 16, NTL = NBM == 2 ? 6 : 2, NWS = NBM == 2 ? 4 : 2;
+    static_assert(NB == 8 || NB == 16, "one or two blocks of 16 columns");
+    static_assert(GT >= 32 * NWS, "the summing warps");
     const int warp = gt >> 5, lane = gt & 31, g = lane >> 2, t = lane & 3;
-    double sum[6][4];
+    auto col = [&](int c) { return (c < NB ? cbi + c : cbj + c - NB) * ldw; };
+    double sum[NTL][4];
 #pragma unroll
-    for (int u = 0; u < 6; ++u)
+    for (int u = 0; u < NTL; ++u)
 #pragma unroll
         for (int i = 0; i < 4; ++i) sum[u][i] = 0.0;
-    constexpr int NWS = 4;
-    static_assert(GT >= 32 * NWS, "four warps");
     for (int k0 = warp < NWS ? 16 * warp : M; k0 < M; k0 += 16 * NWS) {
-        uint32_t D[kDigits][2][4];
+        uint32_t D[kDigits][NBM][4];
 #pragma unroll
-        for (int bm = 0; bm < 2; ++bm)
+        for (int bm = 0; bm < NBM; ++bm)
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                const int c = 8 * h + g;
-                const double* x = W + ((bm ? cbj : cbi) + c) * ldw;
-                const int E = ec[16 * bm + c];
+                const int c = 16 * bm + 8 * h + g;
+                const double* x = W + col(c);
+                const int E = ec[c];
                 unsigned long long v[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
@@ -156,7 +159,7 @@ __device__ __forceinline__ void gram_f64_split(const double* W, long long ldw, i
                 D[5][bm][h] = digit_pair<5>(v[0], v[1]); D[5][bm][2 + h] = digit_pair<5>(v[2], v[3]);
             }
 #pragma unroll
-        for (int u = 0; u < 6; ++u) {
+        for (int u = 0; u < NTL; ++u) {
             const int bm = u < 4 ? 0 : 1, nt = u < 4 ? u : u - 2, bn = nt >> 1, h = nt & 1;
             float acc[kWeights][4];
 #pragma unroll
@@ -181,7 +184,7 @@ __device__ __forceinline__ void gram_f64_split(const double* W, long long ldw, i
     for (int w = 0; w < NWS; ++w) {
         if (warp == w) {
 #pragma unroll
-            for (int u = 0; u < 6; ++u)
+            for (int u = 0; u < NTL; ++u)
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const int bm = u < 4 ? 0 : 1, nt = u < 4 ? u : u - 2;
@@ -196,20 +199,27 @@ __device__ __forceinline__ void gram_f64_split(const double* W, long long ldw, i
     }
 }
 
-// J (32 x 32, column stride ldj) for the update of columns scaled by 2^-ek[k]
+// Exponents of the columns' norms from the Gram block's diagonal (of 2^-511
+// where the square underflows): the scales of the update.
+__device__ __forceinline__ int norm_exponent_f64(double gkk) { return (max(exp_f64(gkk), 1) + 1023) / 2; }
+
+// J (2 NB x 2 NB, column stride ldj) for the update of columns scaled by 2^-ek[k]
 // (ek null: unscaled): B fragments of the digits of J_kc 2^(ek[k] - fc[c]), fc[c]
-// the largest exponent of column c.  Jd[((d * 2 + ks) * 4 + nt) * 32 + lane]:
-// 12 KB.  GT threads; the caller synchronises.
-constexpr int kJDigitBytes = kDigits * 2 * 4 * 32 * 8;
-template <int GT>
+// the largest exponent of column c.  Jd[((d * KS + ks) * NT + nt) * 32 + lane], KS
+// = NB / 8 steps of 16, NT = NB / 4 tiles of 8 columns: 12 KB (NB = 8: 3 KB).  GT
+// threads; the caller synchronises.
+template <int NB>
+__host__ __device__ constexpr int j_digit_bytes() { return kDigits * (NB / 8) * (NB / 4) * 32 * 8; }
+template <int NB, int GT>
 __device__ __forceinline__ void j_digits_f64(const double* J, int ldj, const int* ek, uint2* Jd, int* fc, int gt) {
     const int warp = gt >> 5, lane = gt & 31, g = lane >> 2, t = lane & 3;
-    for (int nt = warp; nt < 4; nt += GT / 32) {
+    constexpr int KS = NB / 8, NT = NB / 4;
+    for (int nt = warp; nt < NT; nt += GT / 32) {
         const int c = 8 * nt + g;
-        double x[8];
-        int e[8], f = kNoExp;
+        double x[4 * KS];
+        int e[4 * KS], f = kNoExp;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < 4 * KS; ++i) {
             const int k = 16 * (i >> 2) + 2 * t + (i & 1) + 8 * ((i >> 1) & 1);
             x[i] = J[k + c * ldj];
             e[i] = exp_f64(x[i]) + (ek ? ek[k] : 0);
@@ -218,37 +228,39 @@ __device__ __forceinline__ void j_digits_f64(const double* J, int ldj, const int
         f = max(f, __shfl_xor_sync(0xffffffffu, f, 1));
         f = max(f, __shfl_xor_sync(0xffffffffu, f, 2));
         if (t == 0) fc[c] = f;
-        unsigned long long v[8];
+        unsigned long long v[4 * KS];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) v[i] = fixed_f64(x[i], f - e[i]);
+        for (int i = 0; i < 4 * KS; ++i) v[i] = fixed_f64(x[i], f - e[i]);
 #pragma unroll
-        for (int ks = 0; ks < 2; ++ks) {
-            uint2* o = Jd + (ks * 4 + nt) * 32 + lane;
-            o[0 * 256] = make_uint2(digit_pair<0>(v[4 * ks], v[4 * ks + 1]), digit_pair<0>(v[4 * ks + 2], v[4 * ks + 3]));
-            o[1 * 256] = make_uint2(digit_pair<1>(v[4 * ks], v[4 * ks + 1]), digit_pair<1>(v[4 * ks + 2], v[4 * ks + 3]));
-            o[2 * 256] = make_uint2(digit_pair<2>(v[4 * ks], v[4 * ks + 1]), digit_pair<2>(v[4 * ks + 2], v[4 * ks + 3]));
-            o[3 * 256] = make_uint2(digit_pair<3>(v[4 * ks], v[4 * ks + 1]), digit_pair<3>(v[4 * ks + 2], v[4 * ks + 3]));
-            o[4 * 256] = make_uint2(digit_pair<4>(v[4 * ks], v[4 * ks + 1]), digit_pair<4>(v[4 * ks + 2], v[4 * ks + 3]));
-            o[5 * 256] = make_uint2(digit_pair<5>(v[4 * ks], v[4 * ks + 1]), digit_pair<5>(v[4 * ks + 2], v[4 * ks + 3]));
+        for (int ks = 0; ks < KS; ++ks) {
+            uint2* o = Jd + (ks * NT + nt) * 32 + lane;
+            o[0 * KS * NT * 32] = make_uint2(digit_pair<0>(v[4 * ks], v[4 * ks + 1]), digit_pair<0>(v[4 * ks + 2], v[4 * ks + 3]));
+            o[1 * KS * NT * 32] = make_uint2(digit_pair<1>(v[4 * ks], v[4 * ks + 1]), digit_pair<1>(v[4 * ks + 2], v[4 * ks + 3]));
+            o[2 * KS * NT * 32] = make_uint2(digit_pair<2>(v[4 * ks], v[4 * ks + 1]), digit_pair<2>(v[4 * ks + 2], v[4 * ks + 3]));
+            o[3 * KS * NT * 32] = make_uint2(digit_pair<3>(v[4 * ks], v[4 * ks + 1]), digit_pair<3>(v[4 * ks + 2], v[4 * ks + 3]));
+            o[4 * KS * NT * 32] = make_uint2(digit_pair<4>(v[4 * ks], v[4 * ks + 1]), digit_pair<4>(v[4 * ks + 2], v[4 * ks + 3]));
+            o[5 * KS * NT * 32] = make_uint2(digit_pair<5>(v[4 * ks], v[4 * ks + 1]), digit_pair<5>(v[4 * ks + 2], v[4 * ks + 3]));
         }
     }
 }
 
 // Rows [r0, r0 + 16) of a column-major X (rows valid below `rows`), columns
-// [cbi, cbi + 16) and [cbj, cbj + 16), times J in place, with the fragments of
+// [cbi, cbi + NB) and [cbj, cbj + NB), times J in place, with the fragments of
 // j_digits_f64 for the same ek.  One warp; it reads all its inputs before it
 // writes any output, and no other warp touches these rows.
+template <int NB>
 __device__ __forceinline__ void update_rows_f64(double* X, long long ld, int rows, int r0, int cbi, int cbj, const int* ek,
                                                 const uint2* Jd, const int* fc, int lane) {
     const int g = lane >> 2, t = lane & 3, ra = r0 + g, rb = r0 + g + 8;
-    auto col = [&](int c) { return (long long)(c < 16 ? cbi + c : cbj + c - 16) * ld; };
-    uint32_t A[kDigits][2][4];
+    constexpr int KS = NB / 8, NT = NB / 4;
+    auto col = [&](int c) { return (long long)(c < NB ? cbi + c : cbj + c - NB) * ld; };
+    uint32_t A[kDigits][KS][4];
     int Ea = kNoExp, Eb = kNoExp;
     {
-        double x[2][8];                                    // [row][entry]
-        int e[2][8];
+        double x[2][4 * KS];                               // [row][entry]
+        int e[2][4 * KS];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < 4 * KS; ++i) {
             const int k = 16 * (i >> 2) + 2 * t + (i & 1) + 8 * ((i >> 1) & 1);
             const long long o = col(k);
             x[0][i] = ra < rows ? X[ra + o] : 0.0;
@@ -266,7 +278,7 @@ __device__ __forceinline__ void update_rows_f64(double* X, long long ld, int row
         Ea = max(Ea, __shfl_xor_sync(0xffffffffu, Ea, 2));
         Eb = max(Eb, __shfl_xor_sync(0xffffffffu, Eb, 2));
 #pragma unroll
-        for (int p = 0; p < 4; ++p) {                      // entry pairs (2p, 2p + 1): k-step p / 2, half p % 2
+        for (int p = 0; p < 2 * KS; ++p) {                 // entry pairs (2p, 2p + 1): k-step p / 2, half p % 2
             const unsigned long long a0 = fixed_f64(x[0][2 * p], Ea - e[0][2 * p]), a1 = fixed_f64(x[0][2 * p + 1], Ea - e[0][2 * p + 1]);
             const unsigned long long b0 = fixed_f64(x[1][2 * p], Eb - e[1][2 * p]), b1 = fixed_f64(x[1][2 * p + 1], Eb - e[1][2 * p + 1]);
             const int ks = p >> 1, h = 2 * (p & 1);
@@ -279,7 +291,7 @@ __device__ __forceinline__ void update_rows_f64(double* X, long long ld, int row
         }
     }
     __syncwarp();
-    for (int nt = 0; nt < 4; ++nt) {
+    for (int nt = 0; nt < NT; ++nt) {
         float acc[kWeights][4];
 #pragma unroll
         for (int o = 0; o < kWeights; ++o)
@@ -287,12 +299,14 @@ __device__ __forceinline__ void update_rows_f64(double* X, long long ld, int row
             for (int i = 0; i < 4; ++i) acc[o][i] = 0.f;
 #pragma unroll
         for (int j = 0; j < kDigits; ++j) {
-            const uint2 b0 = Jd[(j * 8 + nt) * 32 + lane], b1 = Jd[(j * 8 + 4 + nt) * 32 + lane];
+            uint2 bj[KS];
+#pragma unroll
+            for (int ks = 0; ks < KS; ++ks) bj[ks] = Jd[((j * KS + ks) * NT + nt) * 32 + lane];
 #pragma unroll
             for (int i = 0; i < kDigits; ++i) {
                 if (i + j >= kWeights) continue;
-                mma_f16(acc[i + j], A[i][0], b0.x, b0.y);
-                mma_f16(acc[i + j], A[i][1], b1.x, b1.y);
+#pragma unroll
+                for (int ks = 0; ks < KS; ++ks) mma_f16(acc[i + j], A[i][ks], bj[ks].x, bj[ks].y);
             }
         }
 #pragma unroll
@@ -311,25 +325,25 @@ __device__ __forceinline__ void update_rows_f64(double* X, long long ld, int row
 // S4/S5: [W_i W_j] <- [W_i W_j] J for rowsW rows of W (its columns scaled by
 // their exponents ek) and [V_i V_j] <- [V_i V_j] J for rowsV rows of V (0: V not
 // kept; unscaled), 16-row tiles tile0, tile0 + step .. dealt to the group's
-// warps.  Jd: kJDigitBytes, fc: 32 ints, both in shared memory.
-template <int GT>
+// warps.  Jd: j_digit_bytes, fc: 2 NB ints, both in shared memory.
+template <int NB, int GT>
 __device__ __forceinline__ void update_f64_split(double* W, long long ldw, int rowsW, double* V, long long ldv, int rowsV,
                                                  int cbi, int cbj, const double* J, int ldj, const int* ek, uint2* Jd,
                                                  int* fc, int gt, int bar, int block = 0, int blocks = 1) {
     constexpr int NWG = GT / 32;
     const int warp = gt >> 5, lane = gt & 31, tw = (rowsW + 15) / 16, tv = (rowsV + 15) / 16, step = NWG * blocks;
     if (block * NWG < tw) {
-        j_digits_f64<GT>(J, ldj, ek, Jd, fc, gt);
+        j_digits_f64<NB, GT>(J, ldj, ek, Jd, fc, gt);
         named_sync(bar, GT);
         for (int t = block * NWG + warp; t < tw; t += step)
-            update_rows_f64(W, ldw, rowsW, 16 * t, cbi, cbj, ek, Jd, fc, lane);
+            update_rows_f64<NB>(W, ldw, rowsW, 16 * t, cbi, cbj, ek, Jd, fc, lane);
     }
     if (block * NWG < tv) {
         named_sync(bar, GT);
-        j_digits_f64<GT>(J, ldj, nullptr, Jd, fc, gt);
+        j_digits_f64<NB, GT>(J, ldj, nullptr, Jd, fc, gt);
         named_sync(bar, GT);
         for (int t = block * NWG + warp; t < tv; t += step)
-            update_rows_f64(V, ldv, rowsV, 16 * t, cbi, cbj, nullptr, Jd, fc, lane);
+            update_rows_f64<NB>(V, ldv, rowsV, 16 * t, cbi, cbj, nullptr, Jd, fc, lane);
     }
 }
 
