@@ -124,7 +124,7 @@ cudaError_t blk_run_nb(BlockedArgs a, void* work, cudaStream_t st, bool two_stag
     a.J = base;  base += (size_t)nJ;
     a.T = base;
 
-    constexpr bool kSplit = std::is_same<T, double>::value && (NB == 8 || NB == 16);   // tc_f64.cuh
+    constexpr bool kSplit = sizeof(R) == 8 && (NB == 8 || NB == 16);   // tc_f64.cuh
     const int heevj_smem = 2 * TWO * LDG * (int)sizeof(T) + InnerTables<T, NB>::bytes();
     const int fin_smem = (kBlkThreads / 32) * (int)sizeof(R) + 16 + 2 * (int)sizeof(T) +
                          a.N * ((int)sizeof(R) + 4) + 16;
@@ -132,7 +132,7 @@ cudaError_t blk_run_nb(BlockedArgs a, void* work, cudaStream_t st, bool two_stag
     const int upd_smem = std::max(TWO * (TWO + 1) * (int)sizeof(T),
                                   std::is_same<T, float>::value    ? j_fragment_bytes<NB>()
                                   : std::is_same<T, float2>::value ? jc_fragment_bytes<NB>()
-                                  : kSplit                         ? j_digit_bytes<NB <= 16 ? NB : 16>() + 2 * TWO * (int)sizeof(int) : 0);
+                                  : kSplit                         ? j_digit_bytes<T, NB <= 16 ? NB : 16>() + 2 * TWO * (int)sizeof(int) : 0);
     if ((e = allow_dynamic_smem<blk_heevj<T, NB, GT>>()) != cudaSuccess ||
         (e = allow_dynamic_smem<blk_finalize<T>>()) != cudaSuccess ||
         (e = allow_dynamic_smem<blk_update_fused<T, NB>>()) != cudaSuccess ||
@@ -182,7 +182,7 @@ cudaError_t blk_run_nb(BlockedArgs a, void* work, cudaStream_t st, bool two_stag
             }
             else if constexpr (kSplit) {
                 if (two_stage) blk_gram<T, NB><<<gpair, kBlkThreads, 0, s>>>(a, r);
-                else blk_gram_f64_tc<NB><<<gpair, 8 * NB, 0, s>>>(a, r);
+                else blk_gram_f64_tc<T, NB><<<gpair, 8 * NB, 0, s>>>(a, r);
             }
             else
                 blk_gram<T, NB><<<gpair, kBlkThreads, 0, s>>>(a, r);

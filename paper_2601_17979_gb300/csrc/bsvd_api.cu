@@ -211,7 +211,7 @@ bsvd_status plan_group(int max_smem, const TypeOps& ops, int m, int n, int count
     if (r.path == BSVD_PATH_FUSED || (r.path == BSVD_PATH_AUTO && !want_blocked_opts)) {
         if (fused_nb(r.nb)) {
             p.smem = ops.plan(r.nb, M, N, needVs, p.a, p.threads);
-            if (p.smem > 0 && p.smem <= (size_t)max_smem) {
+            if (p.smem > 0 && p.smem + p.a.spare <= (size_t)max_smem) {
                 FusedArgs& a = p.a;
                 a.m = m; a.n = n; a.trans = m < n; a.M = M; a.N = N;
                 a.wantU = wantU; a.wantV = wantV;

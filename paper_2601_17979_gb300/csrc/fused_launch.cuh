@@ -43,6 +43,7 @@ size_t fused_plan_nb(int M, int N, bool needVs, FusedArgs& a, int& nthreads) {
     a.offG = (int)off;
     a.groupBytes = fused_group_bytes<T, NB>();
     off += (size_t)ng * a.groupBytes;
+    a.spare = ng * fused_group_spare<T, NB>();
     a.offMisc = (int)off;
     const int NT = C::NG * C::GT, NW = NT / 32;
     off += kMaxSweeps * 4 + 16 + 2 * sizeof(T);

@@ -398,24 +398,24 @@ __global__ void __launch_bounds__(kBlkThreads) blk_gram(const BlockedArgs a, int
     }
 }
 
-// ---- S2, real FP64, nb = 8, 16: exact digit products on the tensor cores ------------
+// ---- S2, FP64 and complex128, nb = 8, 16: exact digit products on the tensor cores ------------
 // (tc_f64.cuh).  The FP64 pipe bounds blk_gram (95 % busy, 206 us a round for
 // 64 matrices of 256 x 256); here it only adds a few partial sums.
-template <int NB>
+template <class T, int NB>
 __global__ void __launch_bounds__(8 * NB) blk_gram_f64_tc(const BlockedArgs a, int r) {
     constexpr int TWO = 2 * NB, NT = 8 * NB;
     __shared__ int ec[TWO];
-    __shared__ double Gs[TWO * (TWO + 1)];
+    __shared__ T Gs[TWO * (TWO + 1)];
     const int b = blockIdx.x, q = blockIdx.y, tid = threadIdx.x;
     if (blk_skip(a, b)) return;
     const BlkShape sh = blk_shape(a, b);
     int bi, bj;
     if (!blk_pair(sh, r, q, bi, bj)) return;
-    const double* W = static_cast<const double*>(a.W) + sh.oW;
+    const T* W = static_cast<const T*>(a.W) + sh.oW;
     column_exponents_f64<NB, NT>(W, sh.M, sh.M, bi * NB, bj * NB, ec, tid);
     __syncthreads();
     gram_f64_split<NB, NT, TWO + 1>(W, sh.M, sh.M, bi * NB, bj * NB, ec, Gs, tid, 1);
-    double* G = static_cast<double*>(a.G) + sh.oG + (long long)q * TWO * TWO;
+    T* G = static_cast<T*>(a.G) + sh.oG + (long long)q * TWO * TWO;
     for (int e = tid; e < TWO * TWO; e += NT) G[e] = Gs[e % TWO + (e / TWO) * (TWO + 1)];
 }
 
@@ -479,7 +479,7 @@ __global__ void __launch_bounds__(kUpdRows) blk_update_fused(const BlockedArgs a
     int bi, bj;
     if (!blk_pair(sh, r, q, bi, bj)) return;
     const int rows = sh.M + sh.N;
-    constexpr bool kSplit = std::is_same<T, double>::value && (NB == 8 || NB == 16);
+    constexpr bool kSplit = sizeof(Real<T>) == 8 && (NB == 8 || NB == 16);
     if (!kSplit && blockIdx.z * kUpdRows >= rows) return;
     const T* Jg = static_cast<const T*>(a.J) + sh.oJ + (long long)q * TWO * TWO;
     if constexpr (std::is_same<T, float>::value && (NB == 8 || NB == 16))
@@ -518,16 +518,16 @@ __global__ void __launch_bounds__(kUpdRows) blk_update_fused(const BlockedArgs a
         return;
       }
     if constexpr (kSplit) {
-        // real FP64: exact digit products on the tensor cores (tc_f64.cuh);
+        // FP64, complex128: exact digit products on the tensor cores (tc_f64.cuh);
         // a CTA's four warps take the 16-row tiles of its share of W, then of V.
         // On the FP64 pipe this update ran at 93 % of it: 480 us a round for
         // 64 matrices of 256 x 256.
         uint2* Jd = reinterpret_cast<uint2*>(smem_js);
-        int* ek = reinterpret_cast<int*>(smem_js + j_digit_bytes<NB>());
-        const double* Gg = static_cast<const double*>(a.G) + sh.oG + (long long)q * TWO * TWO;
-        if (tid < TWO) ek[tid] = norm_exponent_f64(Gg[tid + tid * TWO]);
+        int* ek = reinterpret_cast<int*>(smem_js + j_digit_bytes<T, NB>());
+        const T* Gg = static_cast<const T*>(a.G) + sh.oG + (long long)q * TWO * TWO;
+        if (tid < TWO) ek[tid] = norm_exponent_f64(re(Gg[tid + tid * TWO]));
         __syncthreads();
-        update_f64_split<NB, kUpdRows>(static_cast<double*>(a.W) + sh.oW, sh.M, sh.M, static_cast<double*>(a.Vw) + sh.oV, sh.N,
+        update_f64_split<NB, kUpdRows>(static_cast<T*>(a.W) + sh.oW, sh.M, sh.M, static_cast<T*>(a.Vw) + sh.oV, sh.N,
                                    sh.N, bi * NB, bj * NB, Jg, TWO, ek, Jd, ek + TWO, tid, 1, blockIdx.z, gridDim.z);
         return;
     }

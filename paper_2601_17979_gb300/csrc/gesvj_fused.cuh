@@ -37,7 +37,7 @@ struct FusedArgs {
     int m, n;              // caller's shape
     int l, L, Np;          // l >= 2 real blocks, L = l + (l odd), Np = l * nb columns
     int ldw, ldvs, lde;    // shared-memory leading dimensions
-    int offW, offV, offG, offMisc, groupBytes;
+    int offW, offV, offG, offMisc, groupBytes, spare;
     // strided addressing (p* == nullptr) or pointer arrays
     const void* A; long long sA; int lda; const void* const* Ap; const int* ldap;
     const void* V0; long long sV0; int ldv0;   // initial V (N x N, by matrix id) or nullptr for I
@@ -95,10 +95,10 @@ __host__ __device__ inline long long fused_slot_elems(const FusedArgs& a) {
     return w + (long long)a.ldvs * a.Np;
 }
 
-// Real FP64 with nb = 8 or 16 forms the Gram block and the update as exact digit
-// products on the tensor cores (tc_f64.cuh).
+// FP64 and complex128 with nb = 8 or 16 form the Gram block and the update as
+// exact digit products on the tensor cores (tc_f64.cuh).
 template <class T, int NB>
-__host__ __device__ constexpr bool fused_split() { return std::is_same<T, double>::value && NB >= 8; }
+__host__ __device__ constexpr bool fused_split() { return sizeof(Real<T>) == 8 && NB >= 8; }
 
 // FP32 adds J as split-TF32 fragments for the tensor-core update (nb >= 8:
 // 8 (2nb)^2 bytes) or J^T for the FFMA-tiled update (nb = 4), 16-byte
@@ -108,10 +108,23 @@ __host__ __device__ constexpr bool fused_split() { return std::is_same<T, double
 template <class T, int NB>
 __host__ __device__ constexpr int fused_group_bytes() {
     constexpr int mat = (2 * NB) * (2 * NB + 1) * (int)sizeof(T);
-    if (fused_split<T, NB>()) return ((mat + InnerTables<T, NB>::bytes() + 15) & ~15) + j_digit_bytes<NB>() + 16 * NB;
+    if (fused_split<T, NB>()) return ((mat + InnerTables<T, NB>::bytes() + 15) & ~15) + j_digit_bytes<T, NB>() + 16 * NB;
     return ((2 * mat + InnerTables<T, NB>::bytes() + 15) & ~15) +
            (std::is_same<T, float>::value ? (NB >= 8 ? 8 * (2 * NB) * (2 * NB) : (2 * NB) * (2 * NB) * 4)
                                           : ((mat + 15) & ~15));
+}
+
+// Shared memory per group that a shape must leave free to run on chip: the
+// three matrices of the layout without digits, less what is in use.  The
+// shapes in between (N = 100..103 with V in FP64, 62..64 in complex128) fit,
+// but the multi-kernel path is the faster one for them: 1000 of 101x101 FP64
+// 64.2 ms there and 84.0 on chip, one 6.1 and 12.2 ms; 1000 of 86x86
+// complex128 without V 121 and 124 ms, one 8.4 and 16.8.
+template <class T, int NB>
+constexpr int fused_group_spare() {
+    constexpr int mat = (2 * NB) * (2 * NB + 1) * (int)sizeof(T);
+    constexpr int full = ((2 * mat + InnerTables<T, NB>::bytes() + 15) & ~15) + ((mat + 15) & ~15);
+    return fused_split<T, NB>() && full > fused_group_bytes<T, NB>() ? full - fused_group_bytes<T, NB>() : 0;
 }
 
 // The V update of a block pair, [V_i V_j] <- [V_i V_j] J, run by whole warps
@@ -206,7 +219,7 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
     const InnerTables<T, NB> tb(J0 + TWO * LDG);
     unsigned char* const gb_tail = gb + ((kMats * TWO * LDG * (int)sizeof(T) + InnerTables<T, NB>::bytes() + 15) & ~15);
     T* const G = reinterpret_cast<T*>(kSplit ? gb_tail : gb);
-    int* const ek = reinterpret_cast<int*>(gb_tail + j_digit_bytes<NB>());   // [2nb] column exponents, [2nb] J's (kSplit)
+    int* const ek = reinterpret_cast<int*>(gb_tail + j_digit_bytes<T, NB>());   // [2nb] column exponents, [2nb] J's (kSplit)
     float* Jt = reinterpret_cast<float*>(gb_tail);
     T* const J1 = reinterpret_cast<T*>(gb_tail);
     T* J = J0;
@@ -310,7 +323,7 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
     const R tol = (R)a.tol;
     int sw = 0;
     bool converged = false;
-    // Complex and narrow FP64 on chip: a pair's V update is deferred to the group's
+    // complex64, and FP64 and complex128 with nb = 4, on chip: a pair's V update is deferred to the group's
     // next pair step and run by the J-update warps during its inner sweep
     // (same arithmetic; the V blocks are read by nothing else in between).
     // Not with V in global memory: a warp reads one row of V, which in
@@ -340,7 +353,7 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
                     column_exponents_f64<NB, GT>(W, ldw, M, bi * NB, bj * NB, ek, gt);
                     group_sync(g, GT);
                     gram_f64_split<NB, GT, LDG>(W, ldw, M, bi * NB, bj * NB, ek, G, gt, g + 1);
-                    if (gt < TWO) ek[gt] = norm_exponent_f64(G[gt + gt * LDG]);   // for the update
+                    if (gt < TWO) ek[gt] = norm_exponent_f64(re(G[gt + gt * LDG]));   // for the update
                 } else if constexpr (!OnChip) {
                     // W in global memory: 2 x 2 tiles of upper entries per lane
                     // pair, four independent sums (half the loads per FMA of

@@ -2,7 +2,7 @@
 //
 // A GB300 SM retires about 1.6 FP64 multiply-adds a clock and 0.47 FP16
 // 16 x 8 x 16 tile products (2,048 multiply-adds each), so the Gram block and
-// the rotation update of real FP64 split every operand into digits that the
+// the rotation update of FP64 and complex128 split every operand into digits that the
 // FP16 units multiply exactly (the scheme of Ozaki, Ogita, Oishi and Rump,
 // "Error-free transformations of matrix multiplication by using fast routines
 // of matrix multiplication and its applications", Numer. Algorithms 59, 2012):
@@ -206,10 +206,12 @@ __device__ __forceinline__ int norm_exponent_f64(double gkk) { return (max(exp_f
 // J (2 NB x 2 NB, column stride ldj) for the update of columns scaled by 2^-ek[k]
 // (ek null: unscaled): B fragments of the digits of J_kc 2^(ek[k] - fc[c]), fc[c]
 // the largest exponent of column c.  Jd[((d * KS + ks) * NT + nt) * 32 + lane], KS
-// = NB / 8 steps of 16, NT = NB / 4 tiles of 8 columns: 12 KB (NB = 8: 3 KB).  GT
-// threads; the caller synchronises.
-template <int NB>
-__host__ __device__ constexpr int j_digit_bytes() { return kDigits * (NB / 8) * (NB / 4) * 32 * 8; }
+// = NB / 8 steps of 16, NT = NB / 4 tiles of 8 columns: 12 KB (NB = 8: 3 KB; complex:
+// twice that).  GT threads; the caller synchronises.
+template <class T, int NB>
+__host__ __device__ constexpr int j_digit_bytes() {
+    return (Traits<T>::kComplex ? 2 : 1) * kDigits * (NB / 8) * (NB / 4) * 32 * 8;
+}
 template <int NB, int GT>
 __device__ __forceinline__ void j_digits_f64(const double* J, int ldj, const int* ek, uint2* Jd, int* fc, int gt) {
     const int warp = gt >> 5, lane = gt & 31, g = lane >> 2, t = lane & 3;
@@ -322,13 +324,273 @@ __device__ __forceinline__ void update_rows_f64(double* X, long long ld, int row
     }
 }
 
+// ---- complex128 -----------------------------------------------------------------
+// The same with real and imaginary parts, one exponent for both:
+//   G = P^H P:  Re = Pr^T Pr + Pi^T Pi,  Im = Pr^T Pi - Pi^T Pr
+//   P J:        Re = Pr Jr - Pi Ji,      Im = Pr Ji + Pi Jr
+// Each real product has its own accumulators (two together could pass 2^24); the
+// two integers of a part are added before the one rounding.
+__device__ __forceinline__ int exp_c128(double2 x) { return max(exp_f64(x.x), exp_f64(x.y)); }
+// x's two parts relative to exponent E (each with its own distance to it)
+__device__ __forceinline__ unsigned long long fixed_part(double x, int E, int sc) { return fixed_f64(x, E - (exp_f64(x) - sc)); }
+
+template <int NB, int GT>
+__device__ __forceinline__ void column_exponents_f64(const double2* W, long long ldw, int M, int cbi, int cbj, int* ec,
+                                                     int gt) {
+    constexpr int P = GT / (2 * NB);
+    static_assert(P >= 1 && P <= 32 && (P & (P - 1)) == 0, "threads a column");
+    const int c = gt / P, q = gt % P;
+    const double2* x = W + (c < NB ? cbi + c : cbj + c - NB) * ldw;
+    int e = kNoExp;
+    for (int r = q; r < M; r += P) e = max(e, exp_c128(x[r]));
+#pragma unroll
+    for (int o = 1; o < P; o <<= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+    if (q == 0) ec[c] = e;
+}
+
+// the digits of four values (a fragment's two pairs) into words h and 2 + h
+template <int I = 0>
+__device__ __forceinline__ void digits4(const unsigned long long (&v)[4], uint32_t (&lo)[kDigits], uint32_t (&hi)[kDigits]) {
+    if constexpr (I < kDigits) {
+        lo[I] = digit_pair<I>(v[0], v[1]);
+        hi[I] = digit_pair<I>(v[2], v[3]);
+        digits4<I + 1>(v, lo, hi);
+    }
+}
+
+// acc <- all digit products of weight below kWeights of fragments A and B
+template <int KS>
+__device__ __forceinline__ void digit_products(float (&acc)[kWeights][4], const uint32_t (&A)[kDigits][KS][4],
+                                               const uint2* Bd, int bstride, int kstride, int lane) {
+#pragma unroll
+    for (int o = 0; o < kWeights; ++o)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[o][i] = 0.f;
+#pragma unroll
+    for (int j = 0; j < kDigits; ++j)
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks) {
+            const uint2 b = Bd[j * bstride + ks * kstride + lane];
+#pragma unroll
+            for (int i = 0; i < kDigits; ++i)
+                if (i + j < kWeights) mma_f16(acc[i + j], A[i][ks], b.x, b.y);
+        }
+}
+__device__ __forceinline__ long long combined(const float (&acc)[kWeights][4], int i) {
+    float c[kWeights];
+#pragma unroll
+    for (int o = 0; o < kWeights; ++o) c[o] = acc[o][i];
+    return combine_weights(c);
+}
+
+// One pass of the Gram block: the tiles of 16-row block BM (columns 8 nt, nt from
+// 2 BM on), as gram_f64_split.  Two passes keep a warp's sums in registers.
+template <int NB, int GT, int LDG, int BM>
+__device__ __forceinline__ void gram_c128_pass(const double2* W, long long ldw, int M, int cbi, int cbj, const int* ec,
+                                               double2* G, int gt, int bar) {
+    constexpr int NBM = 2 * NB / 16, NT0 = 2 * BM, NTL = 2 * (NBM - BM), NWS = NBM == 2 ? 4 : 2;
+    static_assert(GT >= 32 * NWS, "the summing warps");
+    const int warp = gt >> 5, lane = gt & 31, g = lane >> 2, t = lane & 3;
+    auto col = [&](int c) { return (c < NB ? cbi + c : cbj + c - NB) * ldw; };
+    double sr[NTL][4], si[NTL][4];
+#pragma unroll
+    for (int u = 0; u < NTL; ++u)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) sr[u][i] = si[u][i] = 0.0;
+    for (int k0 = warp < NWS ? 16 * warp : M; k0 < M; k0 += 16 * NWS) {
+        uint32_t Dr[kDigits][NBM - BM][4], Di[kDigits][NBM - BM][4];
+#pragma unroll
+        for (int bm = BM; bm < NBM; ++bm)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int c = 16 * bm + 8 * h + g, E = ec[c];
+                const double2* x = W + col(c);
+                unsigned long long vr[4], vi[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int r = k0 + 2 * t + (i & 1) + 8 * (i >> 1);
+                    const double2 y = r < M ? x[r] : make_double2(0.0, 0.0);
+                    vr[i] = fixed_part(y.x, E, 0);
+                    vi[i] = fixed_part(y.y, E, 0);
+                }
+                uint32_t lo[kDigits], hi[kDigits];
+                digits4(vr, lo, hi);
+#pragma unroll
+                for (int d = 0; d < kDigits; ++d) { Dr[d][bm - BM][h] = lo[d]; Dr[d][bm - BM][2 + h] = hi[d]; }
+                digits4(vi, lo, hi);
+#pragma unroll
+                for (int d = 0; d < kDigits; ++d) { Di[d][bm - BM][h] = lo[d]; Di[d][bm - BM][2 + h] = hi[d]; }
+            }
+        auto product = [&](float (&acc)[kWeights][4], const uint32_t (&A)[kDigits][NBM - BM][4],
+                           const uint32_t (&B)[kDigits][NBM - BM][4], int bn, int h) {
+#pragma unroll
+            for (int o = 0; o < kWeights; ++o)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) acc[o][i] = 0.f;
+#pragma unroll
+            for (int j = 0; j < kDigits; ++j)
+#pragma unroll
+                for (int i = 0; i < kDigits; ++i)
+                    if (i + j < kWeights) mma_f16(acc[i + j], A[i][0], B[j][bn][h], B[j][bn][2 + h]);
+        };
+#pragma unroll
+        for (int u = 0; u < NTL; ++u) {
+            const int nt = NT0 + u, bn = (nt >> 1) - BM, h = nt & 1;
+            float a1[kWeights][4], a2[kWeights][4];
+            product(a1, Dr, Dr, bn, h);
+            product(a2, Di, Di, bn, h);
+            int s[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int rr = 16 * BM + g + 8 * (i >> 1), cc = 8 * nt + 2 * t + (i & 1);
+                s[i] = ec[rr] + ec[cc] - 2150 + 51;
+                sr[u][i] += fixed_to_f64(combined(a1, i) + combined(a2, i), s[i]);
+            }
+            product(a1, Dr, Di, bn, h);
+            product(a2, Di, Dr, bn, h);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) si[u][i] += fixed_to_f64(combined(a1, i) - combined(a2, i), s[i]);
+        }
+    }
+    for (int w = 0; w < NWS; ++w) {
+        if (warp == w) {
+#pragma unroll
+            for (int u = 0; u < NTL; ++u)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int rr = 16 * BM + g + 8 * (i >> 1), cc = 8 * (NT0 + u) + 2 * t + (i & 1);
+                    if (rr > cc) continue;                 // lower entries: the mirror of an upper one
+                    double2 x = make_double2(sr[u][i], rr == cc ? 0.0 : si[u][i]);
+                    if (w) x = add(G[rr + cc * LDG], x);
+                    G[rr + cc * LDG] = x;
+                    G[cc + rr * LDG] = conj_s(x);
+                }
+        }
+        named_sync(bar, GT);
+    }
+}
+template <int NB, int GT, int LDG>
+__device__ __forceinline__ void gram_f64_split(const double2* W, long long ldw, int M, int cbi, int cbj, const int* ec,
+                                               double2* G, int gt, int bar) {
+    gram_c128_pass<NB, GT, LDG, 0>(W, ldw, M, cbi, cbj, ec, G, gt, bar);
+    if constexpr (NB == 16) gram_c128_pass<NB, GT, LDG, 1>(W, ldw, M, cbi, cbj, ec, G, gt, bar);
+}
+
+// Digits of Jr, then of Ji, each in the layout of the real form.
+template <int NB, int GT>
+__device__ __forceinline__ void j_digits_f64(const double2* J, int ldj, const int* ek, uint2* Jd, int* fc, int gt) {
+    constexpr int KS = NB / 8, NT = NB / 4, F = kDigits * KS * NT * 32;
+    const int warp = gt >> 5, lane = gt & 31, g = lane >> 2, t = lane & 3;
+    for (int nt = warp; nt < NT; nt += GT / 32) {
+        const int c = 8 * nt + g;
+        double2 x[4 * KS];
+        int sc[4 * KS], f = kNoExp;
+#pragma unroll
+        for (int i = 0; i < 4 * KS; ++i) {
+            const int k = 16 * (i >> 2) + 2 * t + (i & 1) + 8 * ((i >> 1) & 1);
+            x[i] = J[k + c * ldj];
+            sc[i] = ek ? -ek[k] : 0;
+            f = max(f, exp_c128(x[i]) - sc[i]);
+        }
+        f = max(f, __shfl_xor_sync(0xffffffffu, f, 1));
+        f = max(f, __shfl_xor_sync(0xffffffffu, f, 2));
+        if (t == 0) fc[c] = f;
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+            for (int part = 0; part < 2; ++part) {
+                unsigned long long v[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    v[i] = fixed_part(part ? x[4 * ks + i].y : x[4 * ks + i].x, f, sc[4 * ks + i]);
+                uint32_t lo[kDigits], hi[kDigits];
+                digits4(v, lo, hi);
+#pragma unroll
+                for (int d = 0; d < kDigits; ++d) Jd[part * F + ((d * KS + ks) * NT + nt) * 32 + lane] = make_uint2(lo[d], hi[d]);
+            }
+    }
+}
+
+template <int NB>
+__device__ __forceinline__ void update_rows_f64(double2* X, long long ld, int rows, int r0, int cbi, int cbj, const int* ek,
+                                                const uint2* Jd, const int* fc, int lane) {
+    constexpr int KS = NB / 8, NT = NB / 4, F = kDigits * KS * NT * 32;
+    const int g = lane >> 2, t = lane & 3, ra = r0 + g, rb = r0 + g + 8;
+    auto col = [&](int c) { return (long long)(c < NB ? cbi + c : cbj + c - NB) * ld; };
+    uint32_t Ar[kDigits][KS][4], Ai[kDigits][KS][4];
+    int E[2] = {kNoExp, kNoExp};
+    {
+        double2 x[2][4 * KS];
+        int sc[4 * KS];
+#pragma unroll
+        for (int i = 0; i < 4 * KS; ++i) {
+            const int k = 16 * (i >> 2) + 2 * t + (i & 1) + 8 * ((i >> 1) & 1);
+            const long long o = col(k);
+            sc[i] = ek ? ek[k] : 0;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int r = h ? rb : ra;
+                x[h][i] = r < rows ? X[r + o] : make_double2(0.0, 0.0);
+                const int e = exp_c128(x[h][i]);
+                if (e != kNoExp) E[h] = max(E[h], e - sc[i]);      // a zero does not count, whatever its column's scale
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            E[h] = max(E[h], __shfl_xor_sync(0xffffffffu, E[h], 1));
+            E[h] = max(E[h], __shfl_xor_sync(0xffffffffu, E[h], 2));
+        }
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                unsigned long long vr[4], vi[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    vr[i] = fixed_part(x[h][4 * ks + i].x, E[h], sc[4 * ks + i]);
+                    vi[i] = fixed_part(x[h][4 * ks + i].y, E[h], sc[4 * ks + i]);
+                }
+                uint32_t lo[kDigits], hi[kDigits];
+                digits4(vr, lo, hi);
+#pragma unroll
+                for (int d = 0; d < kDigits; ++d) { Ar[d][ks][h] = lo[d]; Ar[d][ks][2 + h] = hi[d]; }
+                digits4(vi, lo, hi);
+#pragma unroll
+                for (int d = 0; d < kDigits; ++d) { Ai[d][ks][h] = lo[d]; Ai[d][ks][2 + h] = hi[d]; }
+            }
+    }
+    __syncwarp();
+    for (int nt = 0; nt < NT; ++nt) {
+        const uint2* Jr = Jd + nt * 32;
+        const uint2* Ji = Jr + F;
+        float a1[kWeights][4], a2[kWeights][4];
+        double yr[4];
+        int s[4];
+        digit_products<KS>(a1, Ar, Jr, KS * NT * 32, NT * 32, lane);
+        digit_products<KS>(a2, Ai, Ji, KS * NT * 32, NT * 32, lane);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            s[i] = E[i >> 1] + fc[8 * nt + 2 * t + (i & 1)] - 2150 + 51;
+            yr[i] = fixed_to_f64(combined(a1, i) - combined(a2, i), s[i]);
+        }
+        digit_products<KS>(a1, Ar, Ji, KS * NT * 32, NT * 32, lane);
+        digit_products<KS>(a2, Ai, Jr, KS * NT * 32, NT * 32, lane);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int cc = 8 * nt + 2 * t + (i & 1), r = i < 2 ? ra : rb;
+            const double yi = fixed_to_f64(combined(a1, i) + combined(a2, i), s[i]);
+            if (r < rows) X[r + col(cc)] = make_double2(yr[i], yi);
+        }
+    }
+}
+
 // S4/S5: [W_i W_j] <- [W_i W_j] J for rowsW rows of W (its columns scaled by
 // their exponents ek) and [V_i V_j] <- [V_i V_j] J for rowsV rows of V (0: V not
 // kept; unscaled), 16-row tiles tile0, tile0 + step .. dealt to the group's
 // warps.  Jd: j_digit_bytes, fc: 2 NB ints, both in shared memory.
-template <int NB, int GT>
-__device__ __forceinline__ void update_f64_split(double* W, long long ldw, int rowsW, double* V, long long ldv, int rowsV,
-                                                 int cbi, int cbj, const double* J, int ldj, const int* ek, uint2* Jd,
+template <int NB, int GT, class T>
+__device__ __forceinline__ void update_f64_split(T* W, long long ldw, int rowsW, T* V, long long ldv, int rowsV,
+                                                 int cbi, int cbj, const T* J, int ldj, const int* ek, uint2* Jd,
                                                  int* fc, int gt, int bar, int block = 0, int blocks = 1) {
     constexpr int NWG = GT / 32;
     const int warp = gt >> 5, lane = gt & 31, tw = (rowsW + 15) / 16, tv = (rowsV + 15) / 16, step = NWG * blocks;
