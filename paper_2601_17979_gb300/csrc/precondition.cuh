@@ -65,7 +65,9 @@ template <> constexpr float kPreTiny<float> = 1e-34f;
 template <> constexpr double kPreTiny<double> = 1e-290;
 
 // Scratch of one matrix, N entries each (two sets of column norms: a step
-// reads one while it writes the other).
+// reads one while it writes the other).  v0 has at least eight: graded_rows
+// keeps two ints a warp of up to 256 threads there, while the norms and the
+// permutation are live.
 template <class T>
 struct PreScratch {
     Real<T>* nrm2;
@@ -75,13 +77,13 @@ struct PreScratch {
     int* perm;
     __device__ explicit PreScratch(void* p, int N) {
         v0 = static_cast<T*>(p);
-        diag = v0 + N;
+        diag = v0 + (N < 8 ? 8 : N);
         nrm2 = reinterpret_cast<Real<T>*>(diag + N);
         tau = nrm2 + 2 * N;
         perm = reinterpret_cast<int*>(tau + N);
     }
     __host__ __device__ static constexpr long long bytes(long long N) {
-        return N * (2 * (long long)sizeof(T) + 3 * (long long)sizeof(Real<T>) + 4);
+        return (N < 8 ? 8 : N) * (long long)sizeof(T) + N * ((long long)sizeof(T) + 3 * (long long)sizeof(Real<T>) + 4);
     }
 };
 
@@ -218,6 +220,7 @@ __device__ __forceinline__ bool eight_lanes(int N) { return NT <= 128 && 8 * N <
 template <class T, int NT>
 __device__ __forceinline__ bool graded_rows(const T* W, int ldw, int M, int N, int* red) {
     constexpr int NW = NT / 32;
+    static_assert(NW <= 8, "PreScratch::v0");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int lo = 1 << 20, hi = 0;
     for (int r = tid; r < M; r += NT) {

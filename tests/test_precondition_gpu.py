@@ -139,3 +139,16 @@ def test_mixed_restoration(m, n, dtype):
     assert (info == 0).all()
     S[2], mats[2] = S[2] * 2.0 ** -500, mats[2] * 2.0 ** -500
     check(mats, S, U, V, info, "mixed")
+
+
+# fewer columns than the CTA has warps: reductions share the scratch with the
+# norms and the permutation
+@pytest.mark.parametrize("dtype", [np.float32, np.float64, np.complex64, np.complex128])
+@pytest.mark.parametrize("m,n", [(1, 1), (40, 1), (1, 9), (40, 2), (2, 2), (40, 3), (3, 60), (90, 7)])
+def test_few_columns(m, n, dtype):
+    rng = np.random.default_rng(31 * m + n)
+    cplx = np.issubdtype(dtype, np.complexfloating)
+    mats = [(rng.standard_normal((m, n)) + (1j * rng.standard_normal((m, n)) if cplx else 0)).astype(dtype) for _ in range(3)]
+    for kw in [dict(nb=8), dict(nb=16)] + ([dict(nb=16, prec="mixed")] if dtype in (np.float64, np.complex128) else []):
+        S, U, V, info = run(mats, **kw)
+        check(mats, S, U, V, info, f"{dtype.__name__} {m}x{n} {kw}")
