@@ -320,12 +320,13 @@ __device__ __forceinline__ bool entry_fires(const T* G, int p, int q, Real<T> to
 // singular values' last digits, and the shorter sweeps (which leave S closer
 // to the exact values: 4.9e-5 against 6.9e-5 relative on 512 x 512) would
 // move them by more than FP32 results may move between versions (2e-5).
-// Complex128 keeps them up to 4 blocks (75 x 50: 47.9 ms against 50.1).
+// Complex128 keeps them up to 3 blocks (2,000 of 20 x 20, nb = 8: 11.8 ms against
+// 12.5; at 4 blocks 500 of 64 x 64 29.2 ms full, 26.7 with cross pairs).
 // Sweeps on 256 x 256 FP32: 11.3 full, 11.6 with cross pairs, half the steps.
 template <class T>
 __device__ __forceinline__ bool cross_only(int inner_sweeps, int l, int r, int bi, int bj) {
     constexpr bool kSingle = sizeof(Real<T>) == 4, kC128 = sizeof(T) == 16;
-    return inner_sweeps == 0 && r > 0 && (!kSingle || l <= 20) && (!kC128 || l > 4) &&
+    return inner_sweeps == 0 && r > 0 && (!kSingle || l <= 20) && (!kC128 || l > 3) &&
            !((l & 1) && r == 1 && (bi == l - 1 || bj == l - 1));
 }
 
