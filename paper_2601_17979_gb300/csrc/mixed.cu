@@ -3,7 +3,7 @@
 // FP64 results from mostly-FP32 work: the FP32 solver runs on an FP32 copy
 // of A until its own convergence test passes, giving V32; this file's
 // kernels then restore an orthonormal V in FP64 (Newton-Schulz steps
-// V <- V - V (V^H V - I) / 2 from the widened V32, up to 127 columns with a
+// V <- V - V (V^H V - I) / 2 from the widened V32, in real FP64 from 33 to 127 columns with a
 // preconditioning and a first-order diagonalisation step between them) and
 // form A_hat = A V in FP64; FP64 polish sweeps on A_hat, starting from that V, win the accuracy
 // back (the FP64 test decides convergence).  On a GB300, whose FP64 rate is
@@ -94,63 +94,12 @@ __device__ __forceinline__ void mx_newton_schulz(const T64* Vin, T64* Vout, T64*
     __syncthreads();
 }
 
-// First-order diagonalisation of L^H L (L: N x N, leading dimension ldl) from
-// the V that belongs to it: Vout = V (I + Omega), Omega antihermitian with
-// omega_ij = g_ij / (g_jj - g_ii), where that is below 1e-2 (closer pairs are
-// left to the sweeps).  One product instead of a sweep's dependent rotations:
-// off-diagonals of 1e-7 become 1e-14.  d: N reals in shared memory.  V (I +
-// Omega) is orthonormal to |Omega|^2; the caller restores it.
-template <class T64, int NT>
-__device__ __forceinline__ void mx_refine(const T64* L, int ldl, const T64* V, T64* Vout, T64* E, Real<T64>* d, int N) {
-    using R = Real<T64>;
-    const int tid = threadIdx.x;
-    for (int e = tid; e < N * (N + 1) / 2; e += NT) {
-        int ca, cb;
-        tri_index(e, ca, cb);
-        T64 acc = make_s<T64>(0);
-        for (int i = cb; i < N; ++i)                       // L is lower triangular
-            acc = cfma(L[i + (long long)ca * ldl], L[i + (long long)cb * ldl], acc);
-        E[ca + (long long)cb * N] = acc;
-        if (ca == cb) d[ca] = re(acc);
-    }
-    __syncthreads();
-    for (int e = tid; e < N * (N + 1) / 2; e += NT) {
-        int ca, cb;
-        tri_index(e, ca, cb);
-        T64 w = make_s<T64>(0);
-        if (ca < cb) {
-            const T64 g = E[ca + (long long)cb * N];
-            const R den = d[cb] - d[ca];
-            if (abs_rot(g) < R(1e-2) * abs_s(den)) w = divr(g, den);
-        }
-        E[ca + (long long)cb * N] = w;
-        E[cb + (long long)ca * N] = scale(conj_s(w), R(-1));
-    }
-    __syncthreads();
-    for (int e = tid; e < N * N; e += NT) {
-        const int i = e % N, k = e / N;
-        T64 acc = V[i + (long long)k * N];
-        for (int j = 0; j < N; ++j) acc = fma_s(V[i + (long long)j * N], E[j + (long long)k * N], acc);
-        Vout[i + (long long)k * N] = acc;
-    }
-    __syncthreads();
-}
-
-// complex128: V (N x N) orthonormal in FP64 from V32, close to the right singular vectors
+// V (N x N) orthonormal in FP64 from V32, close to the right singular vectors
 // of A' = A or A^H; A_hat (M x N, ld M) = A' V.  One CTA per matrix on
-// L2-resident buffers:
-//   V = widen(V32), one Newton-Schulz step; A_hat = A' V (off-diagonal to
-//   1e-7, FP32's accuracy, but O(1) relative to short columns of a graded
-//   matrix); A_hat P = Q L Z^H, V <- V P Z (precondition.cuh: contracts those
-//   by the squared ratio of the singular values); the first-order step on
-//   L^H L; two Newton-Schulz steps; A_hat = A' V.
-// The FP64 sweeps that follow need 2 sweeps instead of 4 on 128 x 64 with
-// kappa = 1e6, 3.5 instead of 8 on the clustered 96 x 96 set.
+// L2-resident buffers: V = widen(V32), two Newton-Schulz steps, A_hat = A' V.
 template <class T64, class T32>
 __global__ void __launch_bounds__(kMxThreads) mx_restore(const MixedArgs a) {
-    using R = Real<T64>;
     constexpr int NT = kMxThreads;
-    extern __shared__ __align__(16) unsigned char smem[];
     const int b = blockIdx.x, tid = threadIdx.x;
     const int M = a.M, N = a.N;
     const long long nn = (long long)N * N;
@@ -173,16 +122,8 @@ __global__ void __launch_bounds__(kMxThreads) mx_restore(const MixedArgs a) {
         }
         __syncthreads();
     };
-    for (int e = tid; e < N * N; e += NT) Vb[e] = widen_s(V32[e]);
+    for (int e = tid; e < N * N; e += NT) Va[e] = widen_s(V32[e]);
     __syncthreads();
-    mx_newton_schulz<T64, NT>(Vb, Va, E, N);
-    product(Va);
-    const PreScratch<T64> sc(smem, N);
-    // A_hat carries A's scale: without it where squares could leave FP64's range (or A is not finite)
-    int wide = 0;
-    for (int e = tid; e < M * N; e += NT) wide |= !(maxabs(Ah[e]) < R(1e100));
-    if (!__syncthreads_or(wide) && precondition<T64, NT>(Ah, M, M, N, Vb, N, Va, N, nullptr, 0, sc))
-        mx_refine<T64, NT>(Ah, M, Vb, Va, E, sc.nrm2, N);
     mx_newton_schulz<T64, NT>(Va, Vb, E, N);
     mx_newton_schulz<T64, NT>(Vb, Va, E, N);
     product(Va);
@@ -354,7 +295,22 @@ cudaError_t mixed_restore_tiled(const MixedArgs& a, int batch, cudaStream_t st) 
 }
 
 // ---- the restoration in real FP64: products as FP16 digits ---------------------
-// The same steps as mx_restore with every product as an exact digit product
+// The steps of mx_restore, and up to 127 columns between a first Newton-Schulz
+// step and its two:
+//   A_hat = A' V (off-diagonal to 1e-7, FP32's accuracy, but O(1) relative to
+//   short columns of a graded matrix); A_hat P = Q L Z^T, V <- V P Z
+//   (precondition.cuh: contracts those by the squared ratio of the singular
+//   values); V <- V (I + Omega), the first-order diagonalisation of L^T L
+//   (antisymmetric, omega_ij = g_ij / (g_jj - g_ii) where that is below 1e-2;
+//   closer pairs are left to the sweeps): one product instead of a sweep's
+//   dependent rotations, off-diagonals of 1e-7 become 1e-14.
+// The FP64 sweeps that follow then need 2 sweeps instead of 4 on 128 x 64 with
+// kappa = 1e6, 3.5 instead of 8 on the clustered 96 x 96 set.  Up to kMxPlainN
+// columns the sweep saved costs less than the launches and that step: 2,000 of
+// 16 x 16 1.25 ms plain and 1.80 so, of 32 x 32 3.68 and 4.59, one 32 x 32 0.56
+// and 0.81; 40 x 40 10.5 (the first version) and 9.7, one 1.55 and 1.51.
+// complex128 stays plain: in one CTA on the FP64 pipe the step made one 96 x 96
+// 17.1 ms instead of 11.5.  Every product is an exact digit product
 // (tc_f64.cuh) over (matrix, 64 rows, 32 columns) grids, 32 terms of the
 // contraction at a time; the chunks' sums are added in FP64 in increasing
 // order.  Per chunk a CTA stages both operands in shared memory, splits the
@@ -365,15 +321,15 @@ enum MxOp {
     kMxGram,      // E = V^T V - I
     kMxGramL,     // E = L^T L, L the lower triangle in A_hat
     kMxNs,        // Vn = V - V E / 2
-    kMxRefine,    // Vn = V (I + Omega), Omega_ij = E_ij / (E_jj - E_ii) as mx_refine
+    kMxRefine,    // Vn = V (I + Omega), Omega_ij = E_ij / (E_jj - E_ii)
     kMxAhat,      // A_hat = A' V
 };
-constexpr int kMxDT = 64, kMxDC = 32, kMxDThreads = 128;
+constexpr int kMxDT = 64, kMxDC = 32, kMxDThreads = 128, kMxPlainN = 32;
 
 // cur: 1 where the current V is Vtmp (the next one then goes to V64)
 template <int OP>
 __global__ void __launch_bounds__(kMxDThreads, 3) mx_digits(const MixedArgs a, int cur) {
-    constexpr int LDA = kMxDT + 2, LDB = kMxDC + 1, KS = 2, NT = 4;
+    constexpr int LDA = kMxDT + 2, LDB = kMxDC + 1, NT = 4;
     static_assert(kMxDC == 32, "a chunk is 2 x 16 columns");
     __shared__ double As[kMxDC * LDA], Bs[kMxDC * LDB];
     __shared__ uint2 Jd[j_digit_bytes<double, 16>() / sizeof(uint2)];
@@ -550,13 +506,12 @@ cudaError_t mixed_prepare(const MixedArgs& a, int batch, cudaStream_t st) {
 
 template <class T64, class T32>
 cudaError_t mixed_restore(const MixedArgs& a, int batch, cudaStream_t st) {
-    if constexpr (sizeof(T64) == 8) {
-        return mixed_restore_digits<T64, T32>(a, batch, st);
-    } else {
+    if constexpr (sizeof(T64) == 8)
+        if (a.N > kMxPlainN) return mixed_restore_digits<T64, T32>(a, batch, st);
+    if constexpr (sizeof(T64) == 16)
         if (a.N >= kMxTiledN) return mixed_restore_tiled<T64, T32>(a, batch, st);
-        mx_restore<T64, T32><<<batch, kMxThreads, (size_t)PreScratch<T64>::bytes(a.N), st>>>(a);
-        return cudaGetLastError();
-    }
+    mx_restore<T64, T32><<<batch, kMxThreads, 0, st>>>(a);
+    return cudaGetLastError();
 }
 
 cudaError_t mixed_prepare_d(const MixedArgs& a, int batch, cudaStream_t st) { return mixed_prepare<double, float>(a, batch, st); }
