@@ -53,15 +53,17 @@ PEAK_FP32 = 152 * 128 * 2 * 2.07e9
 # kernels grows in proportion to the matrices solved).
 CSRC = os.path.join(ROOT, "paper_2601_17979_gb300", "csrc")
 KERNEL_SOURCES = {
-    "fused": ("gesvj_fused.cuh", "jacobi_common.cuh", "fused_f32.cuh", "scalar.cuh", "tc_f32.cuh"),
-    "persistent": ("gesvj_fused.cuh", "jacobi_common.cuh", "fused_f32.cuh", "scalar.cuh", "tc_f32.cuh"),
-    "uneven": ("gesvj_fused.cuh", "jacobi_common.cuh", "fused_f32.cuh", "scalar.cuh", "tc_f32.cuh",
-               "tc_c64.cuh", "gesvj_blocked.cuh", "blocked_launch.cuh", "gesvj_pairstep.cuh"),
+    "fused": ("gesvj_fused.cuh", "jacobi_common.cuh", "precondition.cuh", "fused_f32.cuh", "scalar.cuh", "tc_f32.cuh",
+              "tc_f64.cuh"),
+    "persistent": ("gesvj_fused.cuh", "jacobi_common.cuh", "precondition.cuh", "fused_f32.cuh", "scalar.cuh", "tc_f32.cuh",
+                   "tc_f64.cuh"),
+    "uneven": ("gesvj_fused.cuh", "jacobi_common.cuh", "precondition.cuh", "fused_f32.cuh", "scalar.cuh",
+               "tc_f32.cuh", "tc_f64.cuh", "tc_c64.cuh", "gesvj_blocked.cuh", "blocked_launch.cuh", "gesvj_pairstep.cuh"),
 }
 TRAFFIC_PER_MATRIX = {
     # 128x64, gesvj_fused_kernel<double|float,16,2,128>: 2,000-matrix launches
-    ("fused", "tall128x64_f64", "8b18517283c6"): (137206528 + 143052800) / 2000,
-    ("fused", "tall128x64_f32", "8b18517283c6"): (65873920 + 40259328) / 2000,
+    ("fused", "tall128x64_f64", "ed0a294ded5d"): (135221248 + 145287936) / 2000,
+    ("fused", "tall128x64_f32", "ed0a294ded5d"): (72920064 + 43381504) / 2000,
     # the whole uneven step (every kernel of both types), 2,000-matrix case:
     # 497.6 GB over the warm-up and the timed step
     ("uneven", "uneven", "490147fdfd01"): 497.60e9 / 2 / 2000,

@@ -12,6 +12,11 @@
 //   S4/S5  [W_i W_j] <- [W_i W_j] J, [V_i V_j] <- [V_i V_j] J, each element
 //       read and written once (Design-3, Alg. 4); skipped when no rotation
 //       fired (the pair-level mask of Design-4, Sec. 6)
+// After a sweep's first round only the cross pairs of i and j are swept
+// (cross_only).  Where preconditioned() says so the sweeps run on the triangular
+// factor of W instead (precondition.cuh) and Q is applied to the left vectors at
+// the end; FP64 and complex128 (nb = 8, 16) form S2, S4 and S5 as exact digit
+// products on the tensor cores (tc_f64.cuh).
 // A matrix is converged after a sweep in which no rotation fired.  Then
 // sigma_k = ||w_k||_2, a stable descending sort, U = W Sigma^-1 (Alg. 2), and
 // one Newton-Schulz step V <- V - V (V^H V - I) / 2 that restores the
