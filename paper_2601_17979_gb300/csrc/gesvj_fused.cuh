@@ -619,8 +619,17 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
 template <int Base, int NT>
 constexpr int min_blocks_for() { return Base * (256 / NT > 1 ? 256 / NT : 1); }
 
+// Real FP64 with nb = 8 (128 threads) takes 204 registers with the digit products,
+// two CTAs an SM; latency-bound, it gains from four (128 registers, 56 bytes of
+// spills): 1,000 of 32 x 32 4.00 -> 3.01 ms (three CTAs 3.46), 500 of 64 x 47 4.78
+// (three: 6.93), 2,000 of 16 x 16 2.22 -> 1.59 (three: 1.75).
+template <class T, int NB, int NT>
+constexpr int fused_blocks() {
+    return std::is_same<T, double>::value && NB == 8 ? 4 : min_blocks_for<fused_min_blocks<T>(), NT>();
+}
+
 template <class T, int NB, int NG, int GT>
-__global__ void __launch_bounds__(NG * GT, (min_blocks_for<fused_min_blocks<T>(), NG * GT>()))
+__global__ void __launch_bounds__(NG * GT, (fused_blocks<T, NB, NG * GT>()))
 gesvj_fused_kernel(const FusedArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int mid = a.index ? a.index[blockIdx.x] : (int)blockIdx.x;
