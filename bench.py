@@ -62,8 +62,8 @@ KERNEL_SOURCES = {
 }
 TRAFFIC_PER_MATRIX = {
     # 128x64, gesvj_fused_kernel<double|float,16,2,128>: 2,000-matrix launches
-    ("fused", "tall128x64_f64", "ed0a294ded5d"): (135221248 + 145287936) / 2000,
-    ("fused", "tall128x64_f32", "ed0a294ded5d"): (72920064 + 43381504) / 2000,
+    ("fused", "tall128x64_f64", "3288b67c8abc"): (136445440 + 145813760) / 2000,
+    ("fused", "tall128x64_f32", "3288b67c8abc"): (73290240 + 43410432) / 2000,
     # the whole uneven step (every kernel of both types), 2,000-matrix case:
     # 497.6 GB over the warm-up and the timed step
     ("uneven", "uneven", "490147fdfd01"): 497.60e9 / 2 / 2000,
