@@ -296,14 +296,19 @@ cudaError_t mixed_restore_tiled(const MixedArgs& a, int batch, cudaStream_t st) 
 
 // ---- the restoration in real FP64: products as FP16 digits ---------------------
 // The steps of mx_restore, and up to 127 columns between a first Newton-Schulz
-// step and its two:
+// step and three more:
 //   A_hat = A' V (off-diagonal to 1e-7, FP32's accuracy, but O(1) relative to
 //   short columns of a graded matrix); A_hat P = Q L Z^T, V <- V P Z
 //   (precondition.cuh: contracts those by the squared ratio of the singular
 //   values); V <- V (I + Omega), the first-order diagonalisation of L^T L
 //   (antisymmetric, omega_ij = g_ij / (g_jj - g_ii) where that is below 1e-2;
-//   closer pairs are left to the sweeps): one product instead of a sweep's
-//   dependent rotations, off-diagonals of 1e-7 become 1e-14.
+//   closer pairs, and pairs of a row whose entries sum to more than 0.1, are
+//   left to the sweeps): one product instead of a sweep's dependent rotations,
+//   off-diagonals of 1e-7 become 1e-14.  V^T V - I is then Omega^T Omega, at
+//   most 1e-2 in norm by the row sums, and the three Newton-Schulz steps that
+//   follow (e -> 3/4 e^2) take it to 8e-5, 4e-9 and rounding.  The entries'
+//   own limit does not bound it: with many nearly equal singular values
+//   |Omega| reached 0.08, and two steps left V off by 1e-9.
 // The FP64 sweeps that follow then need 2 sweeps instead of 4 on 128 x 64 with
 // kappa = 1e6, 3.5 instead of 8 on the clustered 96 x 96 set.  Up to kMxPlainN
 // columns the sweep saved costs less than the launches and that step: 2,000 of
@@ -321,7 +326,7 @@ enum MxOp {
     kMxGram,      // E = V^T V - I
     kMxGramL,     // E = L^T L, L the lower triangle in A_hat
     kMxNs,        // Vn = V - V E / 2
-    kMxRefine,    // Vn = V (I + Omega), Omega_ij = E_ij / (E_jj - E_ii)
+    kMxRefine,    // Vn = V (I + Omega), Omega in A_hat (mx_omega)
     kMxAhat,      // A_hat = A' V
 };
 constexpr int kMxDT = 64, kMxDC = 32, kMxDThreads = 128, kMxPlainN = 32;
@@ -355,8 +360,7 @@ __global__ void __launch_bounds__(kMxDThreads, 3) mx_digits(const MixedArgs a, i
         if (OP == kMxGram || OP == kMxAhat) return V[k + (long long)c * N];
         if (OP == kMxGramL) return k >= c ? Ah[k + (long long)c * a.M] : 0.0;
         if (OP == kMxNs) return E[k + (long long)c * N];
-        const double g = E[k + (long long)c * N], den = E[c + (long long)c * N] - E[k + (long long)k * N];
-        return k != c && fabs(g) < 1e-2 * fabs(den) ? g / den : 0.0;
+        return Ah[k + (long long)c * N];
     };
     const bool along_k = OP == kMxGram || OP == kMxGramL || (OP == kMxAhat && a.trans);   // the left operand's contiguous index
     for (int r0 = blockIdx.y * kMxDT; r0 < M; r0 += gridDim.y * kMxDT) {
@@ -472,28 +476,63 @@ __global__ void __launch_bounds__(kMxThreads) mx_precondition(const MixedArgs a)
     }
 }
 
+// Omega (N x N, ld N) of E = L^T L into A_hat, whose L is no longer needed: the
+// entries below 1e-2, without the rows and columns whose entries sum to more
+// than 0.1.  One CTA per matrix; dynamic shared memory: 2 N doubles.
+constexpr double kMxOmegaEntry = 1e-2, kMxOmegaRow = 0.1;
+__global__ void __launch_bounds__(kMxThreads) mx_omega(const MixedArgs a) {
+    constexpr int NT = kMxThreads, NW = NT / 32;
+    extern __shared__ __align__(16) unsigned char smem[];
+    double* const diag = reinterpret_cast<double*>(smem);
+    double* const sum = diag + a.N;
+    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, N = a.N;
+    const double* E = static_cast<const double*>(a.E) + b * (long long)N * N;
+    double* Om = static_cast<double*>(a.Ahat) + (long long)b * a.M * N;
+    for (int i = tid; i < N; i += NT) diag[i] = E[i + (long long)i * N];
+    __syncthreads();
+    bool large = false;
+    for (int c = warp; c < N; c += NW) {                   // a column's sum is its row's: |Omega| is symmetric
+        double s = 0;
+        for (int k = lane; k < N; k += 32) {
+            const double g = E[k + (long long)c * N], den = diag[c] - diag[k];
+            const double w = k != c && fabs(g) < kMxOmegaEntry * fabs(den) ? g / den : 0.0;
+            Om[k + (long long)c * N] = w;
+            s += fabs(w);
+        }
+        s = warp_sum(s);
+        if (lane == 0) sum[c] = s;
+        large |= !(s <= kMxOmegaRow);
+    }
+    if (!__syncthreads_or(large)) return;
+    for (int e = tid; e < N * N; e += NT)
+        if (!(sum[e % N] <= kMxOmegaRow && sum[e / N] <= kMxOmegaRow)) Om[e] = 0.0;
+}
+
 template <class T64, class T32>
 cudaError_t mixed_restore_digits(const MixedArgs& a, int batch, cudaStream_t st) {
     const int tn = (a.N + kMxDT - 1) / kMxDT, tc = (a.N + kMxDC - 1) / kMxDC, tm = std::min((a.M + kMxDT - 1) / kMxDT, 65535);
     const long long nn = (long long)a.N * a.N;
     const int wblocks = (int)std::min<long long>((nn + kMxThreads - 1) / kMxThreads, 1024);
     const dim3 sq(batch, tn, tc), rect(batch, tm, tc);
-    auto newton_schulz = [&](int cur) {
-        mx_digits<kMxGram><<<sq, kMxDThreads, 0, st>>>(a, cur);
-        mx_digits<kMxNs><<<sq, kMxDThreads, 0, st>>>(a, cur);
+    MixedArgs w = a;                                       // V64 and Vtmp the other way round
+    w.V64 = a.Vtmp;
+    w.Vtmp = a.V64;
+    auto newton_schulz = [&](const MixedArgs& x, int cur) {
+        mx_digits<kMxGram><<<sq, kMxDThreads, 0, st>>>(x, cur);
+        mx_digits<kMxNs><<<sq, kMxDThreads, 0, st>>>(x, cur);
     };
-    MixedArgs w = a;
-    if (a.N < kMxTiledN) w.V64 = a.Vtmp;                   // an odd number of steps ends in V64
-    mx_widen<T64, T32><<<dim3(batch, wblocks), kMxThreads, 0, st>>>(w);
+    mx_widen<T64, T32><<<dim3(batch, wblocks), kMxThreads, 0, st>>>(a);
     if (a.N < kMxTiledN) {
-        newton_schulz(1);
-        mx_digits<kMxAhat><<<rect, kMxDThreads, 0, st>>>(a, 0);
-        mx_precondition<<<batch, kMxThreads, (size_t)PreScratch<double>::bytes(a.N), st>>>(a);
-        mx_digits<kMxGramL><<<sq, kMxDThreads, 0, st>>>(a, 1);
-        mx_digits<kMxRefine><<<sq, kMxDThreads, 0, st>>>(a, 1);
+        newton_schulz(a, 0);                               // -> Vtmp
+        mx_digits<kMxAhat><<<rect, kMxDThreads, 0, st>>>(w, 0);
+        mx_precondition<<<batch, kMxThreads, (size_t)PreScratch<double>::bytes(a.N), st>>>(w);   // -> V64
+        mx_digits<kMxGramL><<<sq, kMxDThreads, 0, st>>>(a, 0);
+        mx_omega<<<batch, kMxThreads, 2 * a.N * sizeof(double), st>>>(a);
+        mx_digits<kMxRefine><<<sq, kMxDThreads, 0, st>>>(a, 0);                                   // -> Vtmp
+        newton_schulz(a, 1);                               // -> V64
     }
-    newton_schulz(0);
-    newton_schulz(1);
+    newton_schulz(a, 0);
+    newton_schulz(a, 1);
     mx_digits<kMxAhat><<<rect, kMxDThreads, 0, st>>>(a, 0);
     return cudaGetLastError();
 }
