@@ -99,9 +99,12 @@ __device__ __forceinline__ void reflection(T x0, Real<T> ss, T& ph, Real<T>& tau
     // one warp); tau |v|^2 = 2 to a few ulp
     const R nrm = rmul(ss, rsqrt_r(ss)), a0 = abs_rot(x0);
     ph = make_s<T>(nrm);
-    if (a0 > 0) {
-        if constexpr (Traits<T>::kComplex) ph = rscale(x0, nrm / a0);
-        else                               ph = phase_times(x0, a0, nrm);
+    if constexpr (Traits<T>::kComplex) {
+        // below 2^-60 of the norm any phase will do; nrm / a0 could overflow there,
+        // and a denormal x0 does not give its phase to working accuracy
+        if (a0 > rmul(nrm, R(0x1p-60))) ph = rscale(x0, nrm / a0);
+    } else if (a0 > 0) {
+        ph = phase_times(x0, a0, nrm);
     }
     const R st = rsqrt_r(rmul(nrm, nrm + a0));
     tau = rmul(st, st);

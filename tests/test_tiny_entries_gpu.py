@@ -1,0 +1,43 @@
+"""Entries near the bottom of the type's range beside entries of size one
+(needs a GB300): a reflection whose first entry is denormal, in the QR and in
+the LQ.  Bounds as in test_parity_gpu."""
+import numpy as np
+import pytest
+import torch
+
+import __graft_entry__  # noqa: F401
+import oracle
+import paper_2601_17979_gb300 as bsvd
+from oracle import checks
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    __graft_entry__.build()
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64, np.complex64, np.complex128])
+@pytest.mark.parametrize("m,n,nb", [(64, 64, 16), (97, 45, 16), (90, 40, 8), (300, 20, 16), (45, 97, 16)])
+@pytest.mark.parametrize("path", ["auto", "persistent"])
+def test_denormal_entries(path, m, n, nb, dtype):
+    rng = np.random.default_rng(m + n)
+    cplx = np.issubdtype(dtype, np.complexfloating)
+    tiny = [1e-41, 1e-44, 1e-38] if dtype in (np.float32, np.complex64) else [1e-310, 5e-324, 1e-307]
+    mats = []
+    for t in tiny:
+        for rows in ([0], [0, m // 2], list(range(0, m, 2))):
+            A = rng.standard_normal((m, n)) + (1j * rng.standard_normal((m, n)) if cplx else 0)
+            for r in rows:                                   # some of the row's entries: no row is small
+                A[r, rng.random(n) < 0.6] = t
+            mats.append(A.astype(dtype))
+    r = bsvd.gesvj_batched([torch.from_numpy(np.asfortranarray(x)).cuda() for x in mats], path=path, nb=nb)
+    torch.cuda.synchronize()
+    u = checks.unit_roundoff(dtype)
+    wide = [x.astype(np.complex128 if cplx else np.float64) for x in mats]
+    ref = oracle.gesvj(wide)["S"]
+    for i, A in enumerate(wide):
+        assert int(r.info[i]) == 0, i
+        meas = checks.measures(A, r.S[i].cpu().numpy(), r.U[i].cpu().numpy(), r.V[i].cpu().numpy(), ref[i])
+        assert checks.violations(meas, u) == [], (i, meas)
