@@ -1,0 +1,49 @@
+"""Rows of very different sizes (needs a GB300).  One-sided rotations act on each
+row by itself, so the sweeps lose nothing of a small row: the singular values
+of D B, D diagonal and B well conditioned, come out to a relative error of
+about n u cond(B), however small."""
+import numpy as np
+import pytest
+import torch
+
+import __graft_entry__  # noqa: F401
+import oracle
+import paper_2601_17979_gb300 as bsvd
+from oracle import checks
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    __graft_entry__.build()
+
+
+def row_graded(rng, m, n, span, dtype):
+    """D B and cond(B), D from 1 to 2^-span in any order."""
+    B = rng.standard_normal((m, n)) + (1j * rng.standard_normal((m, n)) if np.issubdtype(dtype, np.complexfloating) else 0)
+    d = 2.0 ** -rng.permutation(np.linspace(0, span, m).round())
+    return (B * d[:, None]).astype(dtype), np.linalg.cond(B)
+
+
+def relative_errors(mats, **kw):
+    wide = [x.astype(np.complex128 if np.iscomplexobj(x) else np.float64) for x in mats]
+    ref = oracle.gesvj(wide)["S"]
+    r = bsvd.gesvj(torch.from_numpy(np.stack(mats)).cuda(), **kw)
+    torch.cuda.synchronize()
+    assert int(r.info.max()) == 0
+    S = r.S.cpu().numpy().astype(np.float64)
+    return np.array([(np.abs(S[k] - ref[k]) / ref[k]).max() for k in range(len(mats))])
+
+
+# The factorisations of the preconditioned start are accurate relative to each
+# column only.  Against the plain start (inner_sweeps = 1) of the same call:
+# both within their scatter, a factor of three, and one rounding per column.
+@pytest.mark.parametrize("dtype", [np.float32, np.float64, np.complex64, np.complex128])
+@pytest.mark.parametrize("span", [6, 8, 10])
+@pytest.mark.parametrize("n,nb", [(40, 8), (40, 16), (64, 16)])
+def test_preconditioned_start_keeps_small_values(n, nb, span, dtype):
+    rng = np.random.default_rng(n + span)
+    mats = [row_graded(rng, n, n, span, dtype)[0] for _ in range(24)]
+    err, plain = relative_errors(mats, nb=nb), relative_errors(mats, nb=nb, inner_sweeps=1)
+    assert np.median(err) <= 3 * np.median(plain) + n * checks.unit_roundoff(dtype), (np.median(err), np.median(plain))
