@@ -26,7 +26,7 @@ struct BlockedArgs {
     // also the finalisation scratch: >= M + N*N + N elements)
     void* W; void* Vw; void* G; void* J; void* T;
     long long sW, sVw, sG, sJ, sT;
-    int* state;                // count x 4: status (1 active, 0 converged, -1 bad), rotated, sweeps, exponent
+    int* state;                // count x 4: status (1 active, 0 converged, -1 bad), rotated, sweeps, exponent (blk_exponent)
     int* pairflag;             // count x L/2: the pair rotated in this round
     int* any_active;           // one int: some matrix still active after a sweep
     // caller's arrays (as FusedArgs)

@@ -263,7 +263,7 @@ int device_smem_or_default(bsvd_handle h) {
 struct MixedPlan {
     Plan p32, p64;
     Resolved r32, r64;
-    size_t off[8];        // A32, V32, S32, info32, V64, Vtmp, E, Ahat
+    size_t off[8];        // A32, V32, S32, info32 and plain64, V64, Vtmp, E, Ahat
     size_t off32, off64;  // workspace of the two solves (multi-kernel paths)
     size_t bytes;
 };
@@ -333,7 +333,7 @@ bsvd_status mixed_impl(char t, bsvd_handle h, bool wantU, bool wantV, int batch,
     ma.V64 = w + mp.off[4]; ma.Vtmp = w + mp.off[5]; ma.E = w + mp.off[6]; ma.Ahat = w + mp.off[7];
     void* S32 = w + mp.off[2];
     int* info32 = reinterpret_cast<int*>(w + mp.off[3]);
-    int* sweeps32 = info32 + batch;
+    ma.plain64 = info32 + batch;
     const TypeOps o32 = ops_for(t == 'd' ? 's' : 'c'), o64 = ops_for(t);
     cudaError_t e = (t == 'd') ? bsvd::mixed_prepare_d(ma, batch, s) : bsvd::mixed_prepare_z(ma, batch, s);
     if (e != cudaSuccess) return fail_cuda(h, e);
@@ -343,14 +343,14 @@ bsvd_status mixed_impl(char t, bsvd_handle h, bool wantU, bool wantV, int batch,
         a.A = ma.A32; a.sA = (long long)M * N; a.lda = M;
         a.S = S32; a.sS = N;
         a.V = ma.V32; a.sV = (long long)N * N; a.ldv = N;
-        a.info = info32; a.sweeps = sweeps32;
+        a.info = info32; a.sweeps = nullptr;
         e = o32.blocked(mp.p32.nb, a, w + mp.off32, s, mp.p32.two_stage, mp.p32.host_sync, capture_stream(h, r.flags));
     } else {
         FusedArgs& a = mp.p32.a;
         a.A = ma.A32; a.sA = (long long)M * N; a.lda = M;
         a.S = S32; a.sS = N;
         a.V = ma.V32; a.sV = (long long)N * N; a.ldv = N;
-        a.info = info32; a.sweeps = sweeps32;
+        a.info = info32; a.sweeps = nullptr;
         e = o32.launch(mp.p32.nb, a, batch, mp.p32.smem, s);
     }
     if (e != cudaSuccess) return fail_cuda(h, e);

@@ -60,6 +60,11 @@ __device__ __forceinline__ bool blk_skip(const BlockedArgs& a, int b) {
     return st < 0 || (a.masks && st == 0);
 }
 
+// state[3]: the exponent ex, doubled, plus one where the rows' sizes keep the
+// matrix on the FP64 pipe (kDigitRowSpan)
+__device__ __forceinline__ int blk_exponent(const BlockedArgs& a, int b) { return a.state[4 * b + 3] >> 1; }
+__device__ __forceinline__ bool blk_plain64(const BlockedArgs& a, int b) { return (a.state[4 * b + 3] & 1) != 0; }
+
 // ---- load: W = A * 2^-ex (or A^H), padded; V = I; status -------------------
 // ---- S2, real FP32: register tiles --------------------------------------------
 // The full 2nb x 2nb Gram block of the pair in 4 x 4 register tiles (float4
@@ -307,7 +312,7 @@ __global__ void __launch_bounds__(kBlkThreads) blk_load(const BlockedArgs a) {
         a.state[4 * b + 0] = bd ? -1 : 1;
         a.state[4 * b + 1] = 0;
         a.state[4 * b + 2] = 0;
-        a.state[4 * b + 3] = ex_s;
+        a.state[4 * b + 3] = 2 * ex_s;
     }
     __syncthreads();
     if (bad_s) return;
@@ -326,6 +331,12 @@ __global__ void __launch_bounds__(kBlkThreads) blk_load(const BlockedArgs a) {
     for (int e = tid; e < N * sh.Np; e += NT) {
         const int i = e % N, j = e / N;
         V[i + (long long)j * N] = (V0 && j < N) ? V0[i + (long long)j * a.ldv0] : make_s<T>(i == j && !V0 ? 1 : 0);
+    }
+    if constexpr (sizeof(R) == 8) {
+        __shared__ int span_s[2 * NW];
+        __syncthreads();
+        const int span = row_span<T, NT>(W, 1, M, M, N, span_s);
+        if (tid == 0) a.state[4 * b + 3] = 2 * ex + (span > kDigitRowSpan ? 1 : 0);
     }
 }
 
@@ -412,9 +423,14 @@ __global__ void __launch_bounds__(8 * NB) blk_gram_f64_tc(const BlockedArgs a, i
     int bi, bj;
     if (!blk_pair(sh, r, q, bi, bj)) return;
     const T* W = static_cast<const T*>(a.W) + sh.oW;
-    column_exponents_f64<NB, NT>(W, sh.M, sh.M, bi * NB, bj * NB, ec, tid);
-    __syncthreads();
-    gram_f64_split<NB, NT, TWO + 1>(W, sh.M, sh.M, bi * NB, bj * NB, ec, Gs, tid, 1);
+    if (blk_plain64(a, b)) {
+        gram_f64_fma<T, NB, NT>(W, sh.M, sh.M, bi * NB, bj * NB, Gs, TWO + 1, tid);
+        __syncthreads();
+    } else {
+        column_exponents_f64<NB, NT>(W, sh.M, sh.M, bi * NB, bj * NB, ec, tid);
+        __syncthreads();
+        gram_f64_split<NB, NT, TWO + 1>(W, sh.M, sh.M, bi * NB, bj * NB, ec, Gs, tid, 1);
+    }
     T* G = static_cast<T*>(a.G) + sh.oG + (long long)q * TWO * TWO;
     for (int e = tid; e < TWO * TWO; e += NT) G[e] = Gs[e % TWO + (e / TWO) * (TWO + 1)];
 }
@@ -522,6 +538,13 @@ __global__ void __launch_bounds__(kUpdRows) blk_update_fused(const BlockedArgs a
         // a CTA's four warps take the 16-row tiles of its share of W, then of V.
         // On the FP64 pipe this update ran at 93 % of it: 480 us a round for
         // 64 matrices of 256 x 256.
+        if (blk_plain64(a, b)) {
+            for (int e = tid; e < TWO * TWO; e += kUpdRows) Js[e] = Jg[e];
+            __syncthreads();
+            update_f64_fma<T, NB, kUpdRows>(static_cast<T*>(a.W) + sh.oW, sh.M, sh.M, static_cast<T*>(a.Vw) + sh.oV, sh.N,
+                                            sh.N, bi * NB, bj * NB, Js, TWO, tid, blockIdx.z, gridDim.z);
+            return;
+        }
         uint2* Jd = reinterpret_cast<uint2*>(smem_js);
         int* ek = reinterpret_cast<int*>(smem_js + j_digit_bytes<T, NB>());
         const T* Gg = static_cast<const T*>(a.G) + sh.oG + (long long)q * TWO * TWO;
@@ -715,7 +738,7 @@ __global__ void __launch_bounds__(kBlkThreads) blk_finalize(const BlockedArgs a)
         Vout = a.Vp ? static_cast<T*>(a.Vp[mid]) : static_cast<T*>(a.V) + (long long)mid * a.sV;
         ldv = a.ldvp ? a.ldvp[mid] : a.ldv;
     }
-    const int status = a.state[4 * b], sw = a.state[4 * b + 2], ex = a.state[4 * b + 3];
+    const int status = a.state[4 * b], sw = a.state[4 * b + 2], ex = blk_exponent(a, b);
     if (status < 0) {
         for (int e = tid; e < N; e += NT) Sout[e] = nan_s<R>();
         if (Uout) for (int e = tid; e < sh.m * N; e += NT) Uout[(e % sh.m) + (long long)(e / sh.m) * ldu] = nan_s<T>();

@@ -314,7 +314,10 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
     T* const Z = a.trans ? Uout : Vout;                        // V; N x N
     const long long ldy = a.trans ? ldv : ldu, ldz = a.trans ? ldu : ldv;
     bool pre = false;
-    if (preconditioned<T, NB>(a)) {
+    const bool try_pre = preconditioned<T, NB>(a);
+    const int span = kSplit || try_pre ? row_span<T, NT>(W, 1, ldw, M0, N, reinterpret_cast<int*>(smem + a.offG)) : 0;
+    const bool plain64 = kSplit && span > kDigitRowSpan;
+    if (try_pre && span <= pre_row_span(M0, N)) {
         if constexpr (std::is_same<T, float>::value)
             pre = precondition_f32<NT>(W, ldw, M0, N, needVs ? Vs : nullptr, ldvs, wantWout ? Y : nullptr, ldy,
                                        PreF32(smem + a.offG, M0, N));
@@ -355,60 +358,17 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
                     if (NB >= 8 && !(a.flags & kFlagF32Ffma)) gram_f32_mma<NB < 8 ? 8 : NB, GT>(W, ldw, M, bi * NB, bj * NB, G, gt);
                     else gram_f32_tiled<NB, GT>(W, ldw, M, bi * NB, bj * NB, G, gt);
                 } else if constexpr (kSplit) {
-                    column_exponents_f64<NB, GT>(W, ldw, M, bi * NB, bj * NB, ek, gt);
-                    group_sync(g, GT);
-                    gram_f64_split<NB, GT, LDG>(W, ldw, M, bi * NB, bj * NB, ek, G, gt, g + 1);
-                    if (gt < TWO) ek[gt] = norm_exponent_f64(re(G[gt + gt * LDG]));   // for the update
-                } else if constexpr (!OnChip) {
-                    // W in global memory: 2 x 2 tiles of upper entries per lane
-                    // pair, four independent sums (half the loads per FMA of
-                    // one entry at a time); each entry still sums k in order
-                    // over its half of the rows, so the bits are those of the
-                    // branch below
-                    constexpr int TH = TWO / 2, NTL = TH * (TH + 1) / 2, NWG = GT / 32;
-                    const int wg = gt >> 5, kh = (gt >> 4) & 1, el = gt & 15;
-                    const int kb = kh ? M / 2 : 0, ke = kh ? M : M / 2;
-                    for (int t0 = wg * 16; t0 < NTL; t0 += NWG * 16) {
-                        const int t = t0 + el;
-                        int ti = 0, tj = 0;
-                        T acc[2][2];
-#pragma unroll
-                        for (int u = 0; u < 2; ++u)
-#pragma unroll
-                            for (int v = 0; v < 2; ++v) acc[u][v] = make_s<T>(0);
-                        if (t < NTL) {
-                            tri_index(t, ti, tj);
-                            const T* x0 = W + col(2 * ti) * ldw;
-                            const T* x1 = W + col(2 * ti + 1) * ldw;
-                            const T* y0 = W + col(2 * tj) * ldw;
-                            const T* y1 = W + col(2 * tj + 1) * ldw;
-#pragma unroll 4
-                            for (int k = kb; k < ke; ++k) {
-                                const T a0 = x0[k], a1 = x1[k], b0 = y0[k], b1 = y1[k];
-                                acc[0][0] = cfma(a0, b0, acc[0][0]);
-                                acc[0][1] = cfma(a0, b1, acc[0][1]);
-                                acc[1][0] = cfma(a1, b0, acc[1][0]);
-                                acc[1][1] = cfma(a1, b1, acc[1][1]);
-                            }
-                        }
-#pragma unroll
-                        for (int u = 0; u < 2; ++u)
-#pragma unroll
-                            for (int v = 0; v < 2; ++v) acc[u][v] = add(acc[u][v], shfl_xor_s(acc[u][v], 16));
-                        if (kh == 0 && t < NTL) {
-#pragma unroll
-                            for (int u = 0; u < 2; ++u)
-#pragma unroll
-                                for (int v = 0; v < 2; ++v) {
-                                    const int ca = 2 * ti + u, cb = 2 * tj + v;
-                                    if (ca > cb) continue;             // lower entry of a diagonal tile
-                                    T x = acc[u][v];
-                                    if (ca == cb) x = make_s<T>(re(x));
-                                    G[ca + cb * LDG] = x;
-                                    G[cb + ca * LDG] = conj_s(x);
-                                }
-                        }
+                    if (plain64) {
+                        gram_f64_fma<T, NB, GT>(W, ldw, M, bi * NB, bj * NB, G, LDG, gt);
+                    } else {
+                        column_exponents_f64<NB, GT>(W, ldw, M, bi * NB, bj * NB, ek, gt);
+                        group_sync(g, GT);
+                        gram_f64_split<NB, GT, LDG>(W, ldw, M, bi * NB, bj * NB, ek, G, gt, g + 1);
+                        if (gt < TWO) ek[gt] = norm_exponent_f64(re(G[gt + gt * LDG]));   // for the update
                     }
+                } else if constexpr (!OnChip) {
+                    // (W in global memory) the bits of the branch below
+                    gram_tiles_fma<T, NB, GT>(W, ldw, M, bi * NB, bj * NB, G, LDG, gt);
                 } else {
                     constexpr int NUP = TWO * (TWO + 1) / 2, NWG = GT / 32;
                     const int wg = gt >> 5, kh = (gt >> 4) & 1, el = gt & 15;
@@ -456,9 +416,6 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
                 if (gt == 0) swflag[sw] = 1;
 
                 // S4/S5: [W_i W_j] <- [W_i W_j] J and [V_i V_j] <- [V_i V_j] J.
-                // A warp takes 16 rows at a time; lanes l and l+16 both read row
-                // l and write the first and the second nb outputs of it, so the
-                // M + n rows spread evenly over the group.  FP32: register tiles.
                 if constexpr (std::is_same<T, float>::value) {
                     if (NB >= 8 && !(a.flags & kFlagF32Ffma)) {
                         constexpr int NBT = NB < 8 ? 8 : NB;       // (nb = 4 never takes this branch)
@@ -472,8 +429,11 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
                         update_f32_tiled<NB, GT, 2>(W, ldw, pre ? (M + 3) & ~3 : ldw, Vs, ldvs, needVs ? ldvs : 0, bi * NB, bj * NB, Jt, gt, g + 1);
                     }
                 } else if constexpr (kSplit) {
-                    update_f64_split<NB, GT>(W, ldw, M, Vs, ldvs, needVs ? N : 0, bi * NB, bj * NB, J, LDG, ek,
-                                         reinterpret_cast<uint2*>(gb_tail), ek + TWO, gt, g + 1);
+                    if (plain64)
+                        update_f64_fma<T, NB, GT>(W, ldw, M, Vs, ldvs, needVs ? N : 0, bi * NB, bj * NB, J, LDG, gt, 0, 1);
+                    else
+                        update_f64_split<NB, GT>(W, ldw, M, Vs, ldvs, needVs ? N : 0, bi * NB, bj * NB, J, LDG, ek,
+                                                 reinterpret_cast<uint2*>(gb_tail), ek + TWO, gt, g + 1);
                 } else if constexpr (std::is_same<T, float2>::value) {
                     // complex64: 4 rows x 2nb/8 columns per lane (columns
                     // cg, cg + 8, ...: conflict-free J reads with its padded
@@ -527,34 +487,8 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
                         J = (J == J0) ? J1 : J0;
                     }
                 } else {
-                    const int rows = M + (needVs && !kDefer ? N : 0);   // on chip V is deferred (DeferredV)
-                    const int wg = gt >> 5, half = (gt >> 4) & 1, rl = gt & 15;
-                    constexpr int NWG = GT / 32;
-                    for (int r0 = wg * 16; r0 < rows; r0 += NWG * 16) {
-                        const int i = r0 + rl;
-                        const bool ok = i < rows;
-                        T* X = W;
-                        int ld = ldw, row = i;
-                        if (i >= M) { X = Vs; ld = ldvs; row = i - M; }
-                        // nb accumulators, each summed over k in order (the
-                        // multi-kernel path's order); x is read one k at a time
-                        T acc[NB];
-#pragma unroll
-                        for (int c = 0; c < NB; ++c) acc[c] = make_s<T>(0);
-                        if (ok) {
-#pragma unroll
-                            for (int k = 0; k < TWO; ++k) {
-                                const T xk = X[row + col(k) * ld];
-#pragma unroll
-                                for (int c = 0; c < NB; ++c) acc[c] = fma_s(xk, J[k + (half * NB + c) * LDG], acc[c]);
-                            }
-                        }
-                        __syncwarp();
-                        if (ok) {
-#pragma unroll
-                            for (int c = 0; c < NB; ++c) X[row + col(half * NB + c) * ld] = acc[c];
-                        }
-                    }
+                    // nb accumulators a lane; on chip V is deferred (DeferredV)
+                    update_rows_fma<T, NB, GT>(W, ldw, M, Vs, ldvs, needVs && !kDefer ? N : 0, bi * NB, bj * NB, J, LDG, gt);
                     if (kDefer && needVs) {   // this pair's V update, run during the next pair step
                         dv.J = J; dv.bi = bi; dv.bj = bj;
                         J = (J == J0) ? J1 : J0;

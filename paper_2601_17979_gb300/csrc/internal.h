@@ -25,6 +25,7 @@ struct MixedArgs {
     void* V32;                              // N x N, ld N: V of the FP32 solve
     void* V64; void* Vtmp; void* E;         // N x N, ld N, FP64: restored V and scratch
     void* Ahat;                             // M x N, ld M, FP64: A V
+    int* plain64;                           // per matrix: no digit products (kDigitRowSpan)
 };
 
 // Buffers of the QR pre-processing path (strided batches; working

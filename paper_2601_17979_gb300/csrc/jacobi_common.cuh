@@ -625,6 +625,122 @@ __device__ int inner_jacobi(T* G, T* J, const InnerTables<T, NB>& tb, Real<T> to
     return seen;
 }
 
+// Binary orders between the rows' largest and smallest largest entry, zero rows
+// apart; entry (r, j) at W[r * sr + j * sj].  red: 2 NT / 32 ints, free on entry.  Called by all NT threads after W is
+// complete and synchronised; returns synchronised.
+template <class T, int NT>
+__device__ __forceinline__ int row_span(const T* W, long long sr, long long sj, int M, int N, int* red) {
+    constexpr int NW = NT / 32;
+    static_assert(NW <= 8, "16 ints of scratch");
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int lo = 1 << 20, hi = 0;
+    for (int r = tid; r < M; r += NT) {
+        int e = 0;
+        for (int j = 0; j < N; ++j) e = max(e, binary_exponent(maxabs(W[r * sr + j * sj])));
+        if (e > 0) {
+            lo = min(lo, e);
+            hi = max(hi, e);
+        }
+    }
+    lo = (int)__reduce_min_sync(0xffffffffu, (unsigned)lo);
+    hi = (int)__reduce_max_sync(0xffffffffu, (unsigned)hi);
+    if (lane == 0) { red[2 * warp] = lo; red[2 * warp + 1] = hi; }
+    __syncthreads();
+    for (int w = 0; w < NW; ++w) { lo = min(lo, red[2 * w]); hi = max(hi, red[2 * w + 1]); }
+    __syncthreads();
+    return hi - lo;
+}
+
+// S2 on the multiply-add pipe: G = P^H P for the panel P of columns [cbi, cbi + NB)
+// and [cbj, cbj + NB) of W, 2 x 2 tiles of upper entries per lane pair, four
+// independent sums (half the loads per multiply-add of one entry at a time).
+// Lanes l and l + 16 of a warp sum the same tile over the two halves of the rows,
+// [0, M/2) and [M/2, M), each in order; one shuffle adds them.  Upper entries are
+// written and mirrored.  The caller synchronises.
+template <class T, int NB, int GT>
+__device__ __forceinline__ void gram_tiles_fma(const T* W, long long ldw, int M, int cbi, int cbj, T* G, int ldg, int gt) {
+    constexpr int TH = NB, NTL = TH * (TH + 1) / 2, NWG = GT / 32;
+    const int wg = gt >> 5, kh = (gt >> 4) & 1, el = gt & 15;
+    const int kb = kh ? M / 2 : 0, ke = kh ? M : M / 2;
+    auto col = [&](int c) { return W + (c < NB ? cbi + c : cbj + c - NB) * ldw; };
+    for (int t0 = wg * 16; t0 < NTL; t0 += NWG * 16) {
+        const int t = t0 + el;
+        int ti = 0, tj = 0;
+        T acc[2][2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int v = 0; v < 2; ++v) acc[u][v] = make_s<T>(0);
+        if (t < NTL) {
+            tri_index(t, ti, tj);
+            const T* x0 = col(2 * ti);
+            const T* x1 = col(2 * ti + 1);
+            const T* y0 = col(2 * tj);
+            const T* y1 = col(2 * tj + 1);
+#pragma unroll 4
+            for (int k = kb; k < ke; ++k) {
+                const T a0 = x0[k], a1 = x1[k], b0 = y0[k], b1 = y1[k];
+                acc[0][0] = cfma(a0, b0, acc[0][0]);
+                acc[0][1] = cfma(a0, b1, acc[0][1]);
+                acc[1][0] = cfma(a1, b0, acc[1][0]);
+                acc[1][1] = cfma(a1, b1, acc[1][1]);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int v = 0; v < 2; ++v) acc[u][v] = add(acc[u][v], shfl_xor_s(acc[u][v], 16));
+        if (kh == 0 && t < NTL) {
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+#pragma unroll
+                for (int v = 0; v < 2; ++v) {
+                    const int ca = 2 * ti + u, cb = 2 * tj + v;
+                    if (ca > cb) continue;                 // lower entry of a diagonal tile
+                    T x = acc[u][v];
+                    if (ca == cb) x = make_s<T>(re(x));
+                    G[ca + cb * ldg] = x;
+                    G[cb + ca * ldg] = conj_s(x);
+                }
+        }
+    }
+}
+
+// S4/S5 on the multiply-add pipe: [X_i X_j] <- [X_i X_j] J for rowsW rows of W,
+// then rowsV rows of V.  A warp takes 16 rows at a time; lanes l and l + 16 both
+// read row l and write the first and the second NB outputs of it, NB accumulators
+// each summed over k in order.  GT threads; blocks > 1: that many groups share
+// the rows.
+template <class T, int NB, int GT>
+__device__ __forceinline__ void update_rows_fma(T* W, long long ldw, int rowsW, T* V, long long ldv, int rowsV, int cbi,
+                                                int cbj, const T* J, int ldj, int gt, int block = 0, int blocks = 1) {
+    constexpr int TWO = 2 * NB, NWG = GT / 32;
+    const int wg = gt >> 5, half = (gt >> 4) & 1, rl = gt & 15, rows = rowsW + rowsV;
+    auto col = [&](int c) { return c < NB ? cbi + c : cbj + c - NB; };
+    for (int r0 = (block * NWG + wg) * 16; r0 < rows; r0 += blocks * NWG * 16) {
+        const int i = r0 + rl;
+        const bool ok = i < rows;
+        T* const X = i < rowsW ? W + i : V + (i - rowsW);
+        const long long ld = i < rowsW ? ldw : ldv;
+        T acc[NB];
+#pragma unroll
+        for (int c = 0; c < NB; ++c) acc[c] = make_s<T>(0);
+        if (ok) {
+#pragma unroll
+            for (int k = 0; k < TWO; ++k) {
+                const T xk = X[col(k) * ld];
+#pragma unroll
+                for (int c = 0; c < NB; ++c) acc[c] = fma_s(xk, J[k + (half * NB + c) * ldj], acc[c]);
+            }
+        }
+        __syncwarp();
+        if (ok) {
+#pragma unroll
+            for (int c = 0; c < NB; ++c) X[col(half * NB + c) * ld] = acc[c];
+        }
+    }
+}
+
 // Shared-memory scratch of finalize_outputs: sig[N], rank[N], red[>= warps],
 // iscr[>= 2], bcast[>= 1].
 template <class T>

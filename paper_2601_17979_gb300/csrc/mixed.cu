@@ -35,13 +35,13 @@ __device__ __forceinline__ const T64* mixed_a(const MixedArgs& a, int b) {
 }
 
 // A32 (M x N, ld M) = fl32(2^-ex A) or fl32(2^-ex A^H) when m < n, ex the
-// exponent of max |a_ij| (exact scaling: FP32's range holds the result).
+// exponent of max |a_ij| (exact scaling: FP32's range holds the result); plain64.
 template <class T64, class T32>
 __global__ void __launch_bounds__(kMxThreads) mx_convert(const MixedArgs a) {
     using R = Real<T64>;
     constexpr int NT = kMxThreads, NW = NT / 32;
     __shared__ R red[NW];
-    __shared__ int ex_s;
+    __shared__ int ex_s, span_s[2 * NW];
     const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const T64* A = mixed_a<T64>(a, b);
     const int lda = a.Ap ? a.ldap[a.index[b]] : a.lda;
@@ -67,6 +67,8 @@ __global__ void __launch_bounds__(kMxThreads) mx_convert(const MixedArgs a) {
         if (a.trans) A32[j + (long long)i * a.M] = narrow_s(conj_s(x));
         else         A32[i + (long long)j * a.M] = narrow_s(x);
     }
+    const int span = row_span<T64, NT>(A, a.trans ? lda : 1, a.trans ? 1 : lda, a.M, a.N, span_s);
+    if (tid == 0) a.plain64[b] = span > kDigitRowSpan;
 }
 
 // V <- V - V (V^H V - I) / 2 (N x N, ld N), from Vin to Vout; E is scratch.
@@ -320,7 +322,8 @@ cudaError_t mixed_restore_tiled(const MixedArgs& a, int batch, cudaStream_t st) 
 // contraction at a time; the chunks' sums are added in FP64 in increasing
 // order.  Per chunk a CTA stages both operands in shared memory, splits the
 // right one into digits once, and each of its four warps splits and multiplies
-// 16 rows.  2,000 of 96x96: the restoration 42 ms as one CTA a matrix on the
+// 16 rows.  A matrix whose rows span more than 2^6 takes multiply-adds on the same
+// tiles (kDigitRowSpan: V's small entries count there).  2,000 of 96x96: the restoration 42 ms as one CTA a matrix on the
 // FP64 pipe, 28.2 so: 9.1 in these products, 19.1 in mx_precondition.
 enum MxOp {
     kMxGram,      // E = V^T V - I
@@ -341,6 +344,7 @@ __global__ void __launch_bounds__(kMxDThreads, 3) mx_digits(const MixedArgs a, i
     __shared__ int ek[kMxDC], fc[kMxDC], range;
     const int b = blockIdx.x, c0 = blockIdx.z * kMxDC, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int N = a.N, M = OP == kMxAhat ? a.M : N;
+    const bool plain = a.plain64[b] != 0;
     const long long nn = (long long)N * N;
     const double* V = static_cast<const double*>(cur ? a.Vtmp : a.V64) + b * nn;
     double* Vn = static_cast<double*>(cur ? a.V64 : a.Vtmp) + b * nn;
@@ -388,6 +392,23 @@ __global__ void __launch_bounds__(kMxDThreads, 3) mx_digits(const MixedArgs a, i
                 const double x = right(k0 + k, c0 + c);
                 Bs[c * LDB + k] = x;
                 bad |= exp_f64(x) == 0x7ff;
+            }
+            if (plain) {                                   // uniform over the CTA: multiply-adds, in order
+                __syncthreads();
+                const int rw = 16 * warp + (lane >> 2), t2 = 2 * (lane & 3);
+                for (int k = 0; k < kMxDC; ++k) {
+                    const double x0 = As[k * LDA + rw], x1 = As[k * LDA + rw + 8];
+#pragma unroll
+                    for (int nt = 0; nt < NT; ++nt) {
+                        const double y0 = Bs[(8 * nt + t2) * LDB + k], y1 = Bs[(8 * nt + t2 + 1) * LDB + k];
+                        sum[nt][0] = fma(x0, y0, sum[nt][0]);
+                        sum[nt][1] = fma(x0, y1, sum[nt][1]);
+                        sum[nt][2] = fma(x1, y0, sum[nt][2]);
+                        sum[nt][3] = fma(x1, y1, sum[nt][3]);
+                    }
+                }
+                __syncthreads();
+                continue;
             }
             if (OP == kMxAhat) {
                 big = __reduce_or_sync(0xffffffffu, big);
@@ -453,7 +474,9 @@ __global__ void __launch_bounds__(kMxDThreads, 3) mx_digits(const MixedArgs a, i
 }
 
 // A_hat P = Q L Z^T with V64 -> Vtmp = V64 P Z, L in A_hat.  Declined (or A_hat too
-// large to square): Vtmp = V64 and L = 0, for which the first-order step is none.
+// large to square, or V's small entries count): Vtmp = V64 and L = 0, for which the
+// first-order step is none.  Only V is kept of it, orthonormal whatever the rows of
+// A_hat span: its rows may.
 // On L2-resident buffers: about half of its 19.1 ms on 2,000 of 96x96 is the FP64
 // pipe's; with A_hat in shared memory (two CTAs an SM instead of four) 19.5 ms.
 __global__ void __launch_bounds__(kMxThreads) mx_precondition(const MixedArgs a) {
@@ -466,7 +489,7 @@ __global__ void __launch_bounds__(kMxThreads) mx_precondition(const MixedArgs a)
     double* Ah = static_cast<double*>(a.Ahat) + (long long)b * M * N;
     int wide = 0;
     for (int e = tid; e < M * N; e += NT) wide |= !(fabs(Ah[e]) < 1e100);
-    if (!__syncthreads_or(wide) &&
+    if (!__syncthreads_or(wide) && !a.plain64[b] &&
         precondition<double, NT>(Ah, M, M, N, Vn, N, V, N, nullptr, 0, PreScratch<double>(smem, N)))
         return;
     __syncthreads();

@@ -65,9 +65,8 @@ template <> constexpr float kPreTiny<float> = 1e-34f;
 template <> constexpr double kPreTiny<double> = 1e-290;
 
 // Scratch of one matrix, N entries each (two sets of column norms: a step
-// reads one while it writes the other).  v0 has at least eight: row_span
-// keeps two ints a warp of up to 256 threads there, while the norms and the
-// permutation are live.
+// reads one while it writes the other).  v0 has at least eight: row_span's two
+// ints a warp of up to 256 threads.
 template <class T>
 struct PreScratch {
     Real<T>* nrm2;
@@ -215,41 +214,17 @@ __device__ __forceinline__ void reflect_columns(T* X, int ldx, int k, int M, int
 template <int NT>
 __device__ __forceinline__ bool eight_lanes(int N) { return NT <= 128 && 8 * N <= NT; }
 
-// Binary orders that the rows' largest entries may span (zero rows apart).  The
+// Binary orders that the rows' largest entries may span (row_span).  The
 // factorisations are accurate relative to each column, not to each row: from a
 // matrix with rows of different sizes they take the relative accuracy of its
 // smallest singular values, which the plain start keeps.  Median over 24
 // matrices D B, FP64 64 x 64, of the largest relative error of a singular value,
-// in units of u, against that of the plain start: D over 2^4 74 and 57, 2^6 179
-// and 69, 2^8 398 and 62, 2^10 848 and 74.  Normal and uniform matrices, and
-// geometric spectra down to 1e-6 of up to three rows a column, span at most four
-// orders; taller ones with such a spectrum (300 x 20: five) take the plain start.
-constexpr int kPreRowSpan = 4;
-
-// Binary orders between the rows' largest and smallest largest entry, zero rows
-// apart.  red: 2 NT / 32 ints.  Synchronised.
-template <class T, int NT>
-__device__ __forceinline__ int row_span(const T* W, int ldw, int M, int N, int* red) {
-    constexpr int NW = NT / 32;
-    static_assert(NW <= 8, "PreScratch::v0");
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    int lo = 1 << 20, hi = 0;
-    for (int r = tid; r < M; r += NT) {
-        int e = 0;
-        for (int j = 0; j < N; ++j) e = max(e, binary_exponent(maxabs(W[r + (long long)j * ldw])));
-        if (e > 0) {
-            lo = min(lo, e);
-            hi = max(hi, e);
-        }
-    }
-    lo = (int)__reduce_min_sync(0xffffffffu, (unsigned)lo);
-    hi = (int)__reduce_max_sync(0xffffffffu, (unsigned)hi);
-    if (lane == 0) { red[2 * warp] = lo; red[2 * warp + 1] = hi; }
-    __syncthreads();
-    for (int w = 0; w < NW; ++w) { lo = min(lo, red[2 * w]); hi = max(hi, red[2 * w + 1]); }
-    __syncthreads();
-    return hi - lo;
-}
+// in units of u, against that of the plain start: D over 2^4 (rows spanning five
+// orders) 74 and 57, 2^5 96 and 57, 2^6 179 and 69, 2^8 398 and 62, 2^10 848 and 74;
+// with two rows a column no more than the plain start's up to 2^10, so those may
+// span one order more (geometric spectra of few columns do by chance: 1000 x 16
+// down to 1e-3 four to six).
+__host__ __device__ constexpr int pre_row_span(int M, int N) { return M >= 2 * N ? 6 : 5; }
 
 // Whether the spectrum is so flat that the sweeps gain little from the
 // preconditioner: the participation ratio (sum sigma^2)^2 / (N sum sigma^4)
@@ -334,9 +309,9 @@ __device__ __forceinline__ void sort_columns(T* W, int ldw, int M, int N, const 
 // V (N x N, unless null) becomes V0 P Z (V0 null: I); the reflections of Q go
 // to refl (M x N, scaled so that tau = 1; null: dropped).  Called by all NT
 // threads after W is complete and synchronised; returns synchronised.
-// Returns false, with nothing changed, when a column is too short to square
-// safely (or zero), when the rows are graded, and in single precision when the
-// spectrum is flat.
+// The caller has seen to it that the rows span at most pre_row_span.  Returns false,
+// with nothing changed, when a column is too short to square safely (or zero), and
+// in single precision when the spectrum is flat.
 //
 // Double precision picks each column by its remaining norm (QR with column
 // pivoting: 128 x 64 with kappa = 1e6 then takes 6.3 sweeps, 7.1 without).
@@ -414,7 +389,6 @@ __device__ __forceinline__ bool precondition(T* W, int ldw, int M, int N, T* V, 
     bool small = false;
     for (int j = lane; j < N; j += 32) small |= !(sc.nrm2[j] > kPreNormMin<R>);
     if (__any_sync(0xffffffffu, small)) { __syncthreads(); return false; }   // uniform: every warp reads all norms
-    if (row_span<T, NT>(W, ldw, M, N, reinterpret_cast<int*>(sc.v0)) > kPreRowSpan) return false;
     if constexpr (sizeof(R) == 4)
         if (M <= 2 * N && flat_spectrum<T, NT>(W, ldw, M, N, sc.nrm2, sc.v0, sc.tau)) return false;
     if constexpr (sizeof(R) == 4)
@@ -716,7 +690,6 @@ __device__ __forceinline__ bool precondition_f32(float* W, int ldw, int M, int N
     bool small = false;
     for (int j = lane; j < N; j += 32) small |= !(sc.nrm2[j] > kPreNormMin<float>);
     if (__any_sync(0xffffffffu, small)) { __syncthreads(); return false; }   // uniform: every warp reads all norms
-    if (row_span<float, NT>(W, ldw, M, N, sc.tmp) > kPreRowSpan) return false;
     if (flat_spectrum<float, NT>(W, ldw, M, N, sc.nrm2, sc.v, sc.tau)) return false;
     sort_columns<float, NT>(W, ldw, M, N, sc.nrm2, sc.perm, sc.tmp, sc.tmp + N);
 

@@ -47,3 +47,46 @@ def test_preconditioned_start_keeps_small_values(n, nb, span, dtype):
     mats = [row_graded(rng, n, n, span, dtype)[0] for _ in range(24)]
     err, plain = relative_errors(mats, nb=nb), relative_errors(mats, nb=nb, inner_sweeps=1)
     assert np.median(err) <= 3 * np.median(plain) + n * checks.unit_roundoff(dtype), (np.median(err), np.median(plain))
+
+
+# The mixed path's restoration of V, whose small entries count where the columns
+# are graded too: within ten times the FP64 pipe's error on the same matrices
+# (complex128 restores V there).
+@pytest.mark.parametrize("n", [40, 96])
+def test_mixed_graded_rows_and_columns(n):
+    rng = np.random.default_rng(n)
+    mats = []
+    for _ in range(12):
+        A = row_graded(rng, n, n, 60, np.float64)[0]
+        mats.append(A * 2.0 ** -rng.permutation(np.linspace(0, 60, n).round()))
+    err = relative_errors(mats, prec="mixed")
+    cplx = relative_errors([x.astype(np.complex128) for x in mats], prec="mixed")
+    assert np.median(err) <= 10 * np.median(cplx), (np.median(err), np.median(cplx))
+
+
+# Gram blocks and updates as digit products (nb = 8, 16) are left out for such
+# matrices, on chip, in global slots and on the multi-kernel path; one row more
+# than the limit of 2^6 spans, and far beyond it.  Wide matrices: graded columns.
+@pytest.mark.parametrize("dtype", [np.float64, np.complex128])
+@pytest.mark.parametrize("nb", [8, 16])
+@pytest.mark.parametrize("path", ["fused", "blocked", "slots"])
+@pytest.mark.parametrize("m,n", [(24, 24), (40, 40), (57, 33), (33, 70)])
+def test_small_values_of_graded_rows(m, n, path, nb, dtype):
+    rng = np.random.default_rng(m + n)
+    u = checks.unit_roundoff(dtype)
+    mats, cond = [], []
+    for span in (7, 8, 20, 40, 60, 100):
+        A, c = row_graded(rng, max(m, n), min(m, n), span, dtype)
+        mats.append(A if m >= n else np.ascontiguousarray(A.conj().T))
+        cond.append(c)
+    T = [torch.from_numpy(np.asfortranarray(x)).cuda() for x in mats]
+    if path == "slots":
+        r = bsvd.gesvj_batched(T, path="persistent", nb=nb, flags=bsvd.FLAG_NO_ONCHIP)
+    else:
+        r = bsvd.gesvj_batched(T, path=path, nb=nb)
+    torch.cuda.synchronize()
+    ref = oracle.gesvj(mats)["S"]
+    for k, A in enumerate(mats):
+        S = r.S[k].cpu().numpy()
+        rel = (np.abs(S - ref[k]) / ref[k]).max()
+        assert int(r.info[k]) == 0 and rel <= 50 * min(m, n) * u * cond[k], (k, int(r.info[k]), rel / u, cond[k])
