@@ -47,13 +47,6 @@ __device__ __forceinline__ bool blk_pair(const BlkShape& s, int r, int q, int& b
     return bj < s.l;
 }
 
-// whether round r's pair step of (bi, bj) takes the cross pairs only (not from
-// a given V, close to convergence: full sweeps save an outer one there)
-template <class T, int NB>
-__device__ __forceinline__ bool blk_cross(const BlockedArgs& a, const BlkShape& s, int r, int bi, int bj) {
-    return NB >= 16 && !a.V0 && cross_only<T>(a.inner_sweeps, s.l, r, bi, bj);
-}
-
 // skip this matrix? (bad input always; converged ones only with masks)
 __device__ __forceinline__ bool blk_skip(const BlockedArgs& a, int b) {
     const int st = a.state[4 * b];
@@ -64,6 +57,14 @@ __device__ __forceinline__ bool blk_skip(const BlockedArgs& a, int b) {
 // matrix on the FP64 pipe (kDigitRowSpan)
 __device__ __forceinline__ int blk_exponent(const BlockedArgs& a, int b) { return a.state[4 * b + 3] >> 1; }
 __device__ __forceinline__ bool blk_plain64(const BlockedArgs& a, int b) { return (a.state[4 * b + 3] & 1) != 0; }
+
+// whether round r's pair step of (bi, bj) takes the cross pairs only (not from
+// a given V, close to convergence: full sweeps save an outer one there; not with
+// rows of different sizes: cross_only)
+template <class T, int NB>
+__device__ __forceinline__ bool blk_cross(const BlockedArgs& a, const BlkShape& s, int b, int r, int bi, int bj) {
+    return NB >= 16 && !a.V0 && !blk_plain64(a, b) && cross_only<T>(a.inner_sweeps, s.l, r, bi, bj);
+}
 
 // ---- load: W = A * 2^-ex (or A^H), padded; V = I; status -------------------
 // ---- S2, real FP32: register tiles --------------------------------------------
@@ -461,7 +462,7 @@ __global__ void __launch_bounds__(GT) blk_heevj(const BlockedArgs a, int r) {
     }
     __syncthreads();
     const int seen = inner_jacobi<T, NB, GT>(G, J, tb, (Real<T>)a.tol, max(a.inner_sweeps, 1), tid, 1, NoBackground(),
-                                             nullptr, (a.flags & 256) != 0, blk_cross<T, NB>(a, sh, r, bi, bj));
+                                             nullptr, (a.flags & 256) != 0, blk_cross<T, NB>(a, sh, b, r, bi, bj));
     T* Jg = static_cast<T*>(a.J) + sh.oJ + (long long)q * TWO * TWO;
     for (int e = tid; e < TWO * TWO; e += GT) Jg[(e % TWO) + (e / TWO) * TWO] = J[(e % TWO) + (e / TWO) * LDG];
     if (tid == 0) {

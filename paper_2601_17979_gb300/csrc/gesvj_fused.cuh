@@ -396,7 +396,7 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
                 // S3: inner Jacobi sweeps on G (round-robin over the 2nb indices)
                 int seen;
                 stepped = true;
-                const bool cross = (NB >= 16 || pre) && !a.V0 && cross_only<T>(a.inner_sweeps, a.l, r, bi, bj);
+                const bool cross = (NB >= 16 || pre) && !a.V0 && !plain64 && cross_only<T>(a.inner_sweeps, a.l, r, bi, bj);
                 const int isw = a.inner_sweeps > 0 ? a.inner_sweeps : 1;
                 if constexpr (kDefer) {
                     int ns = 0;

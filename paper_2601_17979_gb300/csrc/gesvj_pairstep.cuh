@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kPairThreads, pair_min_blocks<T>()) blk_pairst
 
     // ---- S3: one sweep of the inner Jacobi solver (as blk_heevj) ------------
     const int seen = inner_jacobi<T, NB, NT>(G, J, tb, (float)a.tol, max(a.inner_sweeps, 1), tid, 1, NoBackground(),
-                                             nullptr, (a.flags & 256) != 0, blk_cross<T, NB>(a, sh, r, bi, bj));
+                                             nullptr, (a.flags & 256) != 0, blk_cross<T, NB>(a, sh, b, r, bi, bj));
     if (tid == 0) {
         *pf = seen > 0;
         if (seen > 0) a.state[4 * b + 1] = 1;

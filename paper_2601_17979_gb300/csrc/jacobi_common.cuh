@@ -323,6 +323,9 @@ __device__ __forceinline__ bool entry_fires(const T* G, int p, int q, Real<T> to
 // Complex128 keeps them up to 3 blocks (2,000 of 20 x 20, nb = 8: 11.8 ms against
 // 12.5; at 4 blocks 500 of 64 x 64 29.2 ms full, 26.7 with cross pairs).
 // Sweeps on 256 x 256 FP32: 11.3 full, 11.6 with cross pairs, half the steps.
+// FP64 and complex128 matrices with rows of different sizes (kDigitRowSpan) keep
+// full sweeps, the caller sees to that: Kahan's matrix 200 x 140 takes 10 sweeps
+// with them and 16 with cross pairs.
 template <class T>
 __device__ __forceinline__ bool cross_only(int inner_sweeps, int l, int r, int bi, int bj) {
     constexpr bool kSingle = sizeof(Real<T>) == 4, kC128 = sizeof(T) == 16;

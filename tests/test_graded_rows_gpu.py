@@ -90,3 +90,25 @@ def test_small_values_of_graded_rows(m, n, path, nb, dtype):
         S = r.S[k].cpu().numpy()
         rel = (np.abs(S - ref[k]) / ref[k]).max()
         assert int(r.info[k]) == 0 and rel <= 50 * min(m, n) * u * cond[k], (k, int(r.info[k]), rel / u, cond[k])
+
+
+def kahan(m, n, theta=1.2):
+    s, c = np.sin(theta), np.cos(theta)
+    return (s ** np.arange(m))[:, None] * (np.eye(m, n) - c * np.triu(np.ones((m, n)), 1))
+
+
+# Cross-only sweeps take more of them on such matrices (Kahan's 200 x 140: 16
+# against 10), so these run the sweeps of inner_sweeps = 1: the same bits.
+@pytest.mark.parametrize("dtype", [np.float64, np.complex128])
+@pytest.mark.parametrize("path", ["auto", "blocked", "slots"])
+@pytest.mark.parametrize("m,n", [(64, 64), (96, 70), (200, 140)])
+def test_graded_rows_take_full_sweeps(m, n, path, dtype):
+    rng = np.random.default_rng(m)
+    mats = [kahan(m, n).astype(dtype), row_graded(rng, m, n, 30, dtype)[0]]
+    T = [torch.from_numpy(np.asfortranarray(x)).cuda() for x in mats]
+    kw = dict(path="persistent", flags=bsvd.FLAG_NO_ONCHIP) if path == "slots" else dict(path=path)
+    r, f = bsvd.gesvj_batched(T, **kw), bsvd.gesvj_batched(T, inner_sweeps=1, **kw)
+    torch.cuda.synchronize()
+    for k in range(len(mats)):
+        assert int(r.info[k]) == 0 and int(r.sweeps[k]) == int(f.sweeps[k]), (k, int(r.sweeps[k]), int(f.sweeps[k]))
+        assert torch.equal(r.S[k], f.S[k]) and torch.equal(r.U[k], f.U[k]) and torch.equal(r.V[k], f.V[k])
