@@ -239,12 +239,21 @@ __device__ __forceinline__ float phase_times(float g, float, float s) {
 __device__ __forceinline__ double phase_times(double g, double, double s) {
     return __longlong_as_double(__double_as_longlong(s) ^ (__double_as_longlong(g) & (long long)0x8000000000000000ull));
 }
+// (g near the bottom of the range is scaled up exactly first: 1 / a could overflow,
+// and |g| of a denormal g is not accurate enough for a unitary rotation)
 __device__ __forceinline__ float2 phase_times(float2 g, float a, float s) {
-    if (a < 1e-37f) return make_float2(g.x / a * s, g.y / a * s);   // 1 / a would overflow
+    if (a < 1e-30f) {
+        g = make_float2(g.x * 0x1p96f, g.y * 0x1p96f);
+        a = hypotf(g.x, g.y);
+    }
     const float k = s * (1.0f / a);
     return make_float2(g.x * k, g.y * k);
 }
 __device__ __forceinline__ double2 phase_times(double2 g, double a, double s) {
+    if (a < 1e-290) {
+        g = make_double2(g.x * 0x1p512, g.y * 0x1p512);
+        a = hypot(g.x, g.y);
+    }
     const double k = s * (1.0 / a);
     return make_double2(g.x * k, g.y * k);
 }

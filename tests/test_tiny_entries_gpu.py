@@ -41,3 +41,25 @@ def test_denormal_entries(path, m, n, nb, dtype):
         assert int(r.info[i]) == 0, i
         meas = checks.measures(A, r.S[i].cpu().numpy(), r.U[i].cpu().numpy(), r.V[i].cpu().numpy(), ref[i])
         assert checks.violations(meas, u) == [], (i, meas)
+
+
+@pytest.mark.parametrize("dtype,low", [(np.complex64, 62), (np.complex128, 508)])
+@pytest.mark.parametrize("m,n,nb", [(60, 48, 16), (30, 24, 8), (40, 40, 4), (90, 40, 16)])
+@pytest.mark.parametrize("path", ["auto", "blocked"])
+def test_rotations_of_denormal_gram_entries(path, m, n, nb, dtype, low):
+    """Short columns whose Gram entries are near the bottom of the range or
+    denormal: the rotations stay unitary, so V and the product keep their
+    bounds (U's columns then have no accurate Gram entries to go by)."""
+    rng = np.random.default_rng(m)
+    u = checks.unit_roundoff(dtype)
+    mats = []
+    for k in (low, low + 4, low + 8, low + 12):
+        A = rng.standard_normal((m, n)) + 1j * rng.standard_normal((m, n))
+        A[:, n // 2:] *= 2.0 ** -k
+        mats.append(A.astype(dtype))
+        mats.append((A.conj() * 2.0 ** -np.linspace(0, 3, n).round()).astype(dtype))
+    r = bsvd.gesvj_batched([torch.from_numpy(np.asfortranarray(x)).cuda() for x in mats], path=path, nb=nb)
+    torch.cuda.synchronize()
+    for i, A in enumerate(mats):
+        meas = checks.measures(A.astype(np.complex128), r.S[i].cpu().numpy(), r.U[i].cpu().numpy(), r.V[i].cpu().numpy())
+        assert not {"resid", "orth_v"} & set(checks.violations(meas, u)), (i, meas)
