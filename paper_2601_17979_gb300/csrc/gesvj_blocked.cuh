@@ -53,8 +53,8 @@ __device__ __forceinline__ bool blk_skip(const BlockedArgs& a, int b) {
     return st < 0 || (a.masks && st == 0);
 }
 
-// state[3]: the exponent ex, doubled, plus one where the rows' sizes keep the
-// matrix on the FP64 pipe (kDigitRowSpan)
+// state[3]: the exponent ex, doubled, plus one where the matrix keeps the FP64 pipe
+// (kDigitRowSpan, short_column)
 __device__ __forceinline__ int blk_exponent(const BlockedArgs& a, int b) { return a.state[4 * b + 3] >> 1; }
 __device__ __forceinline__ bool blk_plain64(const BlockedArgs& a, int b) { return (a.state[4 * b + 3] & 1) != 0; }
 
@@ -337,7 +337,8 @@ __global__ void __launch_bounds__(kBlkThreads) blk_load(const BlockedArgs a) {
         __shared__ int span_s[2 * NW];
         __syncthreads();
         const int span = row_span<T, NT>(W, 1, M, M, N, span_s);
-        if (tid == 0) a.state[4 * b + 3] = 2 * ex + (span > kDigitRowSpan ? 1 : 0);
+        const bool shortc = short_column<T, NT>(W, M, M, N);
+        if (tid == 0) a.state[4 * b + 3] = 2 * ex + (span > kDigitRowSpan || shortc ? 1 : 0);
     }
 }
 

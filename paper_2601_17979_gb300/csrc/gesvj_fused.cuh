@@ -316,7 +316,7 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
     bool pre = false;
     const bool try_pre = preconditioned<T, NB>(a);
     const int span = kSplit || try_pre ? row_span<T, NT>(W, 1, ldw, M0, N, reinterpret_cast<int*>(smem + a.offG)) : 0;
-    const bool plain64 = kSplit && span > kDigitRowSpan;
+    bool plain64 = kSplit && span > kDigitRowSpan;
     if (try_pre && span <= pre_row_span(M0, N)) {
         if constexpr (std::is_same<T, float>::value)
             pre = precondition_f32<NT>(W, ldw, M0, N, needVs ? Vs : nullptr, ldvs, wantWout ? Y : nullptr, ldy,
@@ -326,6 +326,8 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
                                       PreScratch<T>(smem + a.offG, N));
         if (pre) M = N;
     }
+    if constexpr (kSplit)                                      // (a preconditioned matrix has no short columns)
+        if (!pre && !plain64) plain64 = short_column<T, NT>(W, ldw, M, N);
 
     // ---- sweeps -----------------------------------------------------------------
     const R tol = (R)a.tol;

@@ -636,8 +636,25 @@ __device__ __forceinline__ void update_f64_split(T* W, long long ldw, int rowsW,
 // units of u, with digits and on the FP64 pipe: D over 2^6 45 and 45, 2^10 85 and
 // 49, 2^20 608 and 67, 2^40 5.8e3 and 76, 2^100 2.4e6 and 76.  So a matrix whose
 // rows span more than 2^6 keeps the FP64 pipe (not inlined: the digit path keeps
-// its registers).
+// its registers).  So does a matrix with a column shorter than 2^-400: the update
+// scales columns by their norms, which the Gram block's diagonal gives down to
+// 2^-511 only; a column of 2^-540 kept 24 bits per update and one of 2^-570 none.
 constexpr int kDigitRowSpan = 6;
+
+// Whether a column of W (M x N, largest entry between 1 and 2) is shorter than
+// 2^-400 and not zero.  Called by all NT threads; synchronised.
+template <class T, int NT>
+__device__ __forceinline__ bool short_column(const T* W, long long ldw, int M, int N) {
+    const int lane = threadIdx.x & 31;
+    bool any = false;
+    for (int j = threadIdx.x >> 5; j < N; j += NT / 32) {
+        double mx = 0;
+        for (int r = lane; r < M; r += 32) mx = fmax(mx, maxabs(W[r + j * ldw]));
+        mx = warp_max(mx);
+        any |= mx > 0 && mx < 0x1p-400;
+    }
+    return __syncthreads_or(any) != 0;
+}
 
 template <class T, int NB, int GT>
 __device__ __noinline__ void gram_f64_fma(const T* W, long long ldw, int M, int cbi, int cbj, T* G, int ldg, int gt) {

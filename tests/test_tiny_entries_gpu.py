@@ -63,3 +63,35 @@ def test_rotations_of_denormal_gram_entries(path, m, n, nb, dtype, low):
     for i, A in enumerate(mats):
         meas = checks.measures(A.astype(np.complex128), r.S[i].cpu().numpy(), r.U[i].cpu().numpy(), r.V[i].cpu().numpy())
         assert not {"resid", "orth_v"} & set(checks.violations(meas, u)), (i, meas)
+
+
+@pytest.mark.parametrize("dtype", [np.float64, np.complex128])
+@pytest.mark.parametrize("m,n,nb", [(48, 32, 16), (70, 48, 16), (64, 64, 16), (30, 16, 8), (40, 40, 8)])
+@pytest.mark.parametrize("path", ["auto", "blocked", "slots", "mixed"])
+def test_columns_short_of_the_squares(path, m, n, nb, dtype):
+    """Dense columns of 2^-520, 2^-560 and 2^-600 (their squares underflow) in one
+    block pair with columns of size one: as on the FP64 pipe (nb = 4), which
+    orthogonalises the first and leaves the others as they are."""
+    rng = np.random.default_rng(m + n)
+    mats = []
+    for at in ([0, 1, 2], [n - 1, n // 2, 3], [n - 3, n - 2, n - 1]):
+        A = rng.standard_normal((m, n)) + (1j * rng.standard_normal((m, n)) if dtype == np.complex128 else 0)
+        A[:, at] *= 2.0 ** -np.array([520, 560, 600])
+        mats.append(A.astype(dtype))
+    T = [torch.from_numpy(np.asfortranarray(x)).cuda() for x in mats]
+
+    def call(nb):
+        if path == "slots":
+            return bsvd.gesvj_batched(T, path="persistent", nb=nb, flags=bsvd.FLAG_NO_ONCHIP)
+        return bsvd.gesvj_batched(T, prec="mixed", nb=nb) if path == "mixed" else bsvd.gesvj_batched(T, path=path, nb=nb)
+    r, p = call(nb), call(4)
+    torch.cuda.synchronize()
+    # a pair is rotated to 30 u of orthogonal, so S differs by less than n 30 u of itself; doubled
+    tol = 2 * 30 * n * checks.U64
+    for k, A in enumerate(mats):
+        S, P = r.S[k].cpu().numpy(), p.S[k].cpu().numpy()
+        assert int(r.info[k]) == 0 and int(p.info[k]) == 0
+        rel = np.abs(S - P) / P
+        assert rel[-3:].max() <= tol, (k, S[-3:], P[-3:])
+        meas = checks.measures(A, S, r.U[k].cpu().numpy(), r.V[k].cpu().numpy(), P)
+        assert not {"sigma_err", "resid", "orth_v"} & set(checks.violations(meas, checks.U64)), (k, meas)
