@@ -193,6 +193,19 @@ __device__ __forceinline__ bool preconditioned(const FusedArgs& a) {
     return NB == 16 || (!kReal32 && a.N < 48 && (!kSingle || a.N > 32));
 }
 
+// W = 2^-ex A (or A^H when m < n) once more, after a QR that came to nothing.
+// Synchronised.
+template <class T, int NT>
+__device__ __noinline__ void reload_w(const T* A, int lda, int m, int n, int ex, T* W, int ldw) {
+    for (int e = threadIdx.x; e < m * n; e += NT) {
+        const int i = e % m, j = e / m;
+        const T x = A[i + (long long)j * lda];
+        T* w = m < n ? &W[j + (long long)i * ldw] : &W[i + (long long)j * ldw];
+        *w = scalb_s(m < n ? conj_s(x) : x, -ex);
+    }
+    __syncthreads();
+}
+
 // Real FP32 keeps two CTAs per SM (its shared memory allows them).
 template <class T>
 constexpr int fused_min_blocks() { return std::is_same<T, float>::value ? 2 : 1; }
@@ -318,13 +331,16 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
     const int span = kSplit || try_pre ? row_span<T, NT>(W, 1, ldw, M0, N, reinterpret_cast<int*>(smem + a.offG)) : 0;
     bool plain64 = kSplit && span > kDigitRowSpan;
     if (try_pre && span <= pre_row_span(M0, N)) {
+        Pre st;
         if constexpr (std::is_same<T, float>::value)
-            pre = precondition_f32<NT>(W, ldw, M0, N, needVs ? Vs : nullptr, ldvs, wantWout ? Y : nullptr, ldy,
+            st = precondition_f32<NT>(W, ldw, M0, N, needVs ? Vs : nullptr, ldvs, wantWout ? Y : nullptr, ldy,
                                        PreF32(smem + a.offG, M0, N));
         else
-            pre = precondition<T, NT>(W, ldw, M0, N, needVs ? Vs : nullptr, ldvs, nullptr, 0, wantWout ? Y : nullptr, ldy,
+            st = precondition<T, NT>(W, ldw, M0, N, needVs ? Vs : nullptr, ldvs, nullptr, 0, wantWout ? Y : nullptr, ldy,
                                       PreScratch<T>(smem + a.offG, N));
+        pre = st == Pre::kDone;
         if (pre) M = N;
+        if (st == Pre::kDeficient) reload_w<T, NT>(A, lda, a.m, a.n, ex, W, ldw);
     }
     if constexpr (kSplit)                                      // (a preconditioned matrix has no short columns)
         if (!pre && !plain64) plain64 = short_column<T, NT>(W, ldw, M, N);

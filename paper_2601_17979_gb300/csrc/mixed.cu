@@ -490,7 +490,7 @@ __global__ void __launch_bounds__(kMxThreads) mx_precondition(const MixedArgs a)
     int wide = 0;
     for (int e = tid; e < M * N; e += NT) wide |= !(fabs(Ah[e]) < 1e100);
     if (!__syncthreads_or(wide) && !a.plain64[b] &&
-        precondition<double, NT>(Ah, M, M, N, Vn, N, V, N, nullptr, 0, PreScratch<double>(smem, N)))
+        precondition<double, NT>(Ah, M, M, N, Vn, N, V, N, nullptr, 0, PreScratch<double>(smem, N)) == Pre::kDone)
         return;
     __syncthreads();
     for (int e = tid; e < N * N; e += NT) {

@@ -64,6 +64,18 @@ template <class R> constexpr R kPreTiny = R(0);         // a reflection of a sho
 template <> constexpr float kPreTiny<float> = 1e-34f;
 template <> constexpr double kPreTiny<double> = 1e-290;
 
+// A column of which the QR leaves less than 2^-32 of its norm in single
+// precision, 2^-64 in double (squares here): rounding of rounding, as in matrices
+// of exact low rank, whose equal columns round equally.  From such an R the sweeps
+// get a chain of columns u, u^2, u^3 .. of the largest, whose squares underflow in
+// single precision: constant, checkerboard and block-constant FP32 and complex64
+// matrices ran into the sweep limit.  They keep the plain start.
+template <class R> constexpr R kPreDeficient = R(0);
+template <> constexpr float kPreDeficient<float> = 0x1p-64f;
+template <> constexpr double kPreDeficient<double> = 0x1p-128;
+
+enum class Pre { kNone, kDone, kDeficient };               // unchanged, done, W destroyed and V unchanged
+
 // Scratch of one matrix, N entries each (two sets of column norms: a step
 // reads one while it writes the other).  v0 has at least eight: row_span's two
 // ints a warp of up to 256 threads.
@@ -309,9 +321,9 @@ __device__ __forceinline__ void sort_columns(T* W, int ldw, int M, int N, const 
 // V (N x N, unless null) becomes V0 P Z (V0 null: I); the reflections of Q go
 // to refl (M x N, scaled so that tau = 1; null: dropped).  Called by all NT
 // threads after W is complete and synchronised; returns synchronised.
-// The caller has seen to it that the rows span at most pre_row_span.  Returns false,
-// with nothing changed, when a column is too short to square safely (or zero), and
-// in single precision when the spectrum is flat.
+// The caller has seen to it that the rows span at most pre_row_span.  kNone when a
+// column is too short to square safely (or zero), and in single precision when the
+// spectrum is flat; kDeficient when a column is left with nothing.
 //
 // Double precision picks each column by its remaining norm (QR with column
 // pivoting: 128 x 64 with kappa = 1e6 then takes 6.3 sweeps, 7.1 without).
@@ -322,6 +334,9 @@ __device__ __forceinline__ void qr_steps(T* W, int ldw, int M, int N, const PreS
     using R = Real<T>;
     constexpr bool kPivot = sizeof(R) == 8;
     const int tid = threadIdx.x, lane = tid & 31;
+    R* const own = reinterpret_cast<R*>(sc.v0);            // squared column norms by the caller's column, for the end
+    for (int j = tid; j < N; j += NT) own[j] = sc.nrm2[j];
+    __syncthreads();
     for (int k = 0; k < N; ++k) {
         const R* cur = sc.nrm2 + (k & 1) * N;
         R* next = sc.nrm2 + ((k + 1) & 1) * N;
@@ -374,7 +389,7 @@ __device__ __forceinline__ void qr_steps(T* W, int ldw, int M, int N, const PreS
 }
 
 template <class T, int NT>
-__device__ __forceinline__ bool precondition(T* W, int ldw, int M, int N, T* V, int ldv, const T* V0, long long ldv0,
+__device__ __forceinline__ Pre precondition(T* W, int ldw, int M, int N, T* V, int ldv, const T* V0, long long ldv0,
                                              T* refl, long long ldr, const PreScratch<T>& sc) {
     using R = Real<T>;
     constexpr int NW = NT / 32;
@@ -388,15 +403,20 @@ __device__ __forceinline__ bool precondition(T* W, int ldw, int M, int N, T* V, 
     __syncthreads();
     bool small = false;
     for (int j = lane; j < N; j += 32) small |= !(sc.nrm2[j] > kPreNormMin<R>);
-    if (__any_sync(0xffffffffu, small)) { __syncthreads(); return false; }   // uniform: every warp reads all norms
+    if (__any_sync(0xffffffffu, small)) { __syncthreads(); return Pre::kNone; }   // uniform: every warp reads all norms
     if constexpr (sizeof(R) == 4)
-        if (M <= 2 * N && flat_spectrum<T, NT>(W, ldw, M, N, sc.nrm2, sc.v0, sc.tau)) return false;
+        if (M <= 2 * N && flat_spectrum<T, NT>(W, ldw, M, N, sc.nrm2, sc.v0, sc.tau)) return Pre::kNone;
     if constexpr (sizeof(R) == 4)
         sort_columns<T, NT>(W, ldw, M, N, sc.nrm2, sc.perm, reinterpret_cast<int*>(sc.v0), reinterpret_cast<int*>(sc.diag));
 
     // ---- W P = Q R ---------------------------------------------------------------
     if (eight_lanes<NT>(N)) qr_steps<T, NT, 8>(W, ldw, M, N, sc);
     else                    qr_steps<T, NT, 4>(W, ldw, M, N, sc);
+    bool left = true;
+    for (int k = lane; k < N; k += 32)
+        left &= sq_acc(sc.tau[k] > 0 ? sc.diag[k] : W[k + (long long)k * ldw], R(0)) >
+                rmul(kPreDeficient<R>, reinterpret_cast<const R*>(sc.v0)[sc.perm[k]]);
+    if (!__all_sync(0xffffffffu, left)) { __syncthreads(); return Pre::kDeficient; }   // uniform: every warp reads all
     if (refl)
         for (int k = warp; k < N; k += NW) {
             const R f = sqrt_r(sc.tau[k]);
@@ -470,7 +490,7 @@ __device__ __forceinline__ bool precondition(T* W, int ldw, int M, int N, T* V, 
             else if (i + 1 < N && sc.tau[i] > 0) W[i + (long long)j * ldw] = conj_s(rscale(sc.diag[i], R(-1)));
         }
     __syncthreads();
-    return true;
+    return Pre::kDone;
 }
 
 // ---- real FP32: the same steps on float4 ------------------------------------------
@@ -676,7 +696,7 @@ __device__ __forceinline__ void look_ahead_f32(float* x, int sx, int k, int n, i
 // precondition for real FP32 (W's columns and V's on 16-byte boundaries, zero
 // in the rows that pad them to a multiple of four).
 template <int NT>
-__device__ __forceinline__ bool precondition_f32(float* W, int ldw, int M, int N, float* V, int ldv, float* refl,
+__device__ __forceinline__ Pre precondition_f32(float* W, int ldw, int M, int N, float* V, int ldv, float* refl,
                                                  long long ldr, const PreF32& sc) {
     constexpr int NW = NT / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, mp = PreF32::f32_buf(M), np = PreF32::f32_buf(N);
@@ -689,8 +709,8 @@ __device__ __forceinline__ bool precondition_f32(float* W, int ldw, int M, int N
     __syncthreads();
     bool small = false;
     for (int j = lane; j < N; j += 32) small |= !(sc.nrm2[j] > kPreNormMin<float>);
-    if (__any_sync(0xffffffffu, small)) { __syncthreads(); return false; }   // uniform: every warp reads all norms
-    if (flat_spectrum<float, NT>(W, ldw, M, N, sc.nrm2, sc.v, sc.tau)) return false;
+    if (__any_sync(0xffffffffu, small)) { __syncthreads(); return Pre::kNone; }   // uniform: every warp reads all norms
+    if (flat_spectrum<float, NT>(W, ldw, M, N, sc.nrm2, sc.v, sc.tau)) return Pre::kNone;
     sort_columns<float, NT>(W, ldw, M, N, sc.nrm2, sc.perm, sc.tmp, sc.tmp + N);
 
     if (warp == 0) make_reflection_f32(W, 1, 0, M, mp, sc.v, sc.tau, sc.ph);
@@ -705,13 +725,19 @@ __device__ __forceinline__ bool precondition_f32(float* W, int ldw, int M, int N
         } else {
             if (eight_lanes<NT>(N)) reflect_columns_f32<NT, 8>(W, ldw, k, M, k + 2, N, v, tau, 1);
             else                    reflect_columns_f32<NT, 4>(W, ldw, k, M, k + 2, N, v, tau, 1);
-            if (refl) {
-                const float f = sqrtf(tau);
-                for (int r = k + tid - 32; r < M; r += NT - 32) refl[r + (long long)k * ldr] = rmul(v[r], f);
-            }
         }
         __syncthreads();
     }
+    bool left = true;
+    for (int k = lane; k < N; k += 32)
+        left &= sq_acc(sc.tau[k] > 0.f ? sc.ph[k] : W[k + k * ldw], 0.f) > rmul(kPreDeficient<float>, sc.nrm2[sc.perm[k]]);
+    if (!__all_sync(0xffffffffu, left)) { __syncthreads(); return Pre::kDeficient; }   // uniform: every warp reads all
+    if (refl)
+        for (int k = warp; k < N; k += NW) {
+            const float f = sqrtf(sc.tau[k]);
+            for (int r = k + lane; r < M; r += 32)
+                refl[r + (long long)k * ldr] = rmul(r == k ? W[r + k * ldw] + sc.ph[k] : W[r + k * ldw], f);
+        }
     if (V)
         for (int k = warp; k < N; k += NW) {
             const int c = sc.perm[k];
@@ -828,7 +854,7 @@ __device__ __forceinline__ bool precondition_f32(float* W, int ldw, int M, int N
             else if (i + 1 < N && sc.tau[i] > 0.f) W[i + j * ldw] = -sc.ph[i];
         }
     __syncthreads();
-    return true;
+    return Pre::kDone;
 }
 
 // apply_q for real FP32; buf: kQPanel buffers of f32_buf(M) floats.  A column
