@@ -339,7 +339,10 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
             st = precondition<T, NT>(W, ldw, M0, N, needVs ? Vs : nullptr, ldvs, nullptr, 0, wantWout ? Y : nullptr, ldy,
                                       PreScratch<T>(smem + a.offG, N));
         pre = st == Pre::kDone;
-        if (pre) M = N;
+        if (pre) {
+            M = N;
+            plain64 = false;                                   // L is small relative to each column already
+        }
         if (st == Pre::kDeficient) reload_w<T, NT>(A, lda, a.m, a.n, ex, W, ldw);
     }
     if constexpr (kSplit)                                      // (a preconditioned matrix has no short columns)

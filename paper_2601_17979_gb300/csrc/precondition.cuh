@@ -232,11 +232,15 @@ __device__ __forceinline__ bool eight_lanes(int N) { return NT <= 128 && 8 * N <
 // smallest singular values, which the plain start keeps.  Median over 24
 // matrices D B, FP64 64 x 64, of the largest relative error of a singular value,
 // in units of u, against that of the plain start: D over 2^4 (rows spanning five
-// orders) 74 and 57, 2^5 96 and 57, 2^6 179 and 69, 2^8 398 and 62, 2^10 848 and 74;
-// with two rows a column no more than the plain start's up to 2^10, so those may
-// span one order more (geometric spectra of few columns do by chance: 1000 x 16
-// down to 1e-3 four to six).
-__host__ __device__ constexpr int pre_row_span(int M, int N) { return M >= 2 * N ? 6 : 5; }
+// orders) 74 and 57, 2^5 96 and 57, 2^6 179 and 69, 2^8 398 and 62, 2^10 848 and 74.
+// With two rows a column the larger rows alone determine the matrix as a rule, and
+// nothing is lost: 128 x 64, D over 2^6 86 and 100, over 2^7 91 and 102; where the
+// small rows carry an eighth of the dimensions by themselves up to 1.4 times the
+// plain start's (100 x 48, 2^6: 103 and 72).  Such matrices may span seven orders,
+// at which even a square one stays within a factor of three (179 and 69):
+// geometric spectra reach them by chance, and 3 % of 128 x 64 matrices down to 1e-6
+// on the plain start took a tenth of the time of a batch of 4,000 (95.0 ms, 84.7 so).
+__host__ __device__ constexpr int pre_row_span(int M, int N) { return M >= 2 * N ? 7 : 5; }
 
 // Whether the spectrum is so flat that the sweeps gain little from the
 // preconditioner: the participation ratio (sum sigma^2)^2 / (N sum sigma^4)
