@@ -278,7 +278,7 @@ bsvd_status plan_mixed(int max_smem, char t, int m, int n, int batch, bool wantU
     mp.r32.path = BSVD_PATH_AUTO;
     // FP32 sweeps: FMA tiles / FP64 rotations, and how the sweep loop runs
     // (no graph, host checks, host-replayed graph), as the caller asked
-    mp.r32.flags = r.flags & (128 | 256 | 8 | 16 | 2048 | 4096);
+    mp.r32.flags = (r.flags & (128 | 256 | 8 | 16 | 2048 | 4096)) | bsvd::kFlagVOnly;
     mp.r32.inner_sweeps = r.inner_sweeps ? 1 : 0;
     mp.r32.prec = BSVD_PREC_NATIVE;
     mp.r64 = r;

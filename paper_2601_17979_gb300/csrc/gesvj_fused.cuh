@@ -60,7 +60,9 @@ struct FusedArgs {
 // bsvd_opts.flags bits read by the kernels: 0 no Newton-Schulz step on V;
 // 7 real FP32 Gram and update on the FMA pipes (register tiles) instead of
 // the tensor cores; 8 single-precision rotations and pair test in FP64.
-enum : int { kFlagNoVCorrection = 1, kFlagF32Ffma = 128, kFlagWideAngles = 256 };
+// Not a caller's: kFlagVOnly, set for the mixed path's single-precision solve, of
+// which only an orthonormal V is kept.
+enum : int { kFlagNoVCorrection = 1, kFlagF32Ffma = 128, kFlagWideAngles = 256, kFlagVOnly = 1 << 16 };
 
 // Shared-memory bytes of one thread group's scratch (G, J, rotation table).
 // Working shape and leading dimensions of one matrix: M >= N (A^H when
@@ -330,7 +332,7 @@ __device__ __forceinline__ void fused_solve(const FusedArgs& a, const int mid, c
     const bool try_pre = preconditioned<T, NB>(a);
     const int span = kSplit || try_pre ? row_span<T, NT>(W, 1, ldw, M0, N, reinterpret_cast<int*>(smem + a.offG)) : 0;
     bool plain64 = kSplit && span > kDigitRowSpan;
-    if (try_pre && span <= pre_row_span(M0, N)) {
+    if (try_pre && span <= ((a.flags & kFlagVOnly) ? kPreVOnlySpan : pre_row_span(M0, N))) {
         Pre st;
         if constexpr (std::is_same<T, float>::value)
             st = precondition_f32<NT>(W, ldw, M0, N, needVs ? Vs : nullptr, ldvs, wantWout ? Y : nullptr, ldy,

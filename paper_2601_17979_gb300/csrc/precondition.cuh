@@ -241,6 +241,10 @@ __device__ __forceinline__ bool eight_lanes(int N) { return NT <= 128 && 8 * N <
 // geometric spectra reach them by chance, and 3 % of 128 x 64 matrices down to 1e-6
 // on the plain start took a tenth of the time of a batch of 4,000 (95.0 ms, 84.7 so).
 __host__ __device__ constexpr int pre_row_span(int M, int N) { return M >= 2 * N ? 7 : 5; }
+// Where only V is kept, and FP64 sweeps on A V decide the values (kFlagVOnly): a
+// fifteenth of the 96 x 96 matrices of a clustered spectrum span six orders, and
+// their plain start cost the mixed path 2 ms of 95 on 2,000 of them.
+constexpr int kPreVOnlySpan = 10;
 
 // Whether the spectrum is so flat that the sweeps gain little from the
 // preconditioner: the participation ratio (sum sigma^2)^2 / (N sum sigma^4)

@@ -133,3 +133,15 @@ def test_tall_matrices_of_seven_orders_keep_the_start(m, n, dtype):
     A = torch.from_numpy(np.stack(mats)).cuda()
     sweeps, full = int(bsvd.gesvj(A, nb=16).sweeps.sum()), int(bsvd.gesvj(A, nb=16, inner_sweeps=1).sweeps.sum())
     assert sweeps < full, (sweeps, full)
+
+
+# The mixed path keeps only V of its single-precision solve, which may start
+# preconditioned up to ten orders: the values are the FP64 sweeps' all the same.
+@pytest.mark.parametrize("dtype", [np.float64, np.complex128])
+@pytest.mark.parametrize("span", [5, 7, 9])
+@pytest.mark.parametrize("n", [40, 64, 96])
+def test_mixed_values_of_moderately_graded_rows(n, span, dtype):
+    rng = np.random.default_rng(n + span)
+    mats = [row_graded(rng, n, n, span, dtype)[0] for _ in range(16)]
+    err, plain = relative_errors(mats, prec="mixed"), relative_errors(mats, inner_sweeps=1)
+    assert np.median(err) <= 3 * np.median(plain) + n * checks.unit_roundoff(dtype), (np.median(err), np.median(plain))
