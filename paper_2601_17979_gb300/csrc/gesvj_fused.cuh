@@ -180,8 +180,14 @@ __device__ __forceinline__ long long pre_bytes(int M, int N) {
 //   complex128 40 x 40 17.8 -> 15.8, complex64 97 x 45 13.5 -> 12.5; but FP32
 //   32 x 32 2.3 -> 2.4 and complex64 32 x 32 4.2 -> 4.6;
 //   one pair of blocks (at most 2 nb columns): complex128 24 x 16 1.48 -> 1.76,
-//   FP32 100 x 16 0.85 -> 1.1, worth it only for the rows QR takes off tall
-//   FP64 (1000 x 16, 1,000: 13.1 -> 7.9).
+//   FP32 100 x 16 0.85 -> 1.1.  FP64 with nb = 8, normal entries and sigma down to
+//   1e-3: 1,000 of 128 x 16 1.05 -> 1.39 and 1.41 -> 1.19, one 0.39 -> 0.49 and 0.52 ->
+//   0.41; 384 x 16 1.98 -> 2.53 and 2.59 -> 2.33; 1000 x 16 7.24 -> 8.07 and 9.66 ->
+//   7.51; 288 x 12 1.31 -> 1.42 and 1.65 -> 1.23; 640 x 12 3.12 -> 3.05 and 3.90 ->
+//   2.74: graded spectra gain what flat ones lose.  From 24 rows a column on no call
+//   is slower than it was without the start and the digits (128 x 16 0.41 for one,
+//   384 x 16 0.76); nb = 16 loses more than it gains (256 x 32 6.99 -> 10.99 and
+//   10.56 -> 9.70).
 // Single precision up to 160 columns (on chip about 128): beyond, on global
 // slots, it would move FP32 results as noted at cross_only.  A caller that sets
 // inner_sweeps gets the sweeps of the plain method from the start, and a start
@@ -190,7 +196,7 @@ template <class T, int NB>
 __device__ __forceinline__ bool preconditioned(const FusedArgs& a) {
     constexpr bool kSingle = sizeof(Real<T>) == 4, kReal32 = std::is_same<T, float>::value;
     if (a.inner_sweeps != 0 || a.V0 || NB < 8 || pre_bytes<T>(a.M, a.N) > a.groupBytes) return false;
-    if (a.l == 2 && (kSingle || a.M < 8 * a.N)) return false;
+    if (a.l == 2 && (kSingle || NB != 8 || a.M < 24 * a.N)) return false;
     if (kSingle && a.N > 160) return false;
     return NB == 16 || (!kReal32 && a.N < 48 && (!kSingle || a.N > 32));
 }
