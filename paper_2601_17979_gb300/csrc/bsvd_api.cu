@@ -687,7 +687,19 @@ bsvd_status plan_persistent(bsvd_handle h, char t, int sms, int max_smem, const 
         const int nb = persist_nb(h, t, m[id], n[id], wantU, wantV, opts);
         if (!fused_nb(nb)) return BSVD_ERR_NOT_IMPLEMENTED;
         const size_t wv = ops.slot(nb, m[id], n[id]) * ops.elt;
-        const bool onchip = allow_onchip && ops.smem(nb, wv, pp.maxN) <= budget;
+        // Real FP64 with nb = 16 holds one CTA an SM on chip (registers) and two in
+        // global slots: past one matrix an SM the shapes that only fit beside the
+        // digits' smaller groups (fused_group_spare) stay in slots.  61 x 61 to 64 x 64,
+        // on chip and in slots: 152 of them 3.53 and 3.84 ms, 304 6.71 and 5.51, 2,000
+        // 45.3 and 36.2.  (nb = 8 from 22 columns and complex128 are as fast on chip.)
+        size_t spare = 0;
+        if (t == 'd' && nb == 16 && pp.count > sms) {
+            FusedArgs fa;
+            int threads = 0;
+            ops.plan(nb, std::max(m[id], n[id]), std::min(m[id], n[id]), true, fa, threads);
+            spare = fa.spare;
+        }
+        const bool onchip = allow_onchip && ops.smem(nb, wv, pp.maxN) + spare <= budget;
         auto key = std::make_pair(nb, onchip ? 1 : 0);
         auto it = seg_of.find(key);
         if (it == seg_of.end()) {
