@@ -308,12 +308,15 @@ __device__ __forceinline__ bool entry_fires(const T* G, int p, int q, Real<T> to
     using R = Real<T>;
     if constexpr (Traits<T>::kComplex) {
         // without |g_pq|'s square root: well below the bound the pair does not
-        // fire; near it, or where squares leave the safe range, the full test
+        // fire, well above it it does; near it, or where squares leave the safe
+        // range, the full test
         const T g = G[p + q * LDG];
-        const R prod = rmul(re(G[p + p * LDG]), re(G[q + q * LDG])), g2 = fma_s(g.x, g.x, rmul(g.y, g.y));
-        if (as_ord(prod) > as_ord(kJacobiProdMin<R>) && as_ord(g2) > as_ord(kJacobiProdMin<R>) &&
-            rmul(g2, R(1.001)) < rmul(rmul(tol, tol), prod))
-            return false;
+        const R gpp = re(G[p + p * LDG]), prod = rmul(gpp, re(G[q + q * LDG])), g2 = fma_s(g.x, g.x, rmul(g.y, g.y));
+        if (as_ord(gpp) > 0 && as_ord(prod) > as_ord(kJacobiProdMin<R>) && as_ord(g2) > as_ord(kJacobiProdMin<R>)) {
+            const R bound = rmul(rmul(tol, tol), prod);
+            if (rmul(g2, R(1.001)) < bound) return false;
+            if (rmul(g2, R(0.999)) >= bound) return true;
+        }
     }
     return pair_fires<R>(re(G[p + p * LDG]), re(G[q + q * LDG]), abs_rot(G[p + q * LDG]), tol);
 }
@@ -486,7 +489,8 @@ __device__ int inner_jacobi(T* G, T* J, const InnerTables<T, NB>& tb, Real<T> to
     for (int e = gt; e < TWO * TWO; e += GT) {
         const int i = e % TWO, j = e / TWO;
         J[i + j * LDG] = make_s<T>(i == j ? 1 : 0);
-        if (i < j && (!cross || (i < NB && j >= NB))) any |= entry_fires<T, LDG>(G, i, j, tol, wide);
+        // (far from convergence a thread's first entry settles it)
+        if (!any && i < j && (!cross || (i < NB && j >= NB))) any = entry_fires<T, LDG>(G, i, j, tol, wide);
     }
     if (!named_sync_or(bar, GT, any)) return 0;
     // warp 0 forms the rotations, lane `slot` those of one slot, following
