@@ -100,9 +100,12 @@ typedef struct {
                           0 = 30 u, u the unit roundoff of the type (Sec. 5.4, k = 30)      */
     int inner_sweeps;  /* inner eigensolver sweeps per Gram block (Design-2, Sec. 5).  0 = one,
                           over all index pairs in a sweep's first round and the pairs between
-                          the two blocks in the others (block widths of at least 16; see
-                          cross_only in csrc/jacobi_common.cuh); >= 1: over all index pairs in
-                          every round                                                       */
+                          the two blocks in the others (block widths of at least 16, and 8
+                          where the sweeps start preconditioned; see cross_only in
+                          csrc/jacobi_common.cuh); the on-chip and persistent kernels may then
+                          start from a QR and an LQ factorisation of the matrix (preconditioned
+                          in csrc/gesvj_fused.cuh).  >= 1: over all index pairs in every round,
+                          from the matrix itself                                             */
     int path;          /* bsvd_path                                                         */
     int flags;         /* bit 0: skip the final orthogonality correction of V;
                           bit 1: two-stage vector update (Design-3 off; multi-kernel path);

@@ -411,7 +411,7 @@ __global__ void __launch_bounds__(kBlkThreads) blk_gram(const BlockedArgs a, int
     }
 }
 
-// ---- S2, FP64 and complex128, nb = 8, 16: exact digit products on the tensor cores ------------
+// ---- S2, FP64 and complex128, nb = 8, 16: digit products on the tensor cores ------------------
 // (tc_f64.cuh).  The FP64 pipe bounds blk_gram (95 % busy, 206 us a round for
 // 64 matrices of 256 x 256); here it only adds a few partial sums.
 template <class T, int NB>
@@ -536,7 +536,7 @@ __global__ void __launch_bounds__(kUpdRows) blk_update_fused(const BlockedArgs a
         return;
       }
     if constexpr (kSplit) {
-        // FP64, complex128: exact digit products on the tensor cores (tc_f64.cuh);
+        // FP64, complex128: digit products on the tensor cores (tc_f64.cuh);
         // a CTA's four warps take the 16-row tiles of its share of W, then of V.
         // On the FP64 pipe this update ran at 93 % of it: 480 us a round for
         // 64 matrices of 256 x 256.

@@ -15,7 +15,7 @@
 // After a sweep's first round only the cross pairs of i and j are swept
 // (cross_only).  Where preconditioned() says so the sweeps run on the triangular
 // factor of W instead (precondition.cuh) and Q is applied to the left vectors at
-// the end; FP64 and complex128 (nb = 8, 16) form S2, S4 and S5 as exact digit
+// the end; FP64 and complex128 (nb = 8, 16) form S2, S4 and S5 as digit
 // products on the tensor cores (tc_f64.cuh).
 // A matrix is converged after a sweep in which no rotation fired.  Then
 // sigma_k = ||w_k||_2, a stable descending sort, U = W Sigma^-1 (Alg. 2), and
@@ -103,7 +103,7 @@ __host__ __device__ inline long long fused_slot_elems(const FusedArgs& a) {
 }
 
 // FP64 and complex128 with nb = 8 or 16 form the Gram block and the update as
-// exact digit products on the tensor cores (tc_f64.cuh).
+// digit products on the tensor cores (tc_f64.cuh).
 template <class T, int NB>
 __host__ __device__ constexpr bool fused_split() { return sizeof(Real<T>) == 8 && NB >= 8; }
 
@@ -640,7 +640,8 @@ constexpr int persist_min_blocks() {
 }
 
 // On-chip launches keep the on-chip kernel's occupancy (two CTAs per SM for
-// real FP32, else one).
+// real FP32, else one; more for smaller CTAs, min_blocks_for), without the four
+// CTAs of real FP64 with nb = 8 there (fused_blocks).
 template <class T, bool OnChip>
 constexpr int persist_blocks() { return OnChip ? fused_min_blocks<T>() : persist_min_blocks<T>(); }
 

@@ -88,15 +88,6 @@ __device__ __forceinline__ float2 shfl_xor_s(float2 v, int o) {
 __device__ __forceinline__ double2 shfl_xor_s(double2 v, int o) {
     return make_double2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
 }
-template <class T> __device__ __forceinline__ T shfl_s(T v, int src);
-template <> __device__ __forceinline__ float shfl_s(float v, int src) { return __shfl_sync(0xffffffffu, v, src); }
-template <> __device__ __forceinline__ double shfl_s(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
-template <> __device__ __forceinline__ float2 shfl_s(float2 v, int src) {
-    return make_float2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
-}
-template <> __device__ __forceinline__ double2 shfl_s(double2 v, int src) {
-    return make_double2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
-}
 __device__ __forceinline__ float warp_sum_s(float v) { return warp_sum(v); }
 __device__ __forceinline__ double warp_sum_s(double v) { return warp_sum(v); }
 __device__ __forceinline__ float2 warp_sum_s(float2 v) { return make_float2(warp_sum(v.x), warp_sum(v.y)); }

@@ -317,14 +317,15 @@ cudaError_t mixed_restore_tiled(const MixedArgs& a, int batch, cudaStream_t st) 
 // 16 x 16 1.25 ms plain and 1.80 so, of 32 x 32 3.68 and 4.59, one 32 x 32 0.56
 // and 0.81; 40 x 40 10.5 (the first version) and 9.7, one 1.55 and 1.51.
 // complex128 stays plain: in one CTA on the FP64 pipe the step made one 96 x 96
-// 17.1 ms instead of 11.5.  Every product is an exact digit product
+// 17.1 ms instead of 11.5.  Every product is a digit product
 // (tc_f64.cuh) over (matrix, 64 rows, 32 columns) grids, 32 terms of the
 // contraction at a time; the chunks' sums are added in FP64 in increasing
 // order.  Per chunk a CTA stages both operands in shared memory, splits the
 // right one into digits once, and each of its four warps splits and multiplies
 // 16 rows.  A matrix whose rows span more than 2^6 takes multiply-adds on the same
-// tiles (kDigitRowSpan: V's small entries count there).  2,000 of 96x96: the restoration 42 ms as one CTA a matrix on the
-// FP64 pipe, 28.2 so: 9.1 in these products, 19.1 in mx_precondition.
+// tiles (kDigitRowSpan: V's small entries count there).  2,000 of 96x96: the
+// restoration 42 ms as one CTA a matrix on the FP64 pipe, 28.2 so: 9.1 in these
+// products, 19.1 in mx_precondition.
 enum MxOp {
     kMxGram,      // E = V^T V - I
     kMxGramL,     // E = L^T L, L the lower triangle in A_hat

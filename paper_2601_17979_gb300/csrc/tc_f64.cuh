@@ -1,4 +1,4 @@
-// tc_f64.cuh -- FP64 products on the tensor cores, exact in fixed point.
+// tc_f64.cuh -- FP64 products on the tensor cores, in fixed point.
 //
 // A GB300 SM retires about 1.6 FP64 multiply-adds a clock and 0.47 FP16
 // 16 x 8 x 16 tile products (2,048 multiply-adds each), so the Gram block and
@@ -10,12 +10,15 @@
 // E the largest exponent of the row (or column) the product sums over; an
 // entry keeps 53 bits below that exponent, rounded to nearest.  A product of
 // two digits is below 2^16 and a sum of 32 times the up to six digit products
-// of equal weight i + j below 2^24: exact in the FP32 accumulator.  Weights
-// up to 6 are kept (26 digit products); what is dropped is below 2^-58 of the
-// row's and column's largest product, the digits' own rounding 2^-53 -- the
-// error of one FP64 rounding at that size, where 32 chained multiply-adds
-// round 32 times.  Accumulators are converted and combined as integers and
-// rounded once to FP64; no FP64 instruction is used at all.
+// of equal weight i + j below 2^24: the digit products and their sums are exact
+// in the FP32 accumulator.  The result is not: weights up to 6 are kept (26 of
+// the 36 digit products), and the operands are rounded.  In units of the row's
+// largest entry times the column's, what is dropped is below 2^-59 a term and
+// 2^-54 over 32, the operands' rounding (2^-53 on either side) below 2^-52 a
+// term and 2^-47 over 32; 32 chained multiply-adds, each rounding a partial
+// sum, may lose 2^-44 on the same entries.  Accumulators are converted and
+// combined as integers and rounded once to FP64; no FP64 instruction is used
+// at all.
 //
 // Fragments (PTX ISA, mma.sync.m16n8k16 .f16), g = lane / 4, t = lane % 4:
 //   A (16 x 16)  a0 (g, 2t..2t+1)  a1 (g+8, 2t..)  a2 (g, 2t+8..)  a3 (g+8, 2t+8..)
