@@ -9,7 +9,8 @@ Reported on one JSON line:
   value       device-resident throughput (inputs in HBM before timing)
   e2e         the same through the public API with host buffers: pinned
               H2D of A and D2H of Sigma, U, V, info inside the timed region
-  roofline    the dominant kernel (FP64 fused SVD) against the FP64 pipe
+  roofline    a direct decomposition's operations over the dominant kernel's
+              time (FP64 fused SVD), beside the FP64 pipe's peak
   cpu_baseline the CPU oracle (OpenMP over matrices) on a bounded sample
   plain_fp64  the paper's baseline path (inner solver to convergence, no
               masks) on the FP64 batch, for "vs plain FP64 Jacobi"
@@ -83,21 +84,20 @@ def measured_traffic(kind: str, workload: str, matrices: int):
     return None if per is None else per * matrices
 
 
-def pair_flops(m, n, nb, cplx=False):
-    """Algorithmic flops of one block pair: Gram 4 m nb^2, A update 8 m nb^2,
-    V update 8 n nb^2, one inner sweep 72 nb^3 (x4 for complex)."""
-    f = 12 * m * nb * nb + 8 * n * nb * nb + 72 * nb ** 3
-    return 4 * f if cplx else f
+def direct_flops(m, n, vectors=True):
+    """Real operations of a direct decomposition (R-bidiagonalisation) of one
+    real m x n matrix, m >= n: 6 m n^2 + 11 n^3 with the vectors, 2 m n^2 + 2 n^3
+    without.  A rate in these does not depend on the method, on its sweeps or on
+    the unit that does the work; the solver itself does several times as many."""
+    return 6.0 * m * n * n + 11.0 * n ** 3 if vectors else 2.0 * m * n * n + 2.0 * n ** 3
 
 
-def matrix_flops(m, n, nb, sweeps):
-    """Executed sweeps: all but the last do full pair steps; the last (the
-    sweep that found every block diagonal) forms the Gram blocks only."""
-    l = max(2, -(-n // nb))
-    pairs = l * (l - 1) // 2
-    sweeps = np.asarray(sweeps, dtype=np.float64)
-    return (np.maximum(sweeps - 1, 0) * pairs * pair_flops(m, n, nb)
-            + pairs * 4 * m * nb * nb + 3 * m * n).sum()
+def roofline(tflops, peak, traffic=None, **more):
+    """A rate of direct_flops beside the pipe's peak.  Not a utilisation: the
+    sweeps wait for dependent rotations and barriers, and the FP64 Gram blocks and
+    updates run on the tensor cores."""
+    return {"bound": "latency", "achieved": tflops, "peak": peak / 1e12, "unit": "TFLOP/s",
+            "frac": tflops * 1e12 / peak, "counts": "operations of a direct decomposition", "traffic": traffic, **more}
 
 
 def oracle_flops(m, n, sweeps):
@@ -412,12 +412,11 @@ def run_uneven(args, rank, world, local):
     value = B * world / (ms * 1e-3)
     flops = 0.0
     buckets = {}
-    for dt, r in res.items():
-        sw = r.sweeps.cpu().numpy()
+    for dt in res:
         nbs, where, _ = plans[dt]
-        for x, k, nb_, w in zip(groups[dt], sw, nbs, where):
+        for x, nb_, w in zip(groups[dt], nbs, where):
             m, n = x.shape
-            f = matrix_flops(max(m, n), min(m, n), int(nb_), [k])      # at the executed block width
+            f = direct_flops(max(m, n), min(m, n))
             flops += 4 * f if np.iscomplexobj(x) else f
             key = f"{np.dtype(dt).name} nb={int(nb_)} {['global slot', 'shared memory', 'multi-kernel'][int(w)]}"
             seg = buckets.setdefault(key, {"matrices": 0, "k_min": 10 ** 9, "k_max": 0})
@@ -445,11 +444,9 @@ def run_uneven(args, rank, world, local):
                           "columns": "M, N (rounded up to powers of two), chosen nb, ms at nb 4, 8, 16"}
                          if tuning else None),
             "gflops": flops / (ms * 1e-3) / 1e9,
-            "roofline": {"bound": "alu", "achieved": flops / (ms * 1e-3) / 1e12, "peak": PEAK_FP32 / 1e12,
-                         "unit": "TFLOP/s", "frac": flops / (ms * 1e-3) / PEAK_FP32,
-                         "traffic": measured_traffic("uneven", "uneven", B),
-                         "traffic_note": "every kernel of the step, DRAM read + write (ncu on a 2,000-matrix "
-                                         "case, scaled by matrix count)"},
+            "roofline": roofline(flops / (ms * 1e-3) / 1e12, PEAK_FP32, measured_traffic("uneven", "uneven", B),
+                                 traffic_note="every kernel of the step, DRAM read + write (ncu on a "
+                                              "2,000-matrix case, scaled by matrix count)"),
             "clocks": sampler.summary()}
     # the same matrices with one launch per distinct shape (the pointer-array
     # form grouping by shape) -- the path the persistent launch replaces
@@ -544,10 +541,9 @@ def summarize_stream(tr, ids, t0, t_arrivals, t_stop, rec, idx, before, at_end, 
     m = sizes[tr["bin"][idx[ok]]]
     n = np.where(tr["tall"][idx[ok]], -(-m // 2), m)
     cplx = tr["dtype"][idx[ok]] == "c"
-    sw = rec["sweeps"][ok]
     flops = 0.0
-    for mm, nn, c, k in zip(m.tolist(), n.tolist(), cplx.tolist(), sw.tolist()):
-        f = matrix_flops(mm, nn, 16 if nn >= 48 else (8 if nn >= 12 else 4), [k])
+    for mm, nn, c in zip(m.tolist(), n.tolist(), cplx.tolist()):
+        f = direct_flops(mm, nn)
         flops += 4 * f if c else f
     span = max(float(rec["t_done"][ok].max()) - t0, 1e-9) if n_done else 1e-9
     in_window = int((rec["t_done"][ok] <= t_arrivals).sum())
@@ -719,7 +715,7 @@ def run_tallskinny(args, rank, world, local):
                 row[name + "_info_nonzero"] = int((res.info != 0).sum().item())
                 sw = res.sweeps.cpu().numpy()
                 row[name + "_sweeps_mean"] = float(sw.mean())
-                f = tallskinny_flops(m, 16, sw, name == "qr") * (4 if t in "cz" else 1)
+                f = B * direct_flops(m, 16) * (4 if t in "cz" else 1)
                 row[name + "_tflops"] = f / (ms * 1e-3) / 1e12
             row["qr_speedup"] = row["noqr_ms"] / row["qr_ms"]
             rows.append(row)
@@ -734,12 +730,9 @@ def run_tallskinny(args, rank, world, local):
                                    "U[0,1] (real and imaginary parts); U, Sigma, V; median of steps",
                        "l2": "L2 flushed (256 MB write) before every timed call"},
             "gpu_launches": 2 * max(1, args.steps),
-            # QR factor, Q applied to [U_R; 0] and the SVD of R, algorithmic
-            # FP64 flops of the executed sweeps, against the FP64 pipe
-            "roofline": {"bound": "alu", "achieved": head["qr_tflops"], "peak": PEAK_FP64 / 1e12,
-                         "unit": "TFLOP/s", "frac": head["qr_tflops"] * 1e12 / PEAK_FP64, "traffic": None,
-                         "kernel": "qr_factor + SVD of R + qr_apply (FP64, m = 2000, n = 16)",
-                         "peak_source": "derived: 152 SMs x 2 FP64 FMA/clk x 2 flop x 2.07 GHz"},
+            "roofline": roofline(head["qr_tflops"], PEAK_FP64,
+                                 kernel="qr_factor + SVD of R + qr_apply (FP64, m = 2000, n = 16)",
+                                 peak_source="derived: 152 SMs x 2 FP64 FMA/clk x 2 flop x 2.07 GHz"),
             "clocks": sampler.summary(), "results": rows}
     if rank == 0 and world == 1 and not args.no_cpu:
         import oracle
@@ -757,17 +750,6 @@ def run_tallskinny(args, rank, world, local):
                                           f"passes, Alg. 2 in FP64 (no QR), OpenMP over matrices ({dt_:.1f} s)"}
     if rank == 0:
         print(json.dumps(line), flush=True)
-
-
-def tallskinny_flops(m, n, sweeps, qr):
-    """Algorithmic real flops of the tall-skinny solve: with QR, Householder
-    QR 2 m n^2 - 2 n^3 / 3, Q applied to [U_R; 0] 4 m n^2 - 2 n^3 and the
-    SVD of the n x n factor R; without, the SVD of the m x n matrix."""
-    nb = 16 if n >= 48 else (8 if n >= 12 else 4)
-    if not qr:
-        return matrix_flops(m, n, nb, sweeps)
-    k = len(np.atleast_1d(sweeps))
-    return k * (2 * m * n * n - 2 * n ** 3 / 3 + 4 * m * n * n - 2 * n ** 3) + matrix_flops(n, n, nb, sweeps)
 
 
 # Timed calls per leg of the 32x32 workload (about 6 ms each): enough for
@@ -823,7 +805,7 @@ def run_square32(args, rank, world, local):
         acc = accuracy_over_bounds([Ah[i] for i in samp], [o[0][i].cpu().numpy() for i in samp],
                                    [o[1][i].cpu().numpy() for i in samp], [o[2][i].cpu().numpy() for i in samp],
                                    ref, U64)
-        fl = matrix_flops(m, n, nb, sw)
+        fl = B * direct_flops(m, n)
         return {"matrices_per_s": B * world / (ms * 1e-3), "ms": ms, "ms_all": ts, "sweeps_mean": float(sw.mean()),
                 "sweeps_max": int(sw.max()), "info_nonzero": int((o[3].cpu().numpy() != 0).sum()),
                 "tflops": fl / (ms * 1e-3) / 1e12, "accuracy_worst_over_bound": acc,
@@ -842,11 +824,9 @@ def run_square32(args, rank, world, local):
                        "path": "on-chip batched solver (one CTA per matrix)",
                        "l2": "L2 flushed (256 MB write) before every timed call"},
             "gpu_launches": max(SQ32_STEPS, args.steps), "batched": fused,
-            "roofline": {"bound": "alu", "achieved": fused["tflops"], "peak": PEAK_FP64 / 1e12,
-                         "unit": "TFLOP/s", "frac": fused["tflops"] * 1e12 / PEAK_FP64,
-                         "traffic": measured_traffic("fused", "square32_f64", B),
-                         "kernel": "gesvj_fused_kernel<double,8,2,64>",
-                         "peak_source": "derived: 152 SMs x 2 FP64 FMA/clk x 2 flop x 2.07 GHz"},
+            "roofline": roofline(fused["tflops"], PEAK_FP64, measured_traffic("fused", "square32_f64", B),
+                                 kernel="gesvj_fused_kernel<double,8,2,64>",
+                                 peak_source="derived: 152 SMs x 2 FP64 FMA/clk x 2 flop x 2.07 GHz"),
             "clocks": fused["clocks"]}
     if plain is not None:
         line["plain_fp64"] = plain
@@ -943,13 +923,12 @@ def run_mixed96(args, rank, world, local):
             for key, val in w.items():
                 worst[key] = max(worst.get(key, 0.0), val)
         sw = {t: res[t].sweeps.cpu().numpy() for t in res}
-        # algorithmic FP64 flops of the executed (polish or native) sweeps
-        fl64 = matrix_flops(96, 96, 16, sw["d"]) + 4 * matrix_flops(96, 96, 16, sw["z"])
+        fl = (sw["d"].size + 4 * sw["z"].size) * direct_flops(96, 96)
         out[name] = {"matrices_per_s": len(ids) * world / (total * 1e-3), "ms": total,
                      "ms_real": times["d"], "ms_complex": times["z"],
                      "sweeps_mean": {t: float(sw[t].mean()) for t in sw},
                      "info_nonzero": int(sum(int((res[t].info != 0).sum().item()) for t in res)),
-                     "fp64_sweep_tflops": fl64 / (total * 1e-3) / 1e12,
+                     "tflops": fl / (total * 1e-3) / 1e12,
                      "sigma_err_vs_oracle_over_bound": worst.get("sigma_err"),
                      "accuracy_worst_over_bound": worst, "clocks": sampler.summary()}
         if kw.get("flags"):
@@ -967,12 +946,9 @@ def run_mixed96(args, rank, world, local):
             "variants": {k: v for k, v in out.items() if k not in ("mixed", "native")},
             "speedup_over_native": nat["ms"] / out["mixed"]["ms"],
             "sigma_err_vs_oracle": {k: v["sigma_err_vs_oracle_over_bound"] for k, v in out.items()},
-            # the native FP64 solve against the FP64 pipe (its executed sweeps'
-            # algorithmic flops); the mixed solve's FP64 part is the polish
-            "roofline": {"bound": "alu", "achieved": nat["fp64_sweep_tflops"], "peak": PEAK_FP64 / 1e12,
-                         "unit": "TFLOP/s", "frac": nat["fp64_sweep_tflops"] * 1e12 / PEAK_FP64,
-                         "traffic": None, "kernel": "native FP64 solve (on chip real, multi-kernel complex)",
-                         "peak_source": "derived: 152 SMs x 2 FP64 FMA/clk x 2 flop x 2.07 GHz"},
+            "roofline": roofline(nat["tflops"], PEAK_FP64,
+                                 kernel="native FP64 solve (on chip real, multi-kernel complex)",
+                                 peak_source="derived: 152 SMs x 2 FP64 FMA/clk x 2 flop x 2.07 GHz"),
             "gpu_launches": None, "clocks": out["mixed"]["clocks"]}
     if rank == 0 and world == 1 and not args.no_cpu:
         import oracle
@@ -1025,8 +1001,7 @@ def run_square(args, rank, world, local):
             res = holder["r"]
             ms = statistics.median(times)
             sw = res.sweeps.cpu().numpy()
-            nb = 16 if n >= 48 else (8 if n >= 12 else 4)
-            f = matrix_flops(n, n, nb, sw) * (4 if t in "zc" else 1)     # a complex MAC: four real ones
+            f = B * direct_flops(n, n) * (4 if t in "zc" else 1)         # a complex MAC: four real ones
             rows.append({"dtype": t, "n": n, "batch": B, "ms": ms, "matrices_per_s": B / (ms * 1e-3),
                          "tflops": f / (ms * 1e-3) / 1e12, "sweeps_mean": float(sw.mean()),
                          "info_nonzero": int((res.info != 0).sum().item())})
@@ -1046,11 +1021,10 @@ def run_square(args, rank, world, local):
                                    "(FP64 / complex128 n = 512: 200) unless --batch; median of steps",
                        "flags": args.square_flags,
                        "l2": "L2 flushed (256 MB write) before every timed call"},
-            "roofline": {"bound": "alu", "achieved": head["tflops"], "peak": peak_head / 1e12,
-                         "unit": "TFLOP/s", "frac": head["tflops"] * 1e12 / peak_head, "traffic": None,
-                         "kernel": f"{head['dtype'].upper()} solve at n = {head['n']} (multi-kernel path above "
-                                   "~100 columns)",
-                         "peak_source": "derived: 152 SMs x 2 FP64 FMA/clk x 2 flop x 2.07 GHz"},
+            "roofline": roofline(head["tflops"], peak_head,
+                                 kernel=f"{head['dtype'].upper()} solve at n = {head['n']} (multi-kernel path "
+                                        "above ~100 columns)",
+                                 peak_source="derived: 152 SMs x 2 FP64 (128 FP32) FMA/clk x 2 flop x 2.07 GHz"),
             "roofline_fp32": [{"dtype": r["dtype"], "n": r["n"], "achieved": r["tflops"], "peak": PEAK_FP32 / 1e12,
                                "frac": r["tflops"] * 1e12 / PEAK_FP32} for r in rows if r["dtype"] in "sc"],
             "clocks": sampler.summary(), "results": rows}
@@ -1218,8 +1192,7 @@ def main():
     # results of the last step: convergence and a bounds check on a sample
     info64, sw64 = o64[3].cpu().numpy(), o64[4].cpu().numpy()
     info32, sw32 = o32[3].cpu().numpy(), o32[4].cpu().numpy()
-    flops64 = matrix_flops(M, N, NB, sw64)
-    flops32 = matrix_flops(M, N, NB, sw32)
+    flops = B * direct_flops(M, N)
     t64 = float(np.mean(k64)) * 1e-3
     t32 = float(np.mean(k32)) * 1e-3
     # sampled results against the FP64 oracle (sigma) and the residual and
@@ -1240,19 +1213,16 @@ def main():
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f64+f32",
         "data": "synthetic", "config": config_dict(world, 2 * B),
         "gpu_launches": 2 * args.steps,
-        "fp64": {"matrices_per_s": B / t64, "kernel_ms": t64 * 1e3, "gflops": flops64 / t64 / 1e9,
+        "fp64": {"matrices_per_s": B / t64, "kernel_ms": t64 * 1e3, "gflops": flops / t64 / 1e9,
                  "sweeps_mean": float(sw64.mean()), "sweeps_max": int(sw64.max()),
                  "info_nonzero": int((info64 != 0).sum())},
-        "fp32": {"matrices_per_s": B / t32, "kernel_ms": t32 * 1e3, "gflops": flops32 / t32 / 1e9,
+        "fp32": {"matrices_per_s": B / t32, "kernel_ms": t32 * 1e3, "gflops": flops / t32 / 1e9,
                  "sweeps_mean": float(sw32.mean()), "sweeps_max": int(sw32.max()),
                  "info_nonzero": int((info32 != 0).sum()),
-                 "roofline": {"bound": "alu", "achieved": flops32 / t32 / 1e12, "peak": PEAK_FP32 / 1e12,
-                              "unit": "TFLOP/s", "frac": flops32 / t32 / PEAK_FP32,
-                              "traffic": measured_traffic("fused", "tall128x64_f32", B)}},
-        "roofline": {"bound": "alu", "achieved": flops64 / t64 / 1e12, "peak": PEAK_FP64 / 1e12,
-                     "unit": "TFLOP/s", "frac": flops64 / t64 / PEAK_FP64, "traffic": measured_traffic("fused", "tall128x64_f64", B),
-                     "kernel": "gesvj_fused_kernel<double,16,2,128>",
-                     "peak_source": "derived: 152 SMs x 2 FP64 FMA/clk x 2 flop x 2.07 GHz"},
+                 "roofline": roofline(flops / t32 / 1e12, PEAK_FP32, measured_traffic("fused", "tall128x64_f32", B))},
+        "roofline": roofline(flops / t64 / 1e12, PEAK_FP64, measured_traffic("fused", "tall128x64_f64", B),
+                             kernel="gesvj_fused_kernel<double,16,2,128>",
+                             peak_source="derived: 152 SMs x 2 FP64 FMA/clk x 2 flop x 2.07 GHz"),
         "accuracy_worst_over_bound": worst,
         "clocks": sampler.summary(),
     }
