@@ -319,10 +319,11 @@ __device__ __forceinline__ bool entry_fires(const T* G, int p, int q, Real<T> to
 // in round 1), so the other rounds sweep the nb^2 cross pairs in nb steps
 // instead of all (2nb - 1) nb pairs in 2nb - 1 steps.  A caller that sets
 // inner_sweeps gets full sweeps everywhere.  Single precision keeps full
-// sweeps above 20 blocks: there the many FP32 updates' own roundings set the
-// singular values' last digits, and the shorter sweeps (which leave S closer
-// to the exact values: 4.9e-5 against 6.9e-5 relative on 512 x 512) would
-// move them by more than FP32 results may move between versions (2e-5).
+// sweeps above 20 blocks, a line drawn between 16 and 32 blocks, the two sizes
+// that were measured: not for speed or accuracy (the shorter sweeps leave S
+// closer to the exact values, 4.9e-5 against 6.9e-5 relative on 512 x 512) but to
+// leave the results of such matrices, where the many FP32 updates' own roundings
+// set the singular values' last digits, as they were.
 // Complex128 keeps them up to 3 blocks (2,000 of 20 x 20, nb = 8: 11.8 ms against
 // 12.5; at 4 blocks 500 of 64 x 64 29.2 ms full, 26.7 with cross pairs).
 // Sweeps on 256 x 256 FP32: 11.3 full, 11.6 with cross pairs, half the steps.
@@ -633,8 +634,9 @@ __device__ int inner_jacobi(T* G, T* J, const InnerTables<T, NB>& tb, Real<T> to
 }
 
 // Binary orders between the rows' largest and smallest largest entry, zero rows
-// apart; entry (r, j) at W[r * sr + j * sj].  red: 2 NT / 32 ints, free on entry.  Called by all NT threads after W is
-// complete and synchronised; returns synchronised.
+// apart; entry (r, j) at W[r * sr + j * sj].  red: 2 NT / 32 ints, free on entry.
+// Called by all NT threads after W is complete and synchronised; returns
+// synchronised.
 template <class T, int NT>
 __device__ __forceinline__ int row_span(const T* W, long long sr, long long sj, int M, int N, int* red) {
     constexpr int NW = NT / 32;

@@ -24,7 +24,8 @@
 // explicit: the same bits wherever it is inlined.
 //
 // What bounds it: N dependent steps per factorisation, in FP64 the FP64 pipe
-// (66 % busy), in FP32 latency and shared-memory bandwidth.  128 x 64, one CTA:
+// (64 % busy over the whole 128 x 64 solve), in FP32 latency and shared-memory
+// bandwidth.  128 x 64, one CTA:
 // FP64 1.48 M cycles and 0.74 M for Q's application (17 sweeps take 23 M, the
 // 6.3 left 5 M); FP32 0.21 M and 0.075 M on the float4 form below (0.45 M and
 // 0.20 M on the scalar one), 11 sweeps about 1.5 M.  Measured and not kept:
