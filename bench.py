@@ -63,11 +63,11 @@ KERNEL_SOURCES = {
 }
 TRAFFIC_PER_MATRIX = {
     # 128x64, gesvj_fused_kernel<double|float,16,2,128>: 2,000-matrix launches
-    ("fused", "tall128x64_f64", "3288b67c8abc"): (136445440 + 145813760) / 2000,
-    ("fused", "tall128x64_f32", "3288b67c8abc"): (73290240 + 43410432) / 2000,
+    ("fused", "tall128x64_f64", "f1cd255c8480"): (136263936 + 145203456) / 2000,
+    ("fused", "tall128x64_f32", "f1cd255c8480"): (73431808 + 44118784) / 2000,
     # the whole uneven step (every kernel of both types), 2,000-matrix case:
-    # 497.6 GB over the warm-up and the timed step
-    ("uneven", "uneven", "490147fdfd01"): 497.60e9 / 2 / 2000,
+    # 503.8 GB over the warm-up and the timed step
+    ("uneven", "uneven", "9d790a783735"): 503.78e9 / 2 / 2000,
 }
 
 
