@@ -324,8 +324,8 @@ cudaError_t mixed_restore_tiled(const MixedArgs& a, int batch, cudaStream_t st) 
 // right one into digits once, and each of its four warps splits and multiplies
 // 16 rows.  A matrix whose rows span more than 2^6 takes multiply-adds on the same
 // tiles (kDigitRowSpan: V's small entries count there).  2,000 of 96x96: the
-// restoration 42 ms as one CTA a matrix on the FP64 pipe, 28.2 so: 9.1 in these
-// products, 19.1 in mx_precondition.
+// restoration 42 ms as one CTA a matrix on the FP64 pipe, 29.7 so: 9.9 in these
+// products, 0.6 in mx_omega, 19.1 in mx_precondition.
 enum MxOp {
     kMxGram,      // E = V^T V - I
     kMxGramL,     // E = L^T L, L the lower triangle in A_hat
